@@ -12,7 +12,6 @@ namespace pplbm {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kMaxTileSmem = (256 + 2) * (1 + 2);  // largest (tw + 2)(th + 2) over tw*th = 256
 constexpr unsigned kSpinLimit = 1u << 24;           // x ~100 ns sleeps: ~1.7 s per barrier wait
 constexpr int kErrTimeout = 2;  // batch error word; divergence is flagged per instance
 
@@ -72,8 +71,8 @@ template <int KIND, bool REUSE>
 __device__ __forceinline__ void batch_rho_psi_local(const BatchInst* __restrict__ inst, int id, int local,
                                                     int parity, StepArgs* sa) {
   stage_args(inst, id, parity, sa);
-  const int64_t i = (int64_t)local * kThreads + threadIdx.x;
-  if (i < sa->n) rho_psi_node<KIND>(*sa, sa->f_in, i);
+  const int i = local * kThreads + threadIdx.x;
+  if (i < (int)sa->n) rho_psi_node<KIND>(*sa, sa->f_in, i);
   if (REUSE) __syncthreads();
 }
 
@@ -87,33 +86,20 @@ __device__ __forceinline__ void batch_rho_psi_item(const BatchInst* __restrict__
 // collision pass over tile t of instance id; org: two shared ints for the tile
 // origin, which one thread computes per item; REUSE as for the density pass
 template <int KIND, bool ST, bool REUSE>
-__device__ __forceinline__ void batch_collide_local(const BatchInst* __restrict__ inst, int id, int t, int parity,
-                                                    double* sp, StepArgs* sa, int* org) {
+__device__ __forceinline__ void batch_collide_item(const BatchInst* __restrict__ inst, const int* __restrict__ owner,
+                                                   int w, int parity, StepArgs* sa, int* org) {
+  const int id = owner[w];
   const BatchInst& I = inst[id];
   if (threadIdx.x == 0) {
-    const int tyi = t / I.tiles_x;
+    const int t = w - I.k2_start, tyi = t / I.tiles_x;
     org[0] = (t - tyi * I.tiles_x) * I.tw;
     org[1] = tyi * I.th;
   }
   stage_args(inst, id, parity, sa);  // ends with a barrier: org is visible
   const StepArgs& a = *sa;
-  const int tw = I.tw, th = I.th, log2tw = I.log2tw;
-  const int x0 = org[0], y0 = org[1];
-  const int lx = threadIdx.x & (tw - 1), ly = threadIdx.x >> log2tw;
-  load_psi_tile(a, sp, x0, y0, tw, th, lx, ly, threadIdx.x, kThreads);
-  __syncthreads();
-  const int x = x0 + lx, y = y0 + ly;
-  if (x < a.nx && y < a.ny)
-    collide_node<KIND, false, ST>(a, x, y, sp, (ly + 1) * (tw + 2) + lx + 1, tw + 2, nullptr, nullptr, nullptr,
-                                  nullptr);
+  const int x = org[0] + ((int)threadIdx.x & (I.tw - 1)), y = org[1] + ((int)threadIdx.x >> I.log2tw);
+  if (x < a.nx && y < a.ny) collide_node<KIND, false, ST>(a, x, y, nullptr, nullptr, nullptr, nullptr);
   if (REUSE) __syncthreads();
-}
-
-template <int KIND, bool ST, bool REUSE>
-__device__ __forceinline__ void batch_collide_item(const BatchInst* __restrict__ inst, const int* __restrict__ owner,
-                                                   int w, int parity, double* sp, StepArgs* sa, int* org) {
-  const int id = owner[w];
-  batch_collide_local<KIND, ST, REUSE>(inst, id, w - inst[id].k2_start, parity, sp, sa, org);
 }
 
 template <int KIND>
@@ -132,10 +118,9 @@ constexpr int collide_min_blocks(int kind) { return kind == kUnitTau ? 5 : 4; }
 template <int KIND, bool ST>
 __global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
     k_batch_collide(const BatchInst* inst, const int* owner, int parity) {
-  __shared__ double sp[kMaxTileSmem];
   __shared__ StepArgs sa;
   __shared__ int org[2];
-  batch_collide_item<KIND, ST, false>(inst, owner, blockIdx.x, parity, sp, &sa, org);
+  batch_collide_item<KIND, ST, false>(inst, owner, blockIdx.x, parity, &sa, org);
 }
 
 // ---- the pipelined plan's mixed kernel ----------------------------------------------
@@ -172,53 +157,18 @@ __device__ __forceinline__ void fetch_item_args(const BatchInst* __restrict__ in
   for (int k = threadIdx.x; k < (int)(sizeof(StepArgs) / 8); k += kThreads) cp_async8(d + k, src + k);
 }
 
-// Starts the load of a collision tile's psi halo tile into sp (row stride tw + 2), as
-// load_psi_tile does: psi values by asynchronous copies, the wall ghost values by
-// plain stores.
-__device__ __forceinline__ void fetch_item_tile(const StepArgs& a, const int4& h, double* sp) {
-  const int log2tw = h.y, tw = 1 << log2tw, th = kThreads >> log2tw, sw = tw + 2;
-  const int x0 = h.z, y0 = h.w;
-  const int nh = 2 * sw + 2 * th;
-  for (int k = (int)threadIdx.x - kThreads; k < nh; k += kThreads) {
-    int tx, ty;
-    if (k < 0) {  // the thread's own node
-      tx = 1 + ((int)threadIdx.x & (tw - 1));
-      ty = 1 + ((int)threadIdx.x >> log2tw);
-    } else if (k < 2 * sw) {
-      const bool top = k >= sw;
-      ty = top ? th + 1 : 0;
-      tx = top ? k - sw : k;
-    } else {
-      const int j = k - 2 * sw;
-      ty = 1 + (j >> 1);
-      tx = (j & 1) ? tw + 1 : 0;
-    }
-    const int gx = wrap_near(x0 + tx - 1, a.nx);
-    int gy = y0 + ty - 1;
-    double* d = sp + ty * sw + tx;
-    if (a.walls && (gy < 0 || gy >= a.ny)) {
-      *d = gy < 0 ? a.psi_ghost_bottom : a.psi_ghost_top;
-    } else {
-      if (!a.walls) gy = wrap_near(gy, a.ny);
-      cp_async8(d, a.psi + (int64_t)gy * a.nx + gx);
-    }
-  }
-}
-
-// The item's pass from its staged arguments (and tile)
+// The item's pass from its staged arguments
 template <int KIND, bool ST>
-__device__ __forceinline__ void run_item(const StepArgs& a, const int4& h, const double* sp) {
+__device__ __forceinline__ void run_item(const StepArgs& a, const int4& h) {
   if (!is_collision_item(h)) {
-    const int64_t i = (int64_t)h.y * kThreads + threadIdx.x;
-    if (i < a.n) rho_psi_node<KIND>(a, a.f_in, i);
+    const int i = h.y * kThreads + threadIdx.x;
+    if (i < (int)a.n) rho_psi_node<KIND>(a, a.f_in, i);
     return;
   }
   const int log2tw = h.y, tw = 1 << log2tw;
   const int lx = (int)threadIdx.x & (tw - 1), ly = (int)threadIdx.x >> log2tw;
   const int x = h.z + lx, y = h.w + ly;
-  if (x < a.nx && y < a.ny)
-    collide_node<KIND, false, ST>(a, x, y, sp, (ly + 1) * (tw + 2) + lx + 1, tw + 2, nullptr,
-                                  nullptr, nullptr, nullptr);
+  if (x < a.nx && y < a.ny) collide_node<KIND, false, ST>(a, x, y, nullptr, nullptr, nullptr, nullptr);
 }
 
 // Work items of both passes in one launch (the pipelined plan): density items read
@@ -235,7 +185,6 @@ __device__ __forceinline__ void run_item(const StepArgs& a, const int4& h, const
 template <int KIND, bool ST>
 __global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
     k_batch_mixed(const BatchInst* inst, const int4* items, int n, int p1, int p2, unsigned* queue) {
-  __shared__ double sp[2][kMaxTileSmem];
   __shared__ StepArgs sa[4];
   __shared__ int4 hdr[4];
   __shared__ int qi[4];  // table index of the ring slot's item; -1: none
@@ -255,15 +204,11 @@ __global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
   if (qi[1] >= 0) fetch_item_args(inst, hdr[1], p1, p2, &sa[1]);
   cp_async_wait_all();
   __syncthreads();
-  if (is_collision_item(hdr[0])) fetch_item_tile(sa[0], hdr[0], sp[0]);
-  cp_async_wait_all();
-  __syncthreads();
   // qi[c] is rewritten during iteration k (thread 0, for item k + 4), so whether item
   // k + 1 exists is read from its slot c1 before the iteration's barrier: slot c1 is
   // not written during iteration k, and every thread reads the same value
   for (int k = 0;; ++k) {
     const int c = k & 3, c1 = (k + 1) & 3, c2 = (k + 2) & 3, c3 = (k + 3) & 3;
-    if (qi[c1] >= 0 && is_collision_item(hdr[c1])) fetch_item_tile(sa[c1], hdr[c1], sp[(k + 1) & 1]);
     if (qi[c2] >= 0) fetch_item_args(inst, hdr[c2], p1, p2, &sa[c2]);
     int next = -1;
     if (threadIdx.x == 0) {
@@ -271,7 +216,7 @@ __global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
       const int t = G + (int)atomicAdd(&queue[0], 1u);
       next = t < n ? t : -1;
     }
-    run_item<KIND, ST>(sa[c], hdr[c], sp[k & 1]);
+    run_item<KIND, ST>(sa[c], hdr[c]);
     if (threadIdx.x == 0) qi[c] = next;  // slot c now names item k + 4
     const bool more = qi[c1] >= 0;
     cp_async_wait_all();
@@ -304,7 +249,6 @@ __global__ void __launch_bounds__(kThreads) k_batch_persistent(const BatchInst* 
                                                                const int* owner2, int n2, int parity0, long long nsteps,
                                                                GridBarrier* bar, int* err, unsigned spin_limit,
                                                                int absent_block) {
-  __shared__ double sp[kMaxTileSmem];
   __shared__ StepArgs sa;
   __shared__ int org[2];
   // barrier self-test only: one block leaves without arriving, so the others' waits run out
@@ -314,7 +258,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_persistent(const BatchInst* 
     for (int w = blockIdx.x; w < n1; w += gridDim.x) batch_rho_psi_item<KIND, true>(inst, owner1, w, parity, &sa);
     if (!grid_barrier(bar, err, spin_limit)) return;
     for (int w = blockIdx.x; w < n2; w += gridDim.x)
-      batch_collide_item<KIND, ST, true>(inst, owner2, w, parity, sp, &sa, org);
+      batch_collide_item<KIND, ST, true>(inst, owner2, w, parity, &sa, org);
     if (!grid_barrier(bar, err, spin_limit)) return;
   }
 }

@@ -24,6 +24,34 @@ int collision_kind(const pplbm_relax* r) {
   return kFullMrt;
 }
 
+// x / div as a fixed-point factor m 2^e, 2^62 <= |m| < 2^63, rounded to nearest; m = 0
+// for 0, with an exponent that shifts every product out
+static fx::FixNum fixnum(double x, int div) {
+  fx::FixNum r{0, -4096, 0};
+  if (x == 0.0 || !std::isfinite(x)) return r;
+  int e;
+  const int64_t s = (int64_t)std::ldexp(std::frexp(std::fabs(x), &e), 53);  // |x| = s 2^(e - 53)
+  unsigned __int128 q = ((unsigned __int128)s << 72) / (unsigned)div;       // |x| / div = q 2^(e - 125)
+  e -= 125;
+  while (q >> 63) {
+    q = (q >> 1) + (q & 1 && !(q >> 64));
+    ++e;
+  }
+  r.m = x < 0.0 ? -(int64_t)q : (int64_t)q;
+  r.e = e;
+  return r;
+}
+
+// round(x 2^k) when it is below 2^bits in magnitude; *ok is cleared otherwise
+static int64_t fixed(long double x, int k, int bits, int* ok) {
+  const long double v = std::ldexp(x, k);
+  if (!(std::fabs(v) < std::ldexp(1.0L, bits))) {
+    *ok = 0;
+    return 0;
+  }
+  return (int64_t)std::llrint(v);
+}
+
 void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm_eos_derived& d, double G) {
   // Li forcing parameter (Eq. LiFS): 0 for the Guo scheme (Eq. GFS), or from eps of
   // Eq. VaporLiqEq for the EOS in use (Sec. III.A)
@@ -42,6 +70,13 @@ void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm
   }
   a.zz_scale = sigma * G * G / 432.0;
   a.kappa_q = r.kappa * G / 24.0;
+  a.fix.ch = fixnum(a.half_force, 36);
+  a.fix.zz = fixnum(a.zz_scale, 1);
+  a.fix.kq = fixnum(a.kappa_q, 36);
+  a.fix.tb = fixnum(a.tau_b, 1);
+  int fits = 1;
+  a.fix.ta = kind == kShearTau ? fixed(a.tau_a, 58, 62, &fits) : 0;
+  if (!fits) a.fix.ta = INT64_MIN;  // |tau_a| >= 16: every node takes the general collision
   if (kind == kFullMrt) {
     const double t[9] = {r.tau_rho, r.tau_e, r.tau_zeta, r.tau_j, r.tau_q, r.tau_j, r.tau_q, r.tau_nu, r.tau_nu};
     for (int k = 0; k < 9; ++k) a.omega[k] = 1.0 / t[k];

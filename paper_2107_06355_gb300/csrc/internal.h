@@ -5,6 +5,7 @@
 #include <cstdint>
 
 #include "../../include/pplbm.h"
+#include "collide_fixed.cuh"
 #include "eos.cuh"
 
 namespace pplbm {
@@ -46,13 +47,14 @@ struct StepArgs {
   // surface-tension control: kappa G / 24, so Q = kappa_q psi(x) q with
   // q = 12 sum_i w_i [psi(x + c_i) - psi(x)] c_i c_i; 0 when off
   double kappa_q;
+  fx::CollideFix fix;  // the same constants as fixed-point factors (collide_fixed.cuh)
 };
 
 // Collision kind of a relaxation set (kUnitTau, kShearTau, kFullMrt), -1 if the set
 // is invalid (reserved word, forcing, kappa finite and < 1, relaxation times > 1/2)
 // (collision_args.cpp).
 int collision_kind(const pplbm_relax* r);
-// The collision fields of a (tau_a, tau_b, zz_scale, kappa_q, omega, li_e, li_z) for
+// The collision fields of a (tau_a, tau_b, zz_scale, kappa_q, omega, li_e, li_z, fix) for
 // the relaxation set r of collision kind `kind`, the EOS d and the interaction G.
 void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm_eos_derived& d, double G);
 

@@ -30,8 +30,8 @@ namespace pplbm {
 // K1 body for node i: moments, EOS, psi (Eqs. Density, Momentum, CS, Sec. III.D,
 // InteractionPotential); error word on a non-finite or non-positive density or psi^2.
 template <int KIND>
-__device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __restrict__ f, int64_t i) {
-  const int64_t N = a.n;
+__device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __restrict__ f, int i) {
+  const int N = (int)a.n;  // 9 n < 2^31: plane offsets fit 32 bits
   const double f0 = f[i], f1 = f[N + i], f2 = f[2 * N + i], f3 = f[3 * N + i], f4 = f[4 * N + i];
   const double f5 = f[5 * N + i], f6 = f[6 * N + i], f7 = f[7 * N + i], f8 = f[8 * N + i];
   double rho, jx, jy, m7 = 0.0, m8 = 0.0;
@@ -350,82 +350,161 @@ __device__ __forceinline__ void collide_full(const StepArgs& a, int64_t node, do
   out.f[8] = bm - (Py - Px);
 }
 
-// K2 body for node (x, y), whose psi sits at sp[c] of a tile with row stride sw:
-// force, collision (with the surface-tension source when ST), then push streaming
-// (or the macroscopic fields when FIELDS, which the source does not change).
-template <int KIND, bool FIELDS, bool ST = false>
-__device__ __forceinline__ void collide_node(const StepArgs& a, int x, int y, const double* sp, int c, int sw,
-                                             double* rho_o, double* ux_o, double* uy_o, double* psi_o) {
-  const double p0 = sp[c];
-  const double pE = sp[c + 1], pW = sp[c - 1], pN = sp[c + sw], pS = sp[c - sw];
-  const double pNE = sp[c + sw + 1], pNW = sp[c + sw - 1], pSW = sp[c - sw - 1], pSE = sp[c - sw + 1];
-  // 12 * sum_i w(|c_i|^2) psi(x + c_i) c_i  (w = 1/3 axis, 1/12 diagonal): exact
-  // integer sums in one fixed-point frame, rounded once (fixsum.cuh); psi > 0 is
-  // normal and finite wherever the density pass left the error word clear
+// Where node (x, y)'s neighbours lie: the columns east and west (periodic), the offsets
+// of its row and of the rows north and south (periodic, or the node's own row where a
+// wall lies beyond: up, down). 32-bit, since 9 nx ny < 2^31.
+struct Place {
+  int x, xe, xw, r, rn, rs;
+  bool up, down;
+};
+
+__device__ __forceinline__ Place place_of(const StepArgs& a, int x, int y) {
+  Place p;
+  const int nx = a.nx, ny = a.ny;
+  p.x = x;
+  p.xe = x + 1 == nx ? 0 : x + 1;
+  p.xw = (x == 0 ? nx : x) - 1;
+  const bool top = y + 1 == ny, bottom = y == 0;
+  p.up = a.walls && top;
+  p.down = a.walls && bottom;
+  p.r = y * nx;
+  p.rn = p.up ? p.r : top ? 0 : p.r + nx;
+  p.rs = p.down ? p.r : (bottom ? ny * nx : p.r) - nx;
+  return p;
+}
+
+// psi at the node and its eight neighbours (C, E, W, N, S, NE, NW, SW, SE) by bit pattern,
+// wall ghosts beyond the walls. Loaded from global memory through L1: the nine values of a
+// 32 x 8 tile come from 34 x 10 distinct ones, and a shared-memory tile with its halo
+// arithmetic and barrier cost 150 instructions per node more than these loads.
+__device__ __forceinline__ void load_psi(const StepArgs& a, const Place& p, fx::u64 (&v)[9]) {
+  const unsigned long long* psi = reinterpret_cast<const unsigned long long*>(a.psi);
+  v[0] = psi[p.r + p.x];
+  v[1] = psi[p.r + p.xe];
+  v[2] = psi[p.r + p.xw];
+  v[3] = psi[p.rn + p.x];
+  v[4] = psi[p.rs + p.x];
+  v[5] = psi[p.rn + p.xe];
+  v[6] = psi[p.rn + p.xw];
+  v[7] = psi[p.rs + p.xw];
+  v[8] = psi[p.rs + p.xe];
+  if (p.up) v[3] = v[5] = v[6] = fx::bits_of(a.psi_ghost_top);
+  if (p.down) v[4] = v[7] = v[8] = fx::bits_of(a.psi_ghost_bottom);
+}
+
+// The collision of a node outside the domain of the fixed-point path (collide_fixed.cuh):
+// force sums, then the general forms above. Kept out of line: it is rare, and inlined it
+// would set the kernels' register count.
+template <int KIND, bool ST>
+__device__ __noinline__ void collide_general(const StepArgs& a, int x, int y, Post* out) {
+  const Place pl = place_of(a, x, y);
+  fx::u64 v[9];
+  load_psi(a, pl, v);
+  double p[9];
+  for (int k = 0; k < 9; ++k) p[k] = fx::double_of(v[k]);
   double gx, gy;
-  fx::shan_chen_stencil(pE, pW, pN, pS, pNE, pNW, pSW, pSE, &gx, &gy);
-  const int64_t N = a.n;
-  const int64_t node = (int64_t)y * a.nx + x;
+  fx::shan_chen_stencil(p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8], &gx, &gy);
+  const int64_t N = a.n, node = pl.r + x;
+  const double rho = a.mom[node], jx = a.mom[N + node], jy = a.mom[2 * N + node];
+  if (ST) {
+    double ux, uy;
+    const SurfQ sq = surface_q(a, p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]);
+    collide_reduced<KIND, ST>(a, node, rho, jx, jy, p[0], gx, gy, sq, *out, &ux, &uy);
+  } else {
+    collide_reduced_fx<KIND>(a, node, rho, jx, jy, p[0], gx, gy, *out);
+  }
+}
+
+// Populations of collide_fixed that are rounded to double by the FP64 pipe's conversion
+// rather than in integer code: the two pipes work side by side.
+constexpr int kFp64Conversions = 4;
+
+template <int KIND, bool ST>
+__device__ __forceinline__ void collide_fast(const StepArgs& a, const Place& pl, int y, const fx::u64 (&psi)[9],
+                                             Post& out) {
+  constexpr bool kShear = KIND == kShearTau;
+  const int N = (int)a.n, node = pl.r + pl.x;
+  const double rho = a.mom[node], jx = a.mom[N + node], jy = a.mom[2 * N + node];
+  double m7 = 0.0, m8 = 0.0;
+  if (kShear) {
+    m7 = a.mom[3 * N + node];
+    m8 = a.mom[4 * N + node];
+  }
+  if (!fx::collide_fixed<kShear, ST, kFp64Conversions>(a.fix, psi, rho, jx, jy, m7, m8, out.f)) {
+    Post g;
+    collide_general<KIND, ST>(a, pl.x, y, &g);
+    out = g;
+  }
+}
+
+// K2 body for node (x, y): force, collision (with the surface-tension source when ST),
+// then push streaming (or the macroscopic fields when FIELDS, which the source does not
+// change).
+template <int KIND, bool FIELDS, bool ST = false>
+__device__ __forceinline__ void collide_node(const StepArgs& a, int x, int y, double* rho_o, double* ux_o,
+                                             double* uy_o, double* psi_o) {
+  const Place pl = place_of(a, x, y);
+  const int N = (int)a.n, node = pl.r + x;
+  fx::u64 psi[9];
+  load_psi(a, pl, psi);
   Post o;
-  double rho, ux, uy;
-  SurfQ sq = {0.0, 0.0, 0.0, 0.0};
-  if (ST && !FIELDS) sq = surface_q(a, p0, pE, pW, pN, pS, pNE, pNW, pSW, pSE);
-  constexpr bool kST = ST && !FIELDS;
-  if (KIND == kFullMrt) {
-    collide_full<kST>(a, node, p0, gx, gy, sq, o, &rho, &ux, &uy);
-  } else if (!FIELDS && (!kST || a.kappa_q == 0.0)) {
+  if (!FIELDS && KIND != kFullMrt) {
     // (a kernel built with the source runs lattices without it, kappa = 0, in a batch:
     // they take the same arithmetic as in the kernel without the source)
-    rho = a.mom[node];
-    collide_reduced_fx<KIND>(a, node, rho, a.mom[N + node], a.mom[2 * N + node], p0, gx, gy, o);
+    if (!ST || a.kappa_q == 0.0)
+      collide_fast<KIND, false>(a, pl, y, psi, o);
+    else
+      collide_fast<KIND, ST>(a, pl, y, psi, o);
   } else {
-    rho = a.mom[node];
-    collide_reduced<KIND, kST>(a, node, rho, a.mom[N + node], a.mom[2 * N + node], p0, gx, gy, sq, o, &ux, &uy);
-  }
-  if (FIELDS) {
-    if (rho_o) rho_o[node] = rho;
-    if (ux_o) ux_o[node] = ux;
-    if (uy_o) uy_o[node] = uy;
-    if (psi_o) psi_o[node] = p0;
-    return;
+    double p[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) p[k] = fx::double_of(psi[k]);
+    // 12 * sum_i w(|c_i|^2) psi(x + c_i) c_i  (w = 1/3 axis, 1/12 diagonal): exact
+    // integer sums in one fixed-point frame, rounded once (fixsum.cuh); psi > 0 is
+    // normal and finite wherever the density pass left the error word clear
+    double gx, gy;
+    fx::shan_chen_stencil(p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8], &gx, &gy);
+    double rho, ux, uy;
+    SurfQ sq = {0.0, 0.0, 0.0, 0.0};
+    constexpr bool kST = ST && !FIELDS;
+    if (kST) sq = surface_q(a, p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]);
+    if (KIND == kFullMrt) {
+      collide_full<kST>(a, node, p[0], gx, gy, sq, o, &rho, &ux, &uy);
+    } else {
+      rho = a.mom[node];
+      collide_reduced<KIND, kST>(a, node, rho, a.mom[N + node], a.mom[2 * N + node], p[0], gx, gy, sq, o, &ux, &uy);
+    }
+    if (FIELDS) {
+      if (rho_o) rho_o[node] = rho;
+      if (ux_o) ux_o[node] = ux;
+      if (uy_o) uy_o[node] = uy;
+      if (psi_o) psi_o[node] = p[0];
+      return;
+    }
   }
   // push streaming: f_i(x + c_i, t + 1) = f*_i(x, t); bounce-back into the opposite
   // population of the same node when x + c_i lies in a wall
   double* __restrict__ out = a.f_out;
-  const int nx = a.nx, ny = a.ny;
-  const int xe = (x + 1 == nx) ? 0 : x + 1;
-  const int xw = (x == 0) ? nx - 1 : x - 1;
-  const int64_t row = (int64_t)y * nx;
   out[node] = o.f[0];
-  out[N + row + xe] = o.f[1];
-  out[3 * N + row + xw] = o.f[3];
-  bool up_wall = false, down_wall = false;
-  int yn = y + 1, ys = y - 1;
-  if (a.walls) {
-    up_wall = (yn == ny);
-    down_wall = (ys < 0);
-  } else {
-    if (yn == ny) yn = 0;
-    if (ys < 0) ys = ny - 1;
-  }
-  const int64_t rn = (int64_t)yn * nx, rs = (int64_t)ys * nx;
-  if (up_wall) {
+  out[N + pl.r + pl.xe] = o.f[1];
+  out[3 * N + pl.r + pl.xw] = o.f[3];
+  if (pl.up) {
     out[4 * N + node] = o.f[2];
     out[7 * N + node] = o.f[5];
     out[8 * N + node] = o.f[6];
   } else {
-    out[2 * N + rn + x] = o.f[2];
-    out[5 * N + rn + xe] = o.f[5];
-    out[6 * N + rn + xw] = o.f[6];
+    out[2 * N + pl.rn + x] = o.f[2];
+    out[5 * N + pl.rn + pl.xe] = o.f[5];
+    out[6 * N + pl.rn + pl.xw] = o.f[6];
   }
-  if (down_wall) {
+  if (pl.down) {
     out[2 * N + node] = o.f[4];
     out[5 * N + node] = o.f[7];
     out[6 * N + node] = o.f[8];
   } else {
-    out[4 * N + rs + x] = o.f[4];
-    out[7 * N + rs + xw] = o.f[7];
-    out[8 * N + rs + xe] = o.f[8];
+    out[4 * N + pl.rs + x] = o.f[4];
+    out[7 * N + pl.rs + pl.xw] = o.f[7];
+    out[8 * N + pl.rs + pl.xe] = o.f[8];
   }
 }
 

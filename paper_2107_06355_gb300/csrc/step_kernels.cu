@@ -26,9 +26,9 @@ constexpr int kTX = 32;  // K2 tile width (one warp along x)
 constexpr int kTY = 8;   // K2 tile height
 
 template <int KIND>
-__global__ void __launch_bounds__(256) k_rho_psi(const StepArgs a) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= a.n) return;
+__global__ void __launch_bounds__(256) k_rho_psi(const __grid_constant__ StepArgs a) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // n < 2^31 / 9
+  if (i >= (int)a.n) return;
   rho_psi_node<KIND>(a, a.f_in, i);
 }
 
@@ -38,16 +38,11 @@ __global__ void __launch_bounds__(256) k_rho_psi(const StepArgs a) {
 constexpr int collide_blocks(int kind, bool st) { return (st && kind == kShearTau) ? 4 : 5; }
 
 template <int KIND, bool FIELDS, bool ST = false>
-__global__ void __launch_bounds__(kTX* kTY, collide_blocks(KIND, ST)) k_collide(const StepArgs a, double* rho_o, double* ux_o, double* uy_o,
-                                                      double* psi_o) {
-  __shared__ double sp[(kTY + 2) * (kTX + 2)];
-  const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * kTY;
-  load_psi_tile(a, sp, x0, y0, kTX, kTY, threadIdx.x, threadIdx.y, threadIdx.y * kTX + threadIdx.x, kTX * kTY);
-  __syncthreads();
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+__global__ void __launch_bounds__(kTX* kTY, collide_blocks(KIND, ST)) k_collide(const __grid_constant__ StepArgs a, double* rho_o, double* ux_o,
+                                                                                     double* uy_o, double* psi_o) {
+  const int x = blockIdx.x * kTX + threadIdx.x, y = blockIdx.y * kTY + threadIdx.y;
   if (x >= a.nx || y >= a.ny) return;
-  collide_node<KIND, FIELDS, ST>(a, x, y, sp, (threadIdx.y + 1) * (kTX + 2) + threadIdx.x + 1, kTX + 2, rho_o, ux_o,
-                                 uy_o, psi_o);
+  collide_node<KIND, FIELDS, ST>(a, x, y, rho_o, ux_o, uy_o, psi_o);
 }
 
 // f_i = f_i^eq(rho0, u0), Eq. EquilibriumDistribution (c_s^2 = 1/3)
