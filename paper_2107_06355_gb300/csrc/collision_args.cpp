@@ -52,6 +52,60 @@ static int64_t fixed(long double x, int k, int bits, int* ok) {
   return (int64_t)std::llrint(v);
 }
 
+// A branch psi^2 2^-s = k3 rho + A + B g((rho - rho0) / a), rho up to rho_top: an ellipse
+// (|rho - rho0| <= a) or the cubic (a its span)
+static LoopFix loop_branch(bool ellipse, long double rho_top, long double rho0, long double a, long double A,
+                           long double B, int* ok) {
+  LoopFix L{};
+  int e;
+  std::frexp(ellipse ? std::fmax(rho_top, 2.0L * a) : rho_top, &e);  // < 2^e
+  L.q = (ellipse ? 63 : 62) - e;
+  if (ellipse) {
+    L.c = fixed(a, L.q, 62, ok);
+    B = B / a * std::ldexp(1.0L, 62 - L.q);
+  } else {
+    while (std::ldexp(1.0L / a, 126 - L.up - L.q) >= 0x1.8p62L) ++L.up;
+    if (L.up > 12) *ok = 0;  // the span is far below a frame this coarse
+    L.c = fixed(1.0L / a, 126 - L.up - L.q, 63, ok);
+  }
+  L.rho0 = fixed(rho0, L.q, 63, ok);
+  L.A = fixnum((double)A, 1);
+  L.B = fixnum((double)B, 1);
+  return L;
+}
+
+EosFix make_eos_fix(const pplbm_eos_derived& d, double G) {
+  EosFix e{};
+  int lb;
+  e.ok = std::frexp(d.b / 4.0, &lb) == 0.5 ? 1 : 0;
+  e.log2_b4 = lb - 1;
+  if (e.log2_b4 < -30 || e.log2_b4 > 30) e.ok = 0;
+  const long double sc = 2.0L / (long double)G, k3 = -sc / 3.0L;
+  std::frexp(k3, &e.s);
+  const long double one = std::ldexp(1.0L, -e.s);  // every constant times 2^-s
+  e.k3_57 = fixed(k3 * one, 57, 57, &e.ok);
+  e.k3_60 = fixed(k3 * one, 60, 60, &e.ok);
+  const bool smooth = d.mode == PPLBM_EOS_SMOOTH || d.mode == PPLBM_EOS_SMOOTH_MOD;
+  for (int i = 0; i < 2; ++i) {
+    const bool v = i == 0 && smooth;
+    CsFix& k = e.cs[i];
+    k.c1 = fixed(2.0L * sc * (long double)d.R * (v ? d.T_v : d.T_l) * one, 62, 63, &e.ok);
+    k.k2 = fixed(-sc * (v ? d.a_v : d.a_l) * one, 58, 62, &e.ok);
+    const double k4 = v ? 0.0 : (double)(sc * d.dP * one);
+    k.k4 = fixnum(k4, 1);
+    k.k4.m >>= 2;  // room for the sum with rho x
+    k.k4.e += 2;
+  }
+  if (smooth) {
+    e.loop = 1;
+    const long double pM = d.p_max, pm = d.p_min, b1 = d.b1, b3 = d.b3, s = sc * one;
+    e.loops[0] = loop_branch(true, d.rho_max, d.rho_max, std::sqrt((long double)d.a1sq), s * (pM - b1), s * b1, &e.loop);
+    e.loops[1] = loop_branch(true, d.rho_l, d.rho_min, std::sqrt((long double)d.a3sq), s * (pm + b3), -s * b3, &e.loop);
+    e.loops[2] = loop_branch(false, d.rho_min, d.rho_max, (long double)d.rho_min - d.rho_max, s * pM, s * (pm - pM), &e.loop);
+  }
+  return e;
+}
+
 void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm_eos_derived& d, double G) {
   // Li forcing parameter (Eq. LiFS): 0 for the Guo scheme (Eq. GFS), or from eps of
   // Eq. VaporLiqEq for the EOS in use (Sec. III.A)
@@ -70,6 +124,7 @@ void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm
   }
   a.zz_scale = sigma * G * G / 432.0;
   a.kappa_q = r.kappa * G / 24.0;
+  a.efix = make_eos_fix(d, G);
   a.fix.ch = fixnum(a.half_force, 36);
   a.fix.zz = fixnum(a.zz_scale, 1);
   a.fix.kq = fixnum(a.kappa_q, 36);

@@ -192,6 +192,12 @@ PPLBM_FX u64 to_double_fp64(i64 n) {
 // adds k to the exponent field of the double with bit pattern b
 PPLBM_FX double scale2(u64 b, int k) { return double_of(b + ((u64)(u32)(k << 20) << 32)); }
 
+// n 2^k as a double (normal or zero), on the FP64 pipe
+PPLBM_FX double frame_to_double(i64 n, int k) {
+  const u64 b = to_double_fp64(n);
+  return scale2(b, hi32(b) ? k : 0);
+}
+
 // A constant of the step as a signed 63-bit factor: x = m 2^e, 2^62 <= |m| < 2^63 (0 for 0).
 struct FixNum {
   i64 m;

@@ -7,6 +7,7 @@
 #include "../../include/pplbm.h"
 #include "collide_fixed.cuh"
 #include "eos.cuh"
+#include "eos_fixed.cuh"
 
 namespace pplbm {
 
@@ -48,13 +49,16 @@ struct StepArgs {
   // q = 12 sum_i w_i [psi(x + c_i) - psi(x)] c_i c_i; 0 when off
   double kappa_q;
   fx::CollideFix fix;  // the same constants as fixed-point factors (collide_fixed.cuh)
+  EosFix efix;         // the EOS likewise (eos_fixed.cuh)
 };
 
 // Collision kind of a relaxation set (kUnitTau, kShearTau, kFullMrt), -1 if the set
 // is invalid (reserved word, forcing, kappa finite and < 1, relaxation times > 1/2)
 // (collision_args.cpp).
 int collision_kind(const pplbm_relax* r);
-// The collision fields of a (tau_a, tau_b, zz_scale, kappa_q, omega, li_e, li_z, fix) for
+// The EOS d with interaction parameter G as fixed-point factors (collision_args.cpp).
+EosFix make_eos_fix(const pplbm_eos_derived& d, double G);
+// The collision fields of a (tau_a, tau_b, zz_scale, kappa_q, omega, li_e, li_z, fix) and efix for
 // the relaxation set r of collision kind `kind`, the EOS d and the interaction G.
 void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm_eos_derived& d, double G);
 

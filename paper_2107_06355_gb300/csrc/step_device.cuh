@@ -27,10 +27,11 @@
 
 namespace pplbm {
 
-// K1 body for node i: moments, EOS, psi (Eqs. Density, Momentum, CS, Sec. III.D,
-// InteractionPotential); error word on a non-finite or non-positive density or psi^2.
+// K1 body for node i in double precision: moments, EOS, psi (Eqs. Density, Momentum, CS,
+// Sec. III.D, InteractionPotential); error word on a non-finite or non-positive density or
+// psi^2. Runs for the general MRT kind and for nodes outside the fixed-point path's domain.
 template <int KIND>
-__device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __restrict__ f, int i) {
+__device__ __forceinline__ void rho_psi_double(const StepArgs& a, const double* __restrict__ f, int i) {
   const int N = (int)a.n;  // 9 n < 2^31: plane offsets fit 32 bits
   const double f0 = f[i], f1 = f[N + i], f2 = f[2 * N + i], f3 = f[3 * N + i], f4 = f[4 * N + i];
   const double f5 = f[5 * N + i], f6 = f[6 * N + i], f7 = f[7 * N + i], f8 = f[8 * N + i];
@@ -79,6 +80,68 @@ __device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __
     m[6 * N + i] = -2.0 * (f2 - f4) + ((f5 + f6) - (f7 + f8));   // row 6 (q_y)
     m[7 * N + i] = (f1 + f3) - (f2 + f4);                        // row 7
     m[8 * N + i] = (f5 + f7) - (f6 + f8);                        // row 8
+  }
+}
+
+template <int KIND>
+__device__ __noinline__ void rho_psi_general(const StepArgs& a, const double* __restrict__ f, int i) {
+  rho_psi_double<KIND>(a, f, i);
+}
+
+// K1 body for node i. Unit relaxation times and the two-phase set take it in fixed point:
+// the moments as exact integer sums in one frame (density_moments), the EOS and psi from
+// the unrounded density sum (eos_fixed.cuh); the FP64 pipe only converts rho and j. Nodes
+// the frames cannot hold (a population at or below zero or not finite, a density or EOS
+// branch outside eos_fixed.cuh's domain) run the double-precision body, which raises the
+// error word. What bounds it: the integer ALU pipe (ncu on a 2048 x 1024 droplet whose
+// warps take the C-S and an ellipse branch: 636 instructions per node, ALU 76 % busy, FP64
+// 31 %, 58 us). With the EOS and the root on the FP64 pipe (15 to 26 FP64 instructions per
+// node) that pipe was 85 % busy and the pass took 107 us; over a batch of 12.9 M nodes
+// 0.444 ms before, 0.301 ms now. The rms error of psi is 0.30 ulp on every branch (0.58
+// next to the vapour at T_r = 0.35), where double precision gave 0.4 to 1.0 (22).
+template <int KIND>
+__device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __restrict__ f, int i) {
+  if (KIND == kFullMrt) {
+    rho_psi_double<KIND>(a, f, i);
+    return;
+  }
+  using namespace fx;
+  const int N = (int)a.n;
+  u64 b[9];
+  u32 mn = 0xFFFFFFFFu, mx = 0u;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    b[k] = bits_of(f[k * N + i]);
+    mn = mn < hi32(b[k]) ? mn : hi32(b[k]);
+    mx = mx > hi32(b[k]) ? mx : hi32(b[k]);
+  }
+  // positive normal populations, the largest in [2^-767, 2^993)
+  bool ok = a.efix.ok && mn >= 0x00100000u && mx - 0x10000000u < 0x6E000000u;
+  const int eg = frame_top(mx);
+  u64 t[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) t[k] = shr_u(significand(b[k]), eg - (int)(hi32(b[k]) >> 20));
+  const u64 sxp = t[1] + t[5] + t[8], sxm = t[3] + t[6] + t[7];  // c_x = +1, -1
+  const u64 syp = t[2] + t[5] + t[6], sym = t[4] + t[7] + t[8];  // c_y = +1, -1
+  const u64 S = t[0] + t[2] + t[4] + sxp + sxm;                  // in [2^59, 2^64)
+  const int k0 = eg - 1086;
+  const double rho = scale2(bits_of(__ull2double_rn(S)), k0);
+  const int lz = clz32((u32)(S >> 32));
+  i64 P;
+  int ex;
+  ok = ok && psi2_fixed(a.efix, a.eos, S << (lz & 31), eg - lz, (i64)bits_of(rho), &P, &ex);
+  if (!ok) {
+    rho_psi_general<KIND>(a, f, i);
+    return;
+  }
+  a.psi[i] = sqrt_double(P, ex);
+  double* __restrict__ m = a.mom;
+  m[i] = rho;
+  m[N + i] = frame_to_double((i64)(sxp - sxm), k0);
+  m[2 * N + i] = frame_to_double((i64)(syp - sym), k0);
+  if (KIND == kShearTau) {
+    m[3 * N + i] = frame_to_double((i64)((t[1] + t[3]) - (t[2] + t[4])), k0);  // row 7 of Eq. MatrixMRT
+    m[4 * N + i] = frame_to_double((i64)((t[5] + t[7]) - (t[6] + t[8])), k0);  // row 8
   }
 }
 
