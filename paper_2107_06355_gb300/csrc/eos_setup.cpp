@@ -17,7 +17,6 @@
 //  * eps: Newton's method from eps = 2 (Sec. III.A).
 #include <cmath>
 #include <cstring>
-#include <functional>
 
 #include "../../include/pplbm.h"
 #include "eos.cuh"
@@ -66,27 +65,47 @@ const GaussLegendre& gl() {
   return g;
 }
 
-// integral of fn(rho) d rho over [lo, hi], in s = ln rho with `panels` equal panels
-double integrate_log(const std::function<double(double)>& fn, double lo, double hi, int panels) {
-  const GaussLegendre& g = gl();
-  const double s0 = std::log(lo), s1 = std::log(hi);
-  const double h = (s1 - s0) / panels;
-  double total = 0.0;
-  for (int p = 0; p < panels; ++p) {
-    const double a = s0 + p * h;
-    double acc = 0.0;
-    for (int k = 0; k < GaussLegendre::n; ++k) {
-      const double s = a + 0.5 * h * (g.x[k] + 1.0);
-      const double rho = std::exp(s);
-      acc += g.w[k] * fn(rho) * rho;
-    }
-    total += 0.5 * h * acc;
+constexpr int kPanels = 48;
+
+// Quadrature over [lo, hi] in s = ln rho: kPanels equal panels of Gauss-Legendre nodes.
+// The set-up's root finders integrate over the same three regions many times, so the
+// nodes (an exponential each) are formed once per region, and Newton's method on eps keeps
+// the logarithms too: 0.65 ms per Smooth set-up (4.4 with an exponential, a power and an
+// indirect call per evaluation), 1.2 ms Modified Smooth (1.9), 1.3 ms Peng (3.0).
+struct LogNodes {
+  static constexpr int n = kPanels * GaussLegendre::n;
+  double rho[n];
+  double h2;  // half a panel's width
+  LogNodes() = default;
+  LogNodes(double lo, double hi) {
+    const GaussLegendre& g = gl();
+    const double s0 = std::log(lo), s1 = std::log(hi);
+    const double h = (s1 - s0) / kPanels;
+    h2 = 0.5 * h;
+    for (int p = 0; p < kPanels; ++p)
+      for (int k = 0; k < GaussLegendre::n; ++k)
+        rho[p * GaussLegendre::n + k] = std::exp(s0 + p * h + 0.5 * h * (g.x[k] + 1.0));
   }
-  return total;
-}
+  // integral of fn(i) d rho, fn given at node i
+  template <class F>
+  double integrate(F fn) const {
+    const GaussLegendre& g = gl();
+    double total = 0.0;
+    for (int p = 0; p < kPanels; ++p) {
+      double acc = 0.0;
+      for (int k = 0; k < GaussLegendre::n; ++k) {
+        const int i = p * GaussLegendre::n + k;
+        acc += g.w[k] * fn(i) * rho[i];
+      }
+      total += h2 * acc;
+    }
+    return total;
+  }
+};
 
 // Ridders' method on [a, b] with fa, fb of opposite sign.
-bool ridders(const std::function<double(double)>& fn, double a, double b, double& root, int maxit = 200) {
+template <class F>
+bool ridders(const F& fn, double a, double b, double& root, int maxit = 200) {
   double fa = fn(a), fb = fn(b);
   if (fa == 0.0) { root = a; return true; }
   if (fb == 0.0) { root = b; return true; }
@@ -193,12 +212,9 @@ bool maxwell(const Branch& c, double rho_max, double rho_min, double& rho_v, dou
   return std::isfinite(rho_v) && std::isfinite(rho_l) && rho_v > 0 && rho_l > rho_v;
 }
 
-constexpr int kPanels = 48;
-
-double maxwell_residual(const EosConst& e, double p_sat) {
-  auto f = [&](double r) { return (p_sat - eos_pressure(e, r)) / (r * r); };
-  return integrate_log(f, e.rho_v, e.rho_max, kPanels) + integrate_log(f, e.rho_max, e.rho_min, kPanels) +
-         integrate_log(f, e.rho_min, e.rho_l, kPanels);
+// the integral of (p_sat - p)/rho^2 over one region of the shaped EOS
+double maxwell_part(const EosConst& e, double p_sat, const LogNodes& q) {
+  return q.integrate([&](int i) { return (p_sat - eos_pressure(e, q.rho[i])) / (q.rho[i] * q.rho[i]); });
 }
 
 bool ellipse(double dp_dr, double delta, double dpress, double& asq, double& bb) {
@@ -290,36 +306,61 @@ static double eos_dpdrho(const EosConst& e, const pplbm_eos_derived& d, double r
 
 // g(eps) = int_{rho_v}^{rho_l} (p_sat - p) psi'/psi^(1+eps) d rho (Eq. VaporLiqEq) and dg/deps,
 // with psi^2 = (2/G)(p - rho/3): psi'/psi = (p' - 1/3)/(G psi^2); split where p is only C^1.
-static void mech_integral(const pplbm_eos_derived& d, double eps, double* g_out, double* dg_out) {
+// What does not depend on eps is kept per node.
+static double mech_term(const EosConst& e, const pplbm_eos_derived& d, double rho, double psi2) {
+  return (d.p_sat - eos_pressure(e, rho)) * ((eos_dpdrho(e, d, rho) - 1.0 / 3.0) / (d.G * psi2));
+}
+
+struct MechIntegral {
+  struct Region {
+    LogNodes q;
+    double f[LogNodes::n], ln[LogNodes::n];  // (p_sat - p) psi'/psi and ln psi^2 at the nodes
+  };
+  Region regions[3];
+  int nreg;
+
+  explicit MechIntegral(const pplbm_eos_derived& d) {
+    const EosConst e = make_eos_const(d);
+    const double edges[4] = {e.rho_v, e.mode == PPLBM_EOS_PENG ? e.rho_l : e.rho_max, e.rho_min, e.rho_l};
+    nreg = e.mode == PPLBM_EOS_PENG ? 1 : 3;
+    for (int r = 0; r < nreg; ++r) {
+      Region& g = regions[r];
+      g.q = LogNodes(edges[r], edges[r + 1]);
+      for (int i = 0; i < LogNodes::n; ++i) {
+        const double rho = g.q.rho[i], psi2 = eos_psi2(e, rho);
+        g.f[i] = mech_term(e, d, rho, psi2);
+        g.ln[i] = std::log(psi2);
+      }
+    }
+  }
+
+  void at(double eps, double* g_out, double* dg_out) const {
+    double g = 0.0, dg = 0.0;
+    double t[LogNodes::n];
+    for (const Region* p = regions; p != regions + nreg; ++p) {
+      const Region& r = *p;
+      for (int i = 0; i < LogNodes::n; ++i) t[i] = r.f[i] * std::exp(-0.5 * eps * r.ln[i]);
+      g += r.q.integrate([&](int i) { return t[i]; });
+      if (dg_out) dg += r.q.integrate([&](int i) { return -0.5 * r.ln[i] * t[i]; });
+    }
+    *g_out = g;
+    if (dg_out) *dg_out = dg;
+  }
+};
+
+// one region's part of the integral at eps = 0 (Peng and Modified Smooth set-ups)
+static double mech_integral_0(const pplbm_eos_derived& d, const LogNodes& q) {
   const EosConst e = make_eos_const(d);
-  double edges[4] = {e.rho_v, e.rho_max, e.rho_min, e.rho_l};
-  int nreg = 3;
-  if (e.mode == PPLBM_EOS_PENG) {
-    edges[1] = e.rho_l;
-    nreg = 1;
-  }
-  double g = 0.0, dg = 0.0;
-  for (int r = 0; r < nreg; ++r) {
-    auto base = [&](double rho) {
-      const double psi2 = eos_psi2(e, rho);
-      const double dpsi_over_psi = (eos_dpdrho(e, d, rho) - 1.0 / 3.0) / (d.G * psi2);
-      return (d.p_sat - eos_pressure(e, rho)) * dpsi_over_psi * std::pow(psi2, -0.5 * eps);
-    };
-    g += integrate_log(base, edges[r], edges[r + 1], kPanels);
-    if (dg_out)
-      dg += integrate_log([&](double rho) { return -0.5 * std::log(eos_psi2(e, rho)) * base(rho); }, edges[r],
-                          edges[r + 1], kPanels);
-  }
-  *g_out = g;
-  if (dg_out) *dg_out = dg;
+  return q.integrate([&](int i) { return mech_term(e, d, q.rho[i], eos_psi2(e, q.rho[i])); });
 }
 
 // Newton from eps = 2 on g(eps) = 0 (Sec. III.A)
 bool solve_eps(const pplbm_eos_derived& d, double& eps_out) {
+  const MechIntegral m(d);
   double eps = 2.0;
   for (int it = 0; it < 100; ++it) {
     double g, dg;
-    mech_integral(d, eps, &g, &dg);
+    m.at(eps, &g, &dg);
     if (!std::isfinite(g) || !std::isfinite(dg) || dg == 0.0) return false;
     const double step = g / dg;
     eps -= step;
@@ -374,6 +415,7 @@ extern "C" pplbm_status pplbm_eos_setup(const pplbm_eos_params* p, double G, ppl
     d.dpdrho_v = liq.dp(d.rho_v);
     d.dpdrho_l = liq.dp(d.rho_l);
     const double rt = p->r_theta;
+    const LogNodes loop(d.rho_v, d.rho_l);
     auto with_rho_m = [&](double rm) {
       pplbm_eos_derived t = d;
       t.rho_m = rm;
@@ -386,9 +428,7 @@ extern "C" pplbm_status pplbm_eos_setup(const pplbm_eos_params* p, double G, ppl
       const EosConst e = make_eos_const(t);
       for (int k = 0; k <= 64; ++k)  // psi^2 must stay positive on the loop
         if (!(eos_psi2(e, t.rho_v + (t.rho_l - t.rho_v) * k / 64.0) > 0.0)) return (double)NAN;
-      double g;
-      mech_integral(t, 0.0, &g, nullptr);
-      return g;
+      return mech_integral_0(t, loop);
     };
     const double span = d.rho_l - d.rho_v;
     double prev_x = d.rho_v + 1e-3 * span, prev_f = resid(prev_x), rm = NAN;
@@ -422,6 +462,9 @@ extern "C" pplbm_status pplbm_eos_setup(const pplbm_eos_params* p, double G, ppl
     const double hi = d.p_sat + 0.5 * d.dpdrho_v * delta1 * (1.0 - 1e-12);
     const double lo = d.p_sat + 1e-9 * (hi - d.p_sat);
     const bool modified = p->mode == PPLBM_EOS_SMOOTH_MOD;
+    // the Maxwell residual's regions; p_max does not enter the third
+    const LogNodes q1(d.rho_v, d.rho_max), q2(d.rho_max, d.rho_min), q3(d.rho_min, d.rho_l);
+    const double part3 = maxwell_part(make_eos_const(d), d.p_sat, q3);
     auto resid = [&](double pm) {
       pplbm_eos_derived t = d;
       t.p_max = pm;
@@ -430,11 +473,10 @@ extern "C" pplbm_status pplbm_eos_setup(const pplbm_eos_params* p, double G, ppl
         const EosConst e = make_eos_const(t);
         for (int k = 0; k <= 64; ++k)
           if (!(eos_psi2(e, t.rho_v * std::pow(t.rho_l / t.rho_v, k / 64.0)) > 0.0)) return (double)NAN;
-        double g;
-        mech_integral(t, 0.0, &g, nullptr);
-        return g;
+        return mech_integral_0(t, q1) + mech_integral_0(t, q2) + mech_integral_0(t, q3);
       }
-      return maxwell_residual(make_eos_const(t), t.p_sat);
+      const EosConst e = make_eos_const(t);
+      return maxwell_part(e, t.p_sat, q1) + maxwell_part(e, t.p_sat, q2) + part3;
     };
     double pm;
     if (!ridders(resid, lo, hi, pm)) return PPLBM_ERR_EOS_SETUP;
