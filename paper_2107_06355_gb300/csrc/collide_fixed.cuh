@@ -86,10 +86,10 @@ template <bool SHEAR, bool ST, int NFP64>
 PPLBM_FX bool collide_fixed(const CollideFix& k, const u64 (&psi)[9], double rho, double jx, double jy, double m7,
                             double m8, double (&f)[9]) {
   // Shan-Chen stencil sums in one frame (see shan_chen_stencil)
-  u32 mx = hi32(psi[1]);
+  // (the source's sums take the node itself in too)
+  u32 mx = max3(hi32(psi[1]), hi32(psi[2]), ST ? hi32(psi[0]) : 0u);
 #pragma unroll
-  for (int i = 2; i < 9; ++i) mx = mx > hi32(psi[i]) ? mx : hi32(psi[i]);
-  if (ST) mx = mx > hi32(psi[0]) ? mx : hi32(psi[0]);  // the source's sums take the node in too
+  for (int i = 3; i < 9; i += 2) mx = max3(mx, hi32(psi[i]), hi32(psi[i + 1]));
   const int eg = frame_top(mx);
   auto at = [&](int i, int up) { return shr_u(significand(psi[i]), eg - up - (int)(hi32(psi[i]) >> 20)); };
   const u64 tE = at(1, 2), tW = at(2, 2), tN = at(3, 2), tS = at(4, 2);
@@ -187,7 +187,7 @@ PPLBM_FX bool collide_fixed(const CollideFix& k, const u64 (&psi)[9], double rho
   // all nine positive with a bit above 2^32, so that they can be rounded in integer code
   i32 lo = (i32)(n[0] >> 32);
 #pragma unroll
-  for (int i = 1; i < 9; ++i) lo = lo < (i32)(n[i] >> 32) ? lo : (i32)(n[i] >> 32);
+  for (int i = 1; i < 9; i += 2) lo = min3s(lo, (i32)(n[i] >> 32), (i32)(n[i + 1] >> 32));
   ok = ok && lo > 0;
   const int sh = er - 1086;
 #pragma unroll

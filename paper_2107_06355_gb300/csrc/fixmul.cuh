@@ -19,6 +19,10 @@
 
 #include "fixsum.cuh"
 
+#ifdef __CUDACC__
+#include <cuda_runtime.h>
+#endif
+
 namespace pplbm {
 namespace fx {
 
@@ -51,6 +55,32 @@ PPLBM_FX int clz32(u32 v) {
   return __clz((int)v);
 #else
   return v ? __builtin_clz(v) : 32;
+#endif
+}
+
+// three-operand extrema, one instruction each (with pairs of comparisons and selects the
+// density pass of 12.9 M nodes took 0.300 ms, 0.282 so; the collision 0.400 and 0.389)
+PPLBM_FX u32 max3(u32 a, u32 b, u32 c) {
+#ifdef __CUDA_ARCH__
+  return __vimax3_u32(a, b, c);
+#else
+  return a > b ? (a > c ? a : c) : (b > c ? b : c);
+#endif
+}
+
+PPLBM_FX u32 min3(u32 a, u32 b, u32 c) {
+#ifdef __CUDA_ARCH__
+  return __vimin3_u32(a, b, c);
+#else
+  return a < b ? (a < c ? a : c) : (b < c ? b : c);
+#endif
+}
+
+PPLBM_FX i32 min3s(i32 a, i32 b, i32 c) {
+#ifdef __CUDA_ARCH__
+  return __vimin3_s32(a, b, c);
+#else
+  return a < b ? (a < c ? a : c) : (b < c ? b : c);
 #endif
 }
 

@@ -108,12 +108,13 @@ __device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __
   using namespace fx;
   const int N = (int)a.n;
   u64 b[9];
-  u32 mn = 0xFFFFFFFFu, mx = 0u;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    b[k] = bits_of(f[k * N + i]);
-    mn = mn < hi32(b[k]) ? mn : hi32(b[k]);
-    mx = mx > hi32(b[k]) ? mx : hi32(b[k]);
+  for (int k = 0; k < 9; ++k) b[k] = bits_of(f[k * N + i]);
+  u32 mn = hi32(b[0]), mx = mn;
+#pragma unroll
+  for (int k = 1; k < 9; k += 2) {
+    mn = min3(mn, hi32(b[k]), hi32(b[k + 1]));
+    mx = max3(mx, hi32(b[k]), hi32(b[k + 1]));
   }
   // positive normal populations, the largest in [2^-767, 2^993)
   bool ok = a.efix.ok && mn >= 0x00100000u && mx - 0x10000000u < 0x6E000000u;
@@ -479,8 +480,9 @@ __device__ __noinline__ void collide_general(const StepArgs& a, int x, int y, Po
 }
 
 // Populations of collide_fixed that are rounded to double by the FP64 pipe's conversion
-// rather than in integer code: the two pipes work side by side.
-constexpr int kFp64Conversions = 4;
+// rather than in integer code: the two pipes work side by side. On 12.9 M nodes with unit
+// relaxation times 4 take 0.389 ms, 6 0.383, 7 0.386, 8 0.387 and 9 0.389.
+constexpr int kFp64Conversions = 6;
 
 template <int KIND, bool ST>
 __device__ __forceinline__ void collide_fast(const StepArgs& a, const Place& pl, int y, const fx::u64 (&psi)[9],
