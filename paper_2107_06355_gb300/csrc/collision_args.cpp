@@ -137,6 +137,13 @@ void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm
     for (int k = 0; k < 9; ++k) a.omega[k] = 1.0 / t[k];
     a.li_e = 12.0 * sigma / (r.tau_e - 0.5);
     a.li_z = 12.0 * sigma / (r.tau_zeta - 0.5);
+    int ok = 1;
+    a.fix.we = fixed(a.omega[1], 61, 62, &ok);
+    a.fix.wz = fixed(a.omega[2], 61, 62, &ok);
+    a.fix.wq = fixed(a.omega[4], 61, 62, &ok);
+    a.fix.wn = fixed(a.omega[7], 61, 62, &ok);
+    a.fix.le = fixnum(a.li_e * G * G / 144.0, 36);
+    a.fix.lz = fixnum(a.li_z * G * G / 144.0, 36);
   }
 }
 

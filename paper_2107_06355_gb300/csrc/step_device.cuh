@@ -29,7 +29,7 @@ namespace pplbm {
 
 // K1 body for node i in double precision: moments, EOS, psi (Eqs. Density, Momentum, CS,
 // Sec. III.D, InteractionPotential); error word on a non-finite or non-positive density or
-// psi^2. Runs for the general MRT kind and for nodes outside the fixed-point path's domain.
+// psi^2. Runs for the nodes outside the fixed-point path's domain.
 template <int KIND>
 __device__ __forceinline__ void rho_psi_double(const StepArgs& a, const double* __restrict__ f, int i) {
   const int N = (int)a.n;  // 9 n < 2^31: plane offsets fit 32 bits
@@ -88,23 +88,19 @@ __device__ __noinline__ void rho_psi_general(const StepArgs& a, const double* __
   rho_psi_double<KIND>(a, f, i);
 }
 
-// K1 body for node i. Unit relaxation times and the two-phase set take it in fixed point:
-// the moments as exact integer sums in one frame (density_moments), the EOS and psi from
-// the unrounded density sum (eos_fixed.cuh); the FP64 pipe only converts rho and j. Nodes
-// the frames cannot hold (a population at or below zero or not finite, a density or EOS
-// branch outside eos_fixed.cuh's domain) run the double-precision body, which raises the
-// error word. What bounds it: the integer ALU pipe (ncu on a 2048 x 1024 droplet whose
+// K1 body for node i, in fixed point: the moments as exact integer sums in one frame
+// (density_moments; with six relaxation times also rows 1, 2, 4, 6, 7, 8), the EOS and psi
+// from the unrounded density sum (eos_fixed.cuh); the FP64 pipe only converts the results.
+// Nodes the frames cannot hold (a population at or below zero or not finite, a density or
+// EOS branch outside eos_fixed.cuh's domain) run the double-precision body, which raises
+// the error word. What bounds it: the integer ALU pipe (ncu on a 2048 x 1024 droplet whose
 // warps take the C-S and an ellipse branch: 636 instructions per node, ALU 76 % busy, FP64
 // 31 %, 58 us). With the EOS and the root on the FP64 pipe (15 to 26 FP64 instructions per
 // node) that pipe was 85 % busy and the pass took 107 us; over a batch of 12.9 M nodes
-// 0.444 ms before, 0.301 ms now. The rms error of psi is 0.30 ulp on every branch (0.58
+// 0.444 ms before, 0.282 ms now. The rms error of psi is 0.30 ulp on every branch (0.58
 // next to the vapour at T_r = 0.35), where double precision gave 0.4 to 1.0 (22).
 template <int KIND>
 __device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __restrict__ f, int i) {
-  if (KIND == kFullMrt) {
-    rho_psi_double<KIND>(a, f, i);
-    return;
-  }
   using namespace fx;
   const int N = (int)a.n;
   u64 b[9];
@@ -143,6 +139,15 @@ __device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __
   if (KIND == kShearTau) {
     m[3 * N + i] = frame_to_double((i64)((t[1] + t[3]) - (t[2] + t[4])), k0);  // row 7 of Eq. MatrixMRT
     m[4 * N + i] = frame_to_double((i64)((t[5] + t[7]) - (t[6] + t[8])), k0);  // row 8
+  } else if (KIND == kFullMrt) {
+    // rows 1, 2, 4, 6, 7, 8, each below 2^63 in magnitude
+    const u64 ax = t[1] + t[2] + t[3] + t[4], dg = t[5] + t[6] + t[7] + t[8];
+    m[3 * N + i] = frame_to_double((i64)(2 * dg - ax - 4 * t[0]), k0);
+    m[4 * N + i] = frame_to_double((i64)(4 * t[0] - 2 * ax + dg), k0);
+    m[5 * N + i] = frame_to_double((i64)(2 * (t[3] - t[1]) + ((t[5] - t[6]) - (t[7] - t[8]))), k0);
+    m[6 * N + i] = frame_to_double((i64)(2 * (t[4] - t[2]) + ((t[5] + t[6]) - (t[7] + t[8]))), k0);
+    m[7 * N + i] = frame_to_double((i64)((t[1] + t[3]) - (t[2] + t[4])), k0);
+    m[8 * N + i] = frame_to_double((i64)((t[5] + t[7]) - (t[6] + t[8])), k0);
   }
 }
 
@@ -470,7 +475,12 @@ __device__ __noinline__ void collide_general(const StepArgs& a, int x, int y, Po
   fx::shan_chen_stencil(p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8], &gx, &gy);
   const int64_t N = a.n, node = pl.r + x;
   const double rho = a.mom[node], jx = a.mom[N + node], jy = a.mom[2 * N + node];
-  if (ST) {
+  if (KIND == kFullMrt) {
+    double r, ux, uy;
+    SurfQ sq = {0.0, 0.0, 0.0, 0.0};
+    if (ST) sq = surface_q(a, p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]);
+    collide_full<ST>(a, node, p[0], gx, gy, sq, *out, &r, &ux, &uy);
+  } else if (ST) {
     double ux, uy;
     const SurfQ sq = surface_q(a, p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]);
     collide_reduced<KIND, ST>(a, node, rho, jx, jy, p[0], gx, gy, sq, *out, &ux, &uy);
@@ -487,20 +497,19 @@ constexpr int kFp64Conversions = 6;
 template <int KIND, bool ST>
 __device__ __forceinline__ void collide_fast(const StepArgs& a, const Place& pl, int y, const fx::u64 (&psi)[9],
                                              Post& out) {
-  constexpr bool kShear = KIND == kShearTau;
   const int N = (int)a.n, node = pl.r + pl.x;
-  const double rho = a.mom[node], jx = a.mom[N + node], jy = a.mom[2 * N + node];
-  double m7 = 0.0, m8 = 0.0;
-  if (kShear) {
-    m7 = a.mom[3 * N + node];
-    m8 = a.mom[4 * N + node];
-  }
-  if (!fx::collide_fixed<kShear, ST, kFp64Conversions>(a.fix, psi, rho, jx, jy, m7, m8, out.f)) {
+  constexpr int kMore = KIND == kUnitTau ? 0 : KIND == kShearTau ? 2 : 6;  // planes beside rho and j
+  double m[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int k = 0; k < kMore; ++k) m[k] = a.mom[(3 + k) * N + node];
+  if (!fx::collide_fixed<KIND, ST, kFp64Conversions>(a.fix, psi, a.mom[node], a.mom[N + node], a.mom[2 * N + node], m,
+                                                     out.f)) {
     Post g;
     collide_general<KIND, ST>(a, pl.x, y, &g);
     out = g;
   }
 }
+static_assert(kUnitTau == fx::kFixUnit && kShearTau == fx::kFixShear && kFullMrt == fx::kFixMrt, "collision forms");
 
 // K2 body for node (x, y): force, collision (with the surface-tension source when ST),
 // then push streaming (or the macroscopic fields when FIELDS, which the source does not
@@ -513,7 +522,7 @@ __device__ __forceinline__ void collide_node(const StepArgs& a, int x, int y, do
   fx::u64 psi[9];
   load_psi(a, pl, psi);
   Post o;
-  if (!FIELDS && KIND != kFullMrt) {
+  if (!FIELDS) {
     // (a kernel built with the source runs lattices without it, kappa = 0, in a batch:
     // they take the same arithmetic as in the kernel without the source)
     if (!ST || a.kappa_q == 0.0)
@@ -530,22 +539,18 @@ __device__ __forceinline__ void collide_node(const StepArgs& a, int x, int y, do
     double gx, gy;
     fx::shan_chen_stencil(p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8], &gx, &gy);
     double rho, ux, uy;
-    SurfQ sq = {0.0, 0.0, 0.0, 0.0};
-    constexpr bool kST = ST && !FIELDS;
-    if (kST) sq = surface_q(a, p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]);
+    const SurfQ sq = {0.0, 0.0, 0.0, 0.0};  // the fields do not depend on the source
     if (KIND == kFullMrt) {
-      collide_full<kST>(a, node, p[0], gx, gy, sq, o, &rho, &ux, &uy);
+      collide_full<false>(a, node, p[0], gx, gy, sq, o, &rho, &ux, &uy);
     } else {
       rho = a.mom[node];
-      collide_reduced<KIND, kST>(a, node, rho, a.mom[N + node], a.mom[2 * N + node], p[0], gx, gy, sq, o, &ux, &uy);
+      collide_reduced<KIND, false>(a, node, rho, a.mom[N + node], a.mom[2 * N + node], p[0], gx, gy, sq, o, &ux, &uy);
     }
-    if (FIELDS) {
-      if (rho_o) rho_o[node] = rho;
-      if (ux_o) ux_o[node] = ux;
-      if (uy_o) uy_o[node] = uy;
-      if (psi_o) psi_o[node] = p[0];
-      return;
-    }
+    if (rho_o) rho_o[node] = rho;
+    if (ux_o) ux_o[node] = ux;
+    if (uy_o) uy_o[node] = uy;
+    if (psi_o) psi_o[node] = p[0];
+    return;
   }
   // push streaming: f_i(x + c_i, t + 1) = f*_i(x, t); bounce-back into the opposite
   // population of the same node when x + c_i lies in a wall

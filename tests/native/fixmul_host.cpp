@@ -6,28 +6,47 @@ using namespace pplbm::fx;
 
 namespace {
 
-template <bool SHEAR, bool ST>
+template <int FORM, bool ST>
 bool one(const CollideFix& k, const double* in, double (&f)[9]) {
   u64 p[9];
   for (int i = 0; i < 9; ++i) p[i] = bits_of(in[i]);
-  return collide_fixed<SHEAR, ST, 4>(k, p, in[9], in[10], in[11], in[12], in[13], f);
+  const double m[6] = {in[12], in[13], in[14], in[15], in[16], in[17]};
+  return collide_fixed<FORM, ST, 4>(k, p, in[9], in[10], in[11], m, f);
 }
 
 }  // namespace
 
 extern "C" {
 
-// rows of 14 (psi at C, E, W, N, S, NE, NW, SW, SE; rho, jx, jy, m7, m8) -> out rows of 10:
-// the nine populations, then 1 if the row is in the domain. c: half_force, zz_scale,
-// kappa_q, tau_a, tau_b as in StepArgs.
-void fm_collide(long long n, int shear, int st, const double* c, const double* in, double* out) {
-  const CollideFix k{pplbm::fixnum(c[0], 36), pplbm::fixnum(c[1], 1), pplbm::fixnum(c[2], 36),
-                     pplbm::fixnum(c[4], 1), (i64)std::ldexp(c[3], 58)};
+// rows of 18 (psi at C, E, W, N, S, NE, NW, SW, SE; rho, jx, jy; the moments: m7, m8 for form
+// 1, rows 1, 2, 4, 6, 7, 8 for form 2) -> out rows of 10: the nine populations, then 1 if the
+// row is in the domain. c: half_force, zz_scale, kappa_q, tau_a, tau_b as in StepArgs, then
+// for form 2 the rates of rows 1, 2, (4, 6), (7, 8) and li_e G^2/144, li_z G^2/144.
+void fm_collide(long long n, int form, int st, const double* c, const double* in, double* out) {
+  CollideFix k{};
+  k.ch = pplbm::fixnum(c[0], 36);
+  k.zz = pplbm::fixnum(c[1], 1);
+  k.kq = pplbm::fixnum(c[2], 36);
+  k.tb = pplbm::fixnum(c[4], 1);
+  k.ta = (i64)std::ldexp(c[3], 58);
+  if (form == 2) {
+    i64* w[4] = {&k.we, &k.wz, &k.wq, &k.wn};
+    for (int i = 0; i < 4; ++i) *w[i] = (i64)std::ldexp(c[5 + i], 61);
+    k.le = pplbm::fixnum(c[9], 36);
+    k.lz = pplbm::fixnum(c[10], 36);
+  }
   for (long long i = 0; i < n; ++i) {
     double f[9];
-    const double* r = in + 14 * i;
-    const bool ok = shear ? (st ? one<true, true>(k, r, f) : one<true, false>(k, r, f))
-                          : (st ? one<false, true>(k, r, f) : one<false, false>(k, r, f));
+    const double* r = in + 18 * i;
+    bool ok;
+    switch (2 * form + st) {
+      case 0: ok = one<0, false>(k, r, f); break;
+      case 1: ok = one<0, true>(k, r, f); break;
+      case 2: ok = one<1, false>(k, r, f); break;
+      case 3: ok = one<1, true>(k, r, f); break;
+      case 4: ok = one<2, false>(k, r, f); break;
+      default: ok = one<2, true>(k, r, f); break;
+    }
     for (int j = 0; j < 9; ++j) out[10 * i + j] = f[j];
     out[10 * i + 9] = ok ? 1.0 : 0.0;
   }
