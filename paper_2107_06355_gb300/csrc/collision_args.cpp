@@ -24,9 +24,7 @@ int collision_kind(const pplbm_relax* r) {
   return kFullMrt;
 }
 
-// x / div as a fixed-point factor m 2^e, 2^62 <= |m| < 2^63, rounded to nearest; m = 0
-// for 0, with an exponent that shifts every product out
-static fx::FixNum fixnum(double x, int div) {
+fx::FixNum fixnum(double x, int div) {
   fx::FixNum r{0, -4096, 0};
   if (x == 0.0 || !std::isfinite(x)) return r;
   int e;

@@ -25,11 +25,13 @@
 
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
 
 #include "../../include/pplbm.h"
 #include "eos_dev.cuh"
+#include "eos_fixed.cuh"
 #include "fixsum.cuh"
 #include "fp64.cuh"
 #include "internal.h"
@@ -62,15 +64,60 @@ struct FDArgs {
   double g0, g1, e0;
 };
 
-__global__ void k_fd_eos(const EosConst e, const double* __restrict__ rho, double* __restrict__ psi,
-                         double* __restrict__ p, int64_t n) {
+// The same constants as fixed-point factors, those of one sum in one frame
+struct FDFix {
+  int ok;              // 0: a constant lies outside the frames (every point takes the general form)
+  int eF, ev, eA;
+  fx::i64 kS4, kL, kD;      // kS / 4, kL, kD: m 2^eF, below 2^62
+  fx::i64 v1, v2, v3, v4;   // m 2^ev (constant viscosities)
+  fx::i64 g0, e0;           // m 2^ev (VV)
+  fx::FixNum g1;            // VV
+  fx::i64 cA;               // m 2^eA
+};
+
+struct FDKernelArgs {
+  FDArgs a;
+  FDFix k;
+};
+
+__device__ __noinline__ void fd_eos_double(const EosConst& e, double r, double* psi, double* p) {
+  const double pr = eos_pressure(e, r);
+  *p = pr;
+  const double psi2 = e.psi2_scale * (pr - r * (1.0 / 3.0));
+  *psi = psi2 > 0.0 ? fast_sqrt(psi2) : sqrt(psi2);  // IEEE result at 0, below 0 and NaN
+}
+
+struct FDEosArgs {
+  EosConst eos;
+  EosFix fix;
+  fx::i64 half;  // |G|/2 2^(63 + fix.s), in (2^61, 2^63): p = rho/3 - |G|/2 psi^2
+};
+
+// psi and p of one density: in fixed point on the integer pipes (eos_fixed.cuh), p from
+// psi^2 before its root; a density outside that domain in double precision. In double
+// precision throughout (25 FP64 instructions per point) the pass was bound by the FP64
+// pipe.
+__global__ void __launch_bounds__(256) k_fd_eos(const __grid_constant__ FDEosArgs a, const double* __restrict__ rho,
+                                                double* __restrict__ psi, double* __restrict__ p, int64_t n) {
+  using namespace fx;
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double r = rho[i];
-  const double pr = eos_pressure(e, r);
-  p[i] = pr;
-  const double psi2 = e.psi2_scale * (pr - r * (1.0 / 3.0));
-  psi[i] = psi2 > 0.0 ? fast_sqrt(psi2) : sqrt(psi2);  // IEEE result at 0, below 0 and NaN
+  const u64 b = bits_of(r), L = significand(b);
+  const int er = (int)(b >> 52);
+  i64 P;
+  int ex;
+  if (a.fix.ok && (u32)(er - 256) < 1664u && psi2_fixed(a.fix, a.eos, L, er, (i64)b, &P, &ex)) {
+    psi[i] = sqrt_double(P, ex);
+    // both terms in units of 2^(er - 1081): rho/3 and |G|/2 psi^2 (P < 2^61)
+    const i64 third = mulhi(factor((i64)(L >> 1)), factor(0x0555555555555555ll));
+    p[i] = frame_to_double(third - mulhi(factor(a.half), factor((i64)((u64)P << 1))), er - 1081);
+    return;
+  }
+  double s, q;
+  fd_eos_double(a.eos, r, &s, &q);
+  psi[i] = s;
+  p[i] = q;
 }
 
 // Wall layers (Eqs. B1, B2), one thread per column of a padded plane set: b1 (row
@@ -194,16 +241,11 @@ __device__ __forceinline__ VelDiffs vel_diffs(double c, double e, double w, doub
   return r;
 }
 
-// PRED: predictor (forward differences) or corrector (backward); VV: tau_nu(rho)
-// viscosities, a compile-time choice so the constant-viscosity kernel carries none
-// of their arithmetic
-// 3 resident blocks per SM (80 registers, 16-36 bytes spilled): the two arithmetic pipes
-// issue 10 % faster than at 2 blocks and 89-94 registers
+// The update of point (x, y) with its products in double precision: PRED: predictor
+// (forward differences) or corrector (backward); VV: tau_nu(rho) viscosities. Runs for the
+// points outside the fixed-point path's domain (fd_update_fixed).
 template <bool PRED, bool VV>
-__global__ void __launch_bounds__(256, 3) k_fd_update(const FDArgs a) {
-  const int x = blockIdx.x * 32 + threadIdx.x;
-  const int y = blockIdx.y * 8 + threadIdx.y;
-  if (x >= a.nx || y >= a.ny) return;
+__device__ __noinline__ void fd_update_general(const FDArgs& a, int x, int y) {
   const int nx = a.nx, ny = a.ny;
   // periodic columns and row offsets of the 5 x 5 neighbourhood, wrapped once
   // (offsets reach +-2, so a grid of width 1 or 2 wraps twice)
@@ -291,6 +333,269 @@ __global__ void __launch_bounds__(256, 3) k_fd_update(const FDArgs a) {
   }
 }
 
+
+// ---- the update in fixed point ------------------------------------------------------
+//
+// Every field's stencil values become integers in one frame (psi: 13 values, the two
+// velocity components together: 18, rho and p: 3 each), so differences are exact, and the
+// products of differences are taken to 64 bits (fixmul.cuh) in frames that follow from
+// the fields' and the constants'. With psi in units of 2^es (psi < 2^60), u of 2^eu (u <
+// 2^59), rho of 2^er and p of 2^ep (below 2^61):
+//   F (the psi terms)      in units of 2^(2 es + 125 + eF),
+//   V (the viscous terms)  in units of 2^(er + eu + 127 + ev),
+//   cA dp                  in units of 2^(ep + 64 + eA);
+// V - F - cA dp is formed in the coarsest of the three, divided by rho and joined with the
+// advection. The units are below the rounding errors that the stored doubles bring into
+// the differences (2^-53 psi, u, rho): F is kept to 2^-56 psi^2 of its coefficients, V to
+// 2^-56 rho u, so the results' errors are those of the double-precision form. Conditions:
+// psi, rho positive, all fields between 2^-320 and 2^100 (smaller velocities and pressures
+// count as zero), and accelerations that leave 3 bits of their frame free.
+//
+// What bounds it: instruction issue and the integer ALU pipe (640 instructions per point, 390
+// of them on that pipe). With its products on the FP64 pipe (54 to 60 instructions per
+// point) and every difference rounded to a double in integer code (1,950) both pipes were 80
+// to 90 % busy. Per step (two updates, two density passes): 1200 x 500 264 -> 115 us, 2048 x
+// 1024 804 -> 314, 600 x 250 with tau(rho) 99 -> 55.
+using fx::Factor;
+using fx::factor;
+using fx::i64;
+using fx::mulhi;
+using fx::mulhi2;
+using fx::u32;
+
+__device__ __forceinline__ u32 i32_of(i64 x) { return (u32)((u64)x >> 32); }
+
+constexpr int kFDThreads = 128, kFDBlocks = 5;
+
+// a value of either sign in the frame with top exponent eg, truncated in magnitude
+__device__ __forceinline__ i64 fd_term(u64 b, int eg) {
+  return fx::with_sign(fx::shr_u(fx::significand(b), eg - (int)(fx::mag_hi(b) >> 20)), b);
+}
+
+__device__ __forceinline__ i64 up(i64 x, int k) { return (i64)((u64)x << k); }
+
+template <bool PRED, bool VV>
+__device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k, const int (&cx)[5],
+                                                const int (&ry)[5], double* drho, double* dux, double* duy) {
+  auto at = [&](const double* f, int dx, int dy) { return fx::bits_of(f[ry[dy + 2] + cx[dx + 2]]); };
+  constexpr u32 kTop = 1123u << 20;  // 2^100
+  // psi: C, E, W, N, S, NE, NW, SW, SE, EE, WW, NN, SS
+  const u64 sb[13] = {at(a.psi, 0, 0),  at(a.psi, 1, 0),   at(a.psi, -1, 0), at(a.psi, 0, 1),  at(a.psi, 0, -1),
+                      at(a.psi, 1, 1),  at(a.psi, -1, 1),  at(a.psi, -1, -1), at(a.psi, 1, -1), at(a.psi, 2, 0),
+                      at(a.psi, -2, 0), at(a.psi, 0, 2),   at(a.psi, 0, -2)};
+  u32 mx = fx::hi32(sb[0]);
+#pragma unroll
+  for (int i = 1; i < 13; i += 2) mx = fx::max3(mx, fx::hi32(sb[i]), fx::hi32(sb[i + 1]));
+  bool ok = k.ok && mx < kTop && mx >= (703u << 20);
+  const int egs = (int)(mx >> 20) + 4, es = egs - 1086;
+  i64 t[13];
+#pragma unroll
+  for (int i = 0; i < 13; ++i)
+    t[i] = (i64)fx::shr_u(fx::significand(sb[i]), egs - (int)(fx::hi32(sb[i]) >> 20));
+  const i64 pd0 = t[1] - t[2], pd1 = t[3] - t[4];
+  const i64 pxx = t[1] + t[2] - 2 * t[0], pyy = t[3] + t[4] - 2 * t[0];
+  const i64 dxy = (t[5] - t[8]) - (t[6] - t[7]), Lc = pxx + pyy;
+  const i64 dl0 = (t[9] - t[10]) + (t[5] + t[8]) - (t[6] + t[7]) - 4 * pd0;
+  const i64 dl1 = (t[11] - t[12]) + (t[5] + t[6]) - (t[8] + t[7]) - 4 * pd1;
+  i64 F0, F1;
+  {
+    const Factor q = factor(dxy), f0 = factor(pd0), f1 = factor(pd1), fl = factor(Lc), fc = factor(4 * t[0]);
+    const Factor kS = factor(k.kS4), kL = factor(k.kL), kD = factor(k.kD);
+    // 4 S_a, S_0 = Pd_0 Pxx + Pd_1 Dxy / 4
+    const i64 s0 = mulhi2(factor(4 * pd0), factor(pxx), q, f1), s1 = mulhi2(factor(4 * pd1), factor(pyy), q, f0);
+    F0 = mulhi(kS, factor(up(s0, 3))) + mulhi(kL, factor(up(mulhi(f0, fl), 3))) +
+         mulhi(kD, factor(up(mulhi(fc, factor(dl0)), 1)));
+    F1 = mulhi(kS, factor(up(s1, 3))) + mulhi(kL, factor(up(mulhi(f1, fl), 3))) +
+         mulhi(kD, factor(up(mulhi(fc, factor(dl1)), 1)));
+  }
+  // velocities, one frame for both components (9 values each: C, E, W, N, S, NE, NW, SW, SE)
+  u64 ub[2][9];
+  u32 mu = 0;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const double* f = c == 0 ? a.ux : a.uy;
+    const u64 v[9] = {at(f, 0, 0), at(f, 1, 0), at(f, -1, 0), at(f, 0, 1),  at(f, 0, -1),
+                      at(f, 1, 1), at(f, -1, 1), at(f, -1, -1), at(f, 1, -1)};
+#pragma unroll
+    for (int i = 0; i < 9; ++i) ub[c][i] = v[i];
+#pragma unroll
+    for (int i = 0; i < 9; i += 3)
+      mu = max(mu, fx::max3(fx::mag_hi(v[i]), fx::mag_hi(v[i + 1]), fx::mag_hi(v[i + 2])));
+  }
+  ok = ok && mu < kTop;
+  const int egu = max((int)(mu >> 20), 703) + 5, eu = egu - 1086;
+  i64 vel[2], D[2][2], xx[2], yy[2], xy[2];  // D[axis][component]
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    i64 v[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) v[i] = fd_term(ub[c][i], egu);
+    vel[c] = v[0];
+    D[0][c] = PRED ? v[1] - v[0] : v[0] - v[2];
+    D[1][c] = PRED ? v[3] - v[0] : v[0] - v[4];
+    xx[c] = v[1] + v[2] - 2 * v[0];
+    yy[c] = v[3] + v[4] - 2 * v[0];
+    xy[c] = (v[5] - v[8]) - (v[6] - v[7]);
+  }
+  const i64 Dv = D[0][0] + D[1][1], Sh = D[0][1] + D[1][0];
+  // rho and p at the point and its one-sided neighbours
+  const u64 rb[3] = {at(a.rho, 0, 0), at(a.rho, PRED ? 1 : -1, 0), at(a.rho, 0, PRED ? 1 : -1)};
+  const u64 pb[3] = {at(a.p, 0, 0), at(a.p, PRED ? 1 : -1, 0), at(a.p, 0, PRED ? 1 : -1)};
+  const u32 mr = max(max(fx::hi32(rb[0]), fx::hi32(rb[1])), fx::hi32(rb[2]));
+  const u32 mn = min(min(fx::hi32(rb[0]), fx::hi32(rb[1])), fx::hi32(rb[2]));
+  const u32 mp = max(max(fx::mag_hi(pb[0]), fx::mag_hi(pb[1])), fx::mag_hi(pb[2]));
+  ok = ok && mr < kTop && mn >= (703u << 20) && mp < kTop;
+  const int egr = (int)(mr >> 20) + 3, er = egr - 1086;
+  const int egp = max((int)(mp >> 20), 703) + 3;
+  i64 r[3], p[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    r[i] = (i64)fx::shr_u(fx::significand(rb[i]), egr - (int)(fx::hi32(rb[i]) >> 20));
+    p[i] = fd_term(pb[i], egp);
+  }
+  const i64 Dr0 = PRED ? r[1] - r[0] : r[0] - r[1], Dr1 = PRED ? r[2] - r[0] : r[0] - r[2];
+  const i64 Dp0 = PRED ? p[1] - p[0] : p[0] - p[1], Dp1 = PRED ? p[2] - p[0] : p[0] - p[2];
+  const Factor cA = factor(k.cA), ux = factor(vel[0]), uy = factor(vel[1]), fDv = factor(Dv), fSh = factor(Sh);
+  // mass: -cA (rho div u + u . grad rho)
+  const i64 m = mulhi(factor(r[0]), fDv) + mulhi2(ux, factor(Dr0), uy, factor(Dr1));
+  *drho = fx::frame_to_double(-mulhi(cA, factor(up(m, 3))), er + eu + 125 + k.eA);
+  // viscous terms
+  i64 v1 = k.v1, v2 = k.v2, v3 = k.v3, v4 = k.v4, w1 = k.v1;  // w1: the one of rho U_yy
+  if (VV) {
+    // mu = rho n1, n1 = g0 + g1 rho, mu_B = rho n2, n2 = e0 - g1 rho; d mu / d rho = n1 + g1 rho
+    const int d = k.ev - (er + 64 + k.g1.e);
+    ok = ok && d >= 0;
+    const i64 gr = fx::shr_s(mulhi(factor(k.g1.m), factor(r[0])), d);
+    ok = ok && (u32)(i32_of(gr) + 0x10000000u) < 0x20000000u;
+    const i64 n1 = k.g0 + gr, n2 = k.e0 - gr;
+    w1 = n1;
+    v1 = n1 + gr;
+    v2 = n2 - gr;
+    v3 = 2 * n1 + n2;
+    v4 = (n1 + n2) >> 2;
+  }
+  const Factor f1 = factor(v1), f2 = factor(v2), f3 = factor(v3), f4 = factor(v4), fw = factor(w1);
+  const Factor dr0 = factor(2 * Dr0), dr1 = factor(2 * Dr1), r2 = factor(2 * r[0]);
+  const i64 V0 = mulhi(f1, factor(up(mulhi2(dr0, factor(D[0][0]), factor(Dr1), fSh), 1))) +
+                 mulhi(f2, factor(mulhi(dr0, fDv))) +
+                 mulhi(r2, factor(mulhi2(f3, factor(xx[0]), f4, factor(xy[1])) + mulhi(fw, factor(yy[0]))));
+  const i64 V1 = mulhi(f1, factor(up(mulhi2(dr1, factor(D[1][1]), factor(Dr0), fSh), 1))) +
+                 mulhi(f2, factor(mulhi(dr1, fDv))) +
+                 mulhi(r2, factor(mulhi2(f3, factor(yy[1]), f4, factor(xy[0])) + mulhi(fw, factor(xx[1]))));
+  // (V - F - cA dp) / rho
+  const int eV = er + eu + 127 + k.ev, eF = 2 * es + 125 + k.eF, eP = egp - 1086 + 64 + k.eA;
+  const int e = max(max(eV, eF), eP);
+  const i64 a0 = fx::shr_s(V0, e - eV) - fx::shr_s(F0, e - eF) - fx::shr_s(mulhi(cA, factor(Dp0)), e - eP);
+  const i64 a1 = fx::shr_s(V1, e - eV) - fx::shr_s(F1, e - eF) - fx::shr_s(mulhi(cA, factor(Dp1)), e - eP);
+  ok = ok && (u32)(i32_of(a0) + 0x08000000u) < 0x10000000u && (u32)(i32_of(a1) + 0x08000000u) < 0x10000000u;
+  const Factor inv = factor(fx::reciprocal<8>(fx::significand(rb[0])));
+  const int e1 = e + 1022 - (int)(fx::hi32(rb[0]) >> 20);
+  // advection: cA u . grad u
+  const Factor ux2 = factor(2 * vel[0]), uy2 = factor(2 * vel[1]);
+  const i64 y0 = mulhi(cA, factor(up(mulhi2(ux2, factor(D[0][0]), uy2, factor(D[1][0])), 3)));
+  const i64 y1 = mulhi(cA, factor(up(mulhi2(ux2, factor(D[0][1]), uy2, factor(D[1][1])), 3)));
+  const int e2 = 2 * eu + 124 + k.eA, em = max(e1, e2);
+  *dux = fx::frame_to_double(fx::shr_s(mulhi(factor(up(a0, 3)), inv), em - e1) - fx::shr_s(y0, em - e2), em);
+  *duy = fx::frame_to_double(fx::shr_s(mulhi(factor(up(a1, 3)), inv), em - e1) - fx::shr_s(y1, em - e2), em);
+  return ok;
+}
+
+template <bool PRED, bool VV>
+__global__ void __launch_bounds__(kFDThreads, kFDBlocks) k_fd_update(const __grid_constant__ FDKernelArgs g) {
+  const FDArgs& a = g.a;
+  const int x = blockIdx.x * 32 + threadIdx.x;
+  const int y = blockIdx.y * (kFDThreads / 32) + threadIdx.y;
+  if (x >= a.nx || y >= a.ny) return;
+  const int nx = a.nx, ny = a.ny;
+  // periodic columns and row offsets of the 5 x 5 neighbourhood, wrapped once (offsets
+  // reach +-2, so a grid of width 1 or 2 wraps twice)
+  auto wrap = [](int v, int n) {
+    if (v < 0) v += n;
+    if (v < 0) v += n;
+    if (v >= n) v -= n;
+    if (v >= n) v -= n;
+    return v;
+  };
+  int cx[5], ry[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    cx[k] = wrap(x + k - 2, nx);
+    ry[k] = (a.walls ? y + k : wrap(y + k - 2, ny)) * nx;  // walls: padded rows, no wrap
+  }
+  double drho, dux, duy;
+  if (!fd_update_fixed<PRED, VV>(a, g.k, cx, ry, &drho, &dux, &duy)) {
+    fd_update_general<PRED, VV>(a, x, y);
+    return;
+  }
+  const int i = ry[2] + x, c = ry[2] + cx[2];
+  const double rho = a.rho[c], ux = a.ux[c], uy = a.uy[c];
+  if (PRED) {
+    a.orho[i] = rho + drho;
+    a.oux[i] = ux + dux;
+    a.ouy[i] = uy + duy;
+  } else {
+    a.orho[i] = 0.5 * (a.rho0[i] + (rho + drho));
+    a.oux[i] = 0.5 * (a.ux0[i] + (ux + dux));
+    a.ouy[i] = 0.5 * (a.uy0[i] + (uy + duy));
+  }
+}
+
+// planes of 2^31 values or more: the general form with its 64-bit offsets
+template <bool PRED, bool VV>
+__global__ void __launch_bounds__(256) k_fd_update_large(const __grid_constant__ FDKernelArgs g) {
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+  if (x < g.a.nx && y < g.a.ny) fd_update_general<PRED, VV>(g.a, x, y);
+}
+
+// The constants of one sum, m 2^e with |m| < 2^62 for the largest of them: e from the
+// largest, 0 for zeros; *ok is cleared outside 2^-60 .. 2^60
+int frame_of(std::initializer_list<double> v, int* ok) {
+  double big = 0.0;
+  for (double x : v) big = std::fmax(big, std::fabs(x));
+  if (big == 0.0) return -62;
+  int e;
+  std::frexp(big, &e);
+  if (!std::isfinite(big) || e < -60 || e > 60) *ok = 0;
+  return e - 62;
+}
+
+fx::i64 in_frame(double x, int e) { return (fx::i64)std::llrint(std::ldexp((long double)x, -e)); }
+
+FDFix fd_fix(const FDArgs& a, bool vary) {
+  FDFix k;
+  std::memset(&k, 0, sizeof(k));
+  k.ok = 1;
+  k.eF = frame_of({0.25 * a.kS, a.kL, a.kD}, &k.ok);
+  k.eA = frame_of({a.cA}, &k.ok);
+  // tau_nu(rho): the largest of the combinations for rho up to 4
+  k.ev = vary ? frame_of({16.0 * a.g0, 16.0 * a.e0, 64.0 * a.g1}, &k.ok) : frame_of({a.v1, a.v2, a.v3, a.v4}, &k.ok);
+  if (!k.ok) return k;
+  k.kS4 = in_frame(0.25 * a.kS, k.eF);
+  k.kL = in_frame(a.kL, k.eF);
+  k.kD = in_frame(a.kD, k.eF);
+  k.cA = in_frame(a.cA, k.eA);
+  if (vary) {
+    k.g0 = in_frame(a.g0, k.ev);
+    k.e0 = in_frame(a.e0, k.ev);
+    k.g1 = fixnum(a.g1, 1);
+  } else {
+    k.v1 = in_frame(a.v1, k.ev);
+    k.v2 = in_frame(a.v2, k.ev);
+    k.v3 = in_frame(a.v3, k.ev);
+    k.v4 = in_frame(a.v4, k.ev);
+  }
+  return k;
+}
+
+template <bool PRED, bool VV>
+void launch_fd_update(const FDKernelArgs& g, int64_t plane, cudaStream_t s) {
+  const int rows = kFDThreads / 32;
+  if (plane < (int64_t)INT32_MAX)
+    k_fd_update<PRED, VV><<<dim3((g.a.nx + 31) / 32, (g.a.ny + rows - 1) / rows), dim3(32, rows), 0, s>>>(g);
+  else
+    k_fd_update_large<PRED, VV><<<dim3((g.a.nx + 31) / 32, (g.a.ny + 7) / 8), dim3(32, 8), 0, s>>>(g);
+}
+
 }  // namespace
 }  // namespace pplbm
 
@@ -303,6 +608,7 @@ struct pplbm_fd {
   int64_t np;    // values per plane: n, or nx (ny + 4) with walls
   int64_t off;   // first fluid value of a plane: 0, or 2 nx with walls
   EosConst eos;
+  FDEosArgs eos_args;
   pplbm_eos_derived derived;
   double G, eps, dx, mu_c, muB_c, tau_e;
   double kappa;   // surface-tension control, 0 = off
@@ -357,6 +663,9 @@ pplbm_status pplbm_fd_create(pplbm_fd** out, const pplbm_lattice* lattice, const
   f->off = f->walls ? 2 * (int64_t)f->nx : 0;
   f->derived = d;
   f->eos = make_eos_const(d);
+  f->eos_args.eos = f->eos;
+  f->eos_args.fix = make_eos_fix(d, G);
+  f->eos_args.half = (fx::i64)std::ldexp(-0.5 * G, 63 + f->eos_args.fix.s);
   f->G = G;
   f->eps = d.eps;
   f->dx = dx;
@@ -399,9 +708,9 @@ pplbm_status pplbm_fd_get_state(pplbm_fd* f, double* rho, double* ux, double* uy
 pplbm_status pplbm_fd_step(pplbm_fd* f, int64_t nsteps, double dt) {
   if (!f || nsteps < 0 || !(dt > 0.0)) return PPLBM_ERR_ARG;
   const unsigned eb = (unsigned)((f->n + 255) / 256);
-  const dim3 grid((f->nx + 31) / 32, (f->ny + 7) / 8), block(32, 8);
-  FDArgs a;
-  std::memset(&a, 0, sizeof(a));
+  FDKernelArgs g;
+  std::memset(&g, 0, sizeof(g));
+  FDArgs& a = g.a;
   a.nx = f->nx;
   a.ny = f->ny;
   a.walls = f->walls ? 1 : 0;
@@ -421,12 +730,13 @@ pplbm_status pplbm_fd_step(pplbm_fd* f, int64_t nsteps, double dt) {
   }
   a.psi = f->psi;
   a.p = f->p;
+  g.k = fd_fix(a, f->var_visc);
   const int64_t n = f->n, np = f->np, off = f->off;
   const unsigned wb = (unsigned)((f->nx + 255) / 256);
   const double two_dy = 2.0 * f->dx, psi_l = f->derived.psi_l;
   // psi and p of the state in X, then its wall layers
   auto eos_pass = [&](double* X) {
-    k_fd_eos<<<eb, 256, 0, f->stream>>>(f->eos, X + off, f->psi + off, f->p + off, n);
+    k_fd_eos<<<eb, 256, 0, f->stream>>>(f->eos_args, X + off, f->psi + off, f->p + off, n);
     if (f->walls)
       k_fd_walls<<<wb, 256, 0, f->stream>>>(f->eos, X, X + np, X + 2 * np, f->psi, f->p, f->nx, f->ny, two_dy,
                                            psi_l);
@@ -441,9 +751,9 @@ pplbm_status pplbm_fd_step(pplbm_fd* f, int64_t nsteps, double dt) {
     a.oux = f->S + np;
     a.ouy = f->S + 2 * np;
     if (f->var_visc)
-      k_fd_update<true, true><<<grid, block, 0, f->stream>>>(a);
+      launch_fd_update<true, true>(g, np, f->stream);
     else
-      k_fd_update<true, false><<<grid, block, 0, f->stream>>>(a);
+      launch_fd_update<true, false>(g, np, f->stream);
     // corrector: U <- (U + U* + dt R_b(U*)) / 2
     eos_pass(f->S);
     a.rho = f->S;
@@ -456,9 +766,9 @@ pplbm_status pplbm_fd_step(pplbm_fd* f, int64_t nsteps, double dt) {
     a.oux = f->U + np;
     a.ouy = f->U + 2 * np;
     if (f->var_visc)
-      k_fd_update<false, true><<<grid, block, 0, f->stream>>>(a);
+      launch_fd_update<false, true>(g, np, f->stream);
     else
-      k_fd_update<false, false><<<grid, block, 0, f->stream>>>(a);
+      launch_fd_update<false, false>(g, np, f->stream);
   }
   f->steps += nsteps;
   return cudaGetLastError() == cudaSuccess ? PPLBM_OK : PPLBM_ERR_CUDA;

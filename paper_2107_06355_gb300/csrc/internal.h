@@ -56,6 +56,9 @@ struct StepArgs {
 // is invalid (reserved word, forcing, kappa finite and < 1, relaxation times > 1/2)
 // (collision_args.cpp).
 int collision_kind(const pplbm_relax* r);
+// x / div as a fixed-point factor m 2^e, 2^62 <= |m| < 2^63, rounded to nearest; m = 0
+// for 0, with an exponent that shifts every product out (collision_args.cpp).
+fx::FixNum fixnum(double x, int div);
 // The EOS d with interaction parameter G as fixed-point factors (collision_args.cpp).
 EosFix make_eos_fix(const pplbm_eos_derived& d, double G);
 // The collision fields of a (tau_a, tau_b, zz_scale, kappa_q, omega, li_e, li_z, fix) and efix for
