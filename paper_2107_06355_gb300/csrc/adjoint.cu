@@ -32,6 +32,7 @@
 
 #include "../../include/pplbm.h"
 #include "ctx.h"
+#include "dependent_launch.cuh"
 #include "step_device.cuh"
 
 namespace pplbm {
@@ -425,7 +426,8 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 }
 
 template <int KIND, bool ST>
-__global__ void __launch_bounds__(kNT) k_adj_collide(const AdjArgs g) {
+__global__ void __launch_bounds__(kNT) k_adj_collide(const __grid_constant__ AdjArgs g) {
+  begin_dependent();
   __shared__ double sp[(kTY + 2) * (kTX + 2)];
   __shared__ double red[kNT];
   const StepArgs& a = g.a;
@@ -559,7 +561,8 @@ __device__ __forceinline__ void load_bar_tiles(const AdjArgs& g, int p0, double*
 // 4 resident blocks per SM (64 registers, 8-16 bytes spilled): at 71 registers and 3
 // blocks the pass's FP64 pipe waits on latency (125 against 109 us on 1024^2)
 template <int KIND, bool ST>
-__global__ void __launch_bounds__(kNT, 4) k_adj_rho_psi(const AdjArgs g) {
+__global__ void __launch_bounds__(kNT, 4) k_adj_rho_psi(const __grid_constant__ AdjArgs g) {
+  begin_dependent();
   constexpr int ts = (kTY + 2) * (kTX + 2);
   __shared__ double tiles[(ST ? 5 : 2) * ts];  // gx_bar, gy_bar (and t_bar, sd_bar, xd_bar)
   __shared__ double red[kNT];
@@ -706,18 +709,18 @@ pplbm_status adjoint_core(pplbm_ctx* c, const StepArgs& a, const double* lam1, d
   const bool st = a.kappa_q != 0.0 || ((g.slots >> G_KAPPA) & 1u);  // with the source (kappa_q may be 0)
   if (a.kind == kShearTau) {
     if (st) {
-      k_adj_collide<kShearTau, true><<<grid, block, 0, c->stream>>>(g);
-      k_adj_rho_psi<kShearTau, true><<<grid, block, 0, c->stream>>>(g);
+      launch_dependent(k_adj_collide<kShearTau, true>, grid, block, c->stream, g);
+      launch_dependent(k_adj_rho_psi<kShearTau, true>, grid, block, c->stream, g);
     } else {
-      k_adj_collide<kShearTau, false><<<grid, block, 0, c->stream>>>(g);
-      k_adj_rho_psi<kShearTau, false><<<grid, block, 0, c->stream>>>(g);
+      launch_dependent(k_adj_collide<kShearTau, false>, grid, block, c->stream, g);
+      launch_dependent(k_adj_rho_psi<kShearTau, false>, grid, block, c->stream, g);
     }
   } else if (st) {
-    k_adj_collide<kUnitTau, true><<<grid, block, 0, c->stream>>>(g);
-    k_adj_rho_psi<kUnitTau, true><<<grid, block, 0, c->stream>>>(g);
+    launch_dependent(k_adj_collide<kUnitTau, true>, grid, block, c->stream, g);
+    launch_dependent(k_adj_rho_psi<kUnitTau, true>, grid, block, c->stream, g);
   } else {
-    k_adj_collide<kUnitTau, false><<<grid, block, 0, c->stream>>>(g);
-    k_adj_rho_psi<kUnitTau, false><<<grid, block, 0, c->stream>>>(g);
+    launch_dependent(k_adj_collide<kUnitTau, false>, grid, block, c->stream, g);
+    launch_dependent(k_adj_rho_psi<kUnitTau, false>, grid, block, c->stream, g);
   }
   if (reduce) k_adj_reduce<<<kNGrad, 256, 0, c->stream>>>(g.partial1, g.partial2, nb, grad);
   const cudaError_t e = cudaGetLastError();

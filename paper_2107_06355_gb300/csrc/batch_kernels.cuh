@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include "dependent_launch.cuh"
 #include "step_device.cuh"
 
 namespace pplbm {
@@ -104,6 +105,7 @@ __device__ __forceinline__ void batch_collide_item(const BatchInst* __restrict__
 
 template <int KIND>
 __global__ void __launch_bounds__(kThreads) k_batch_rho_psi(const BatchInst* inst, const int* owner, int parity) {
+  begin_dependent();
   __shared__ StepArgs sa;
   batch_rho_psi_item<KIND, false>(inst, owner, blockIdx.x, parity, &sa);
 }
@@ -118,6 +120,7 @@ constexpr int collide_min_blocks(int kind) { return kind == kUnitTau ? 5 : 4; }
 template <int KIND, bool ST>
 __global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
     k_batch_collide(const BatchInst* inst, const int* owner, int parity) {
+  begin_dependent();
   __shared__ StepArgs sa;
   __shared__ int org[2];
   batch_collide_item<KIND, ST, false>(inst, owner, blockIdx.x, parity, &sa, org);
@@ -325,16 +328,16 @@ void launch_pair_t(int kind, const BatchInst* inst, const int* o1, int n1, const
                    cudaStream_t s) {
   switch (kind) {
     case kUnitTau:
-      k_batch_rho_psi<kUnitTau><<<n1, kThreads, 0, s>>>(inst, o1, parity);
-      k_batch_collide<kUnitTau, ST><<<n2, kThreads, 0, s>>>(inst, o2, parity);
+      launch_dependent(k_batch_rho_psi<kUnitTau>, n1, kThreads, s, inst, o1, parity);
+      launch_dependent(k_batch_collide<kUnitTau, ST>, n2, kThreads, s, inst, o2, parity);
       break;
     case kShearTau:
-      k_batch_rho_psi<kShearTau><<<n1, kThreads, 0, s>>>(inst, o1, parity);
-      k_batch_collide<kShearTau, ST><<<n2, kThreads, 0, s>>>(inst, o2, parity);
+      launch_dependent(k_batch_rho_psi<kShearTau>, n1, kThreads, s, inst, o1, parity);
+      launch_dependent(k_batch_collide<kShearTau, ST>, n2, kThreads, s, inst, o2, parity);
       break;
     default:
-      k_batch_rho_psi<kFullMrt><<<n1, kThreads, 0, s>>>(inst, o1, parity);
-      k_batch_collide<kFullMrt, ST><<<n2, kThreads, 0, s>>>(inst, o2, parity);
+      launch_dependent(k_batch_rho_psi<kFullMrt>, n1, kThreads, s, inst, o1, parity);
+      launch_dependent(k_batch_collide<kFullMrt, ST>, n2, kThreads, s, inst, o2, parity);
       break;
   }
 }
@@ -374,9 +377,9 @@ void launch_collision_pass(int kind, bool st, const BatchInst* inst, const int* 
 #define PPLBM_K2(K)                                                                   \
   do {                                                                                \
     if (st)                                                                           \
-      k_batch_collide<K, true><<<n2, kThreads, 0, s>>>(inst, o2, parity);             \
+      launch_dependent(k_batch_collide<K, true>, n2, kThreads, s, inst, o2, parity); \
     else                                                                              \
-      k_batch_collide<K, false><<<n2, kThreads, 0, s>>>(inst, o2, parity);            \
+      launch_dependent(k_batch_collide<K, false>, n2, kThreads, s, inst, o2, parity); \
   } while (0)
   switch (kind) {
     case kUnitTau: PPLBM_K2(kUnitTau); break;
@@ -389,9 +392,9 @@ void launch_collision_pass(int kind, bool st, const BatchInst* inst, const int* 
 // the density/psi pass alone, over every instance (refreshes psi and the moments)
 void launch_density_pass(int kind, const BatchInst* inst, const int* o1, int n1, int parity, cudaStream_t s) {
   switch (kind) {
-    case kUnitTau: k_batch_rho_psi<kUnitTau><<<n1, kThreads, 0, s>>>(inst, o1, parity); break;
-    case kShearTau: k_batch_rho_psi<kShearTau><<<n1, kThreads, 0, s>>>(inst, o1, parity); break;
-    default: k_batch_rho_psi<kFullMrt><<<n1, kThreads, 0, s>>>(inst, o1, parity); break;
+    case kUnitTau: launch_dependent(k_batch_rho_psi<kUnitTau>, n1, kThreads, s, inst, o1, parity); break;
+    case kShearTau: launch_dependent(k_batch_rho_psi<kShearTau>, n1, kThreads, s, inst, o1, parity); break;
+    default: launch_dependent(k_batch_rho_psi<kFullMrt>, n1, kThreads, s, inst, o1, parity); break;
   }
 }
 

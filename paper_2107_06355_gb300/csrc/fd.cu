@@ -30,6 +30,7 @@
 #include <string>
 
 #include "../../include/pplbm.h"
+#include "dependent_launch.cuh"
 #include "eos_dev.cuh"
 #include "eos_fixed.cuh"
 #include "fixsum.cuh"
@@ -97,9 +98,10 @@ struct FDEosArgs {
 // psi^2 before its root; a density outside that domain in double precision. In double
 // precision throughout (25 FP64 instructions per point) the pass was bound by the FP64
 // pipe.
-__global__ void __launch_bounds__(256) k_fd_eos(const __grid_constant__ FDEosArgs a, const double* __restrict__ rho,
+__global__ void __launch_bounds__(128) k_fd_eos(const __grid_constant__ FDEosArgs a, const double* __restrict__ rho,
                                                 double* __restrict__ psi, double* __restrict__ p, int64_t n) {
   using namespace fx;
+  begin_dependent();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double r = rho[i];
@@ -125,8 +127,9 @@ __global__ void __launch_bounds__(256) k_fd_eos(const __grid_constant__ FDEosArg
 // fluid rows, p of that density; b2 (row 0) in the solid, psi_b2 = psi_b1 + 2 dy
 // (psi_l - psi_b1); top rows mirror the last fluid rows with the velocity
 // reversed (reflexive layers t1 = row ny + 2, t2 = row ny + 3).
-__global__ void k_fd_walls(const EosConst e, double* rho, double* ux, double* uy, double* psi, double* p, int nx,
+__global__ void __launch_bounds__(64) k_fd_walls(const __grid_constant__ EosConst e, double* rho, double* ux, double* uy, double* psi, double* p, int nx,
                            int ny, double two_dy, double psi_l) {
+  begin_dependent();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= nx) return;
   auto at = [&](int row) { return (int64_t)row * nx + x; };
@@ -355,7 +358,7 @@ __device__ __noinline__ void fd_update_general(const FDArgs& a, int x, int y) {
 // of them on that pipe). With its products on the FP64 pipe (54 to 60 instructions per
 // point) and every difference rounded to a double in integer code (1,950) both pipes were 80
 // to 90 % busy. Per step (two updates, two density passes): 1200 x 500 264 -> 115 us, 2048 x
-// 1024 804 -> 314, 600 x 250 with tau(rho) 99 -> 55.
+// 1024 804 -> 314, 600 x 250 with tau(rho) 99 -> 55; 102, 310 and 42 with dependent launches.
 using fx::Factor;
 using fx::factor;
 using fx::i64;
@@ -502,9 +505,10 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
 
 template <bool PRED, bool VV>
 __global__ void __launch_bounds__(kFDThreads, kFDBlocks) k_fd_update(const __grid_constant__ FDKernelArgs g) {
+  begin_dependent();
   const FDArgs& a = g.a;
   const int x = blockIdx.x * 32 + threadIdx.x;
-  const int y = blockIdx.y * (kFDThreads / 32) + threadIdx.y;
+  const int y = tile_row() * (kFDThreads / 32) + threadIdx.y;
   if (x >= a.nx || y >= a.ny) return;
   const int nx = a.nx, ny = a.ny;
   // periodic columns and row offsets of the 5 x 5 neighbourhood, wrapped once (offsets
@@ -543,6 +547,7 @@ __global__ void __launch_bounds__(kFDThreads, kFDBlocks) k_fd_update(const __gri
 // planes of 2^31 values or more: the general form with its 64-bit offsets
 template <bool PRED, bool VV>
 __global__ void __launch_bounds__(256) k_fd_update_large(const __grid_constant__ FDKernelArgs g) {
+  begin_dependent();
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
   if (x < g.a.nx && y < g.a.ny) fd_update_general<PRED, VV>(g.a, x, y);
 }
@@ -591,9 +596,9 @@ template <bool PRED, bool VV>
 void launch_fd_update(const FDKernelArgs& g, int64_t plane, cudaStream_t s) {
   const int rows = kFDThreads / 32;
   if (plane < (int64_t)INT32_MAX)
-    k_fd_update<PRED, VV><<<dim3((g.a.nx + 31) / 32, (g.a.ny + rows - 1) / rows), dim3(32, rows), 0, s>>>(g);
+    launch_dependent(k_fd_update<PRED, VV>, tile_grid((g.a.nx + 31) / 32, (g.a.ny + rows - 1) / rows), dim3(32, rows), s, g);
   else
-    k_fd_update_large<PRED, VV><<<dim3((g.a.nx + 31) / 32, (g.a.ny + 7) / 8), dim3(32, 8), 0, s>>>(g);
+    launch_dependent(k_fd_update_large<PRED, VV>, dim3((g.a.nx + 31) / 32, (g.a.ny + 7) / 8), dim3(32, 8), s, g);
 }
 
 }  // namespace
@@ -707,7 +712,7 @@ pplbm_status pplbm_fd_get_state(pplbm_fd* f, double* rho, double* ux, double* uy
 
 pplbm_status pplbm_fd_step(pplbm_fd* f, int64_t nsteps, double dt) {
   if (!f || nsteps < 0 || !(dt > 0.0)) return PPLBM_ERR_ARG;
-  const unsigned eb = (unsigned)((f->n + 255) / 256);
+  const unsigned eb = (unsigned)((f->n + 127) / 128);
   FDKernelArgs g;
   std::memset(&g, 0, sizeof(g));
   FDArgs& a = g.a;
@@ -732,14 +737,14 @@ pplbm_status pplbm_fd_step(pplbm_fd* f, int64_t nsteps, double dt) {
   a.p = f->p;
   g.k = fd_fix(a, f->var_visc);
   const int64_t n = f->n, np = f->np, off = f->off;
-  const unsigned wb = (unsigned)((f->nx + 255) / 256);
+  const unsigned wb = (unsigned)((f->nx + 63) / 64);
   const double two_dy = 2.0 * f->dx, psi_l = f->derived.psi_l;
   // psi and p of the state in X, then its wall layers
   auto eos_pass = [&](double* X) {
-    k_fd_eos<<<eb, 256, 0, f->stream>>>(f->eos_args, X + off, f->psi + off, f->p + off, n);
+    launch_dependent(k_fd_eos, eb, 128, f->stream, f->eos_args, X + off, f->psi + off, f->p + off, n);
     if (f->walls)
-      k_fd_walls<<<wb, 256, 0, f->stream>>>(f->eos, X, X + np, X + 2 * np, f->psi, f->p, f->nx, f->ny, two_dy,
-                                           psi_l);
+      launch_dependent(k_fd_walls, wb, 64, f->stream, f->eos, X, X + np, X + 2 * np, f->psi, f->p, f->nx, f->ny, two_dy,
+                       psi_l);
   };
   for (int64_t s = 0; s < nsteps; ++s) {
     // predictor: U* = U + dt R_f(U)

@@ -7,8 +7,8 @@
 //              j = sum f c; plus the stress moments when they relax), evaluates the
 //              equation of state and psi (Eq. InteractionPotential), writes psi and
 //              the moments.
-// K2 collide : stages a (32+2) x (8+2) psi tile in shared memory (periodic wrap in
-//              x, periodic or wall ghost rows in y), computes the Shan-Chen force
+// K2 collide : reads the node's psi stencil (periodic wrap in x, periodic or wall
+//              ghost rows in y), computes the Shan-Chen force
 //              (Eq. ShanChenForce), the velocity with the F/2 shift (Eq. Momentum),
 //              the MRT collision with the Li source (Eqs. OperatorMRT, LiFS,
 //              GFS), optionally the surface-tension source of Sec. V's
@@ -16,31 +16,35 @@
 //              with half-way bounce-back at walls (Sec. IV).
 #include <cuda_runtime.h>
 
+#include "dependent_launch.cuh"
 #include "step_device.cuh"
 
 namespace pplbm {
 
 namespace {
 
-constexpr int kTX = 32;  // K2 tile width (one warp along x)
-constexpr int kTY = 8;   // K2 tile height
+// K2's tile, one warp along x, and K1's block of as many nodes. Small blocks spread a small
+// lattice evenly: with 8 warps per block 33,700 nodes are 153 blocks for 152 SMs (two-phase
+// step 16.9 us, 14.5 with 2 warps); large lattices run at the same rate either way.
+constexpr int kTX = 32, kTY = 2, kStepThreads = kTX * kTY;
 
 template <int KIND>
-__global__ void __launch_bounds__(256) k_rho_psi(const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(kStepThreads) k_rho_psi(const __grid_constant__ StepArgs a) {
+  begin_dependent();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;  // n < 2^31 / 9
   if (i >= (int)a.n) return;
   rho_psi_node<KIND>(a, a.f_in, i);
 }
 
-// 5 resident blocks per SM (48 registers, 8-16 bytes spilled) except the two-phase
-// kernel with the surface-tension source, which would spill 60 bytes: the
-// integer-bound pass issues faster with the extra warps
-constexpr int collide_blocks(int kind, bool st) { return (st && kind == kShearTau) ? 4 : 5; }
+// 40 resident warps per SM (48 registers) except the two-phase kernel with the
+// surface-tension source (32 warps, 64 registers), which would spill too much
+constexpr int collide_blocks(int kind, bool st) { return ((st && kind == kShearTau) ? 32 : 40) / kTY; }
 
 template <int KIND, bool FIELDS, bool ST = false>
-__global__ void __launch_bounds__(kTX* kTY, collide_blocks(KIND, ST)) k_collide(const __grid_constant__ StepArgs a, double* rho_o, double* ux_o,
+__global__ void __launch_bounds__(kStepThreads, collide_blocks(KIND, ST)) k_collide(const __grid_constant__ StepArgs a, double* rho_o, double* ux_o,
                                                                                      double* uy_o, double* psi_o) {
-  const int x = blockIdx.x * kTX + threadIdx.x, y = blockIdx.y * kTY + threadIdx.y;
+  begin_dependent();
+  const int x = blockIdx.x * kTX + threadIdx.x, y = tile_row() * kTY + threadIdx.y;
   if (x >= a.nx || y >= a.ny) return;
   collide_node<KIND, FIELDS, ST>(a, x, y, rho_o, ux_o, uy_o, psi_o);
 }
@@ -99,35 +103,36 @@ __global__ void __launch_bounds__(kGuardThreads) k_guard_final(const double* par
   }
 }
 
-dim3 collide_grid(const StepArgs& a) { return dim3((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY); }
+dim3 collide_grid(const StepArgs& a) { return tile_grid((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY); }
 
 }  // namespace
 
 void launch_rho_psi(const StepArgs& a, void* stream) {
-  const unsigned blocks = (unsigned)((a.n + 255) / 256);
+  const unsigned blocks = (unsigned)((a.n + kStepThreads - 1) / kStepThreads);
   cudaStream_t s = (cudaStream_t)stream;
   switch (a.kind) {
-    case kUnitTau: k_rho_psi<kUnitTau><<<blocks, 256, 0, s>>>(a); break;
-    case kShearTau: k_rho_psi<kShearTau><<<blocks, 256, 0, s>>>(a); break;
-    default: k_rho_psi<kFullMrt><<<blocks, 256, 0, s>>>(a); break;
+    case kUnitTau: launch_dependent(k_rho_psi<kUnitTau>, blocks, kStepThreads, s, a); break;
+    case kShearTau: launch_dependent(k_rho_psi<kShearTau>, blocks, kStepThreads, s, a); break;
+    default: launch_dependent(k_rho_psi<kFullMrt>, blocks, kStepThreads, s, a); break;
   }
 }
 
 void launch_collide(const StepArgs& a, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   const dim3 block(kTX, kTY);
+  double* const none = nullptr;
   if (a.kappa_q != 0.0) {  // with the surface-tension source
     switch (a.kind) {
-      case kUnitTau: k_collide<kUnitTau, false, true><<<collide_grid(a), block, 0, s>>>(a, 0, 0, 0, 0); break;
-      case kShearTau: k_collide<kShearTau, false, true><<<collide_grid(a), block, 0, s>>>(a, 0, 0, 0, 0); break;
-      default: k_collide<kFullMrt, false, true><<<collide_grid(a), block, 0, s>>>(a, 0, 0, 0, 0); break;
+      case kUnitTau: launch_dependent(k_collide<kUnitTau, false, true>, collide_grid(a), block, s, a, none, none, none, none); break;
+      case kShearTau: launch_dependent(k_collide<kShearTau, false, true>, collide_grid(a), block, s, a, none, none, none, none); break;
+      default: launch_dependent(k_collide<kFullMrt, false, true>, collide_grid(a), block, s, a, none, none, none, none); break;
     }
     return;
   }
   switch (a.kind) {
-    case kUnitTau: k_collide<kUnitTau, false><<<collide_grid(a), block, 0, s>>>(a, 0, 0, 0, 0); break;
-    case kShearTau: k_collide<kShearTau, false><<<collide_grid(a), block, 0, s>>>(a, 0, 0, 0, 0); break;
-    default: k_collide<kFullMrt, false><<<collide_grid(a), block, 0, s>>>(a, 0, 0, 0, 0); break;
+    case kUnitTau: launch_dependent(k_collide<kUnitTau, false>, collide_grid(a), block, s, a, none, none, none, none); break;
+    case kShearTau: launch_dependent(k_collide<kShearTau, false>, collide_grid(a), block, s, a, none, none, none, none); break;
+    default: launch_dependent(k_collide<kFullMrt, false>, collide_grid(a), block, s, a, none, none, none, none); break;
   }
 }
 
@@ -135,9 +140,9 @@ void launch_fields(const StepArgs& a, double* rho, double* ux, double* uy, doubl
   cudaStream_t s = (cudaStream_t)stream;
   const dim3 block(kTX, kTY);
   switch (a.kind) {
-    case kUnitTau: k_collide<kUnitTau, true><<<collide_grid(a), block, 0, s>>>(a, rho, ux, uy, psi_out); break;
-    case kShearTau: k_collide<kShearTau, true><<<collide_grid(a), block, 0, s>>>(a, rho, ux, uy, psi_out); break;
-    default: k_collide<kFullMrt, true><<<collide_grid(a), block, 0, s>>>(a, rho, ux, uy, psi_out); break;
+    case kUnitTau: launch_dependent(k_collide<kUnitTau, true>, collide_grid(a), block, s, a, rho, ux, uy, psi_out); break;
+    case kShearTau: launch_dependent(k_collide<kShearTau, true>, collide_grid(a), block, s, a, rho, ux, uy, psi_out); break;
+    default: launch_dependent(k_collide<kFullMrt, true>, collide_grid(a), block, s, a, rho, ux, uy, psi_out); break;
   }
 }
 
