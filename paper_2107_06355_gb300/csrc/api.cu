@@ -2,6 +2,7 @@
 // launches of the step kernels, host/device staging and sticky error handling.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -212,6 +213,7 @@ pplbm_status pplbm_create(pplbm_ctx** out, const pplbm_lattice* lattice, const p
   a.psi_ghost_bottom = d.psi_l;  // liquid below the bottom wall (Sec. IV)
   a.psi_ghost_top = d.psi_v;     // vapour above the top wall
   set_collision_args(a, kind, *relax, d, G);
+  c->small = small_lattice_shape(a);
   *out = c;
   return PPLBM_OK;
 }
@@ -238,7 +240,17 @@ pplbm_status pplbm_init_equilibrium(pplbm_ctx* c, const double* rho0, const doub
 pplbm_status pplbm_step(pplbm_ctx* c, int64_t nsteps) {
   if (!c || nsteps < 0) return fail(c, PPLBM_ERR_ARG, "nsteps < 0");
   if (pplbm_status s = check_sticky(c)) return s;
-  for (int64_t k = 0; k < nsteps; ++k) {
+  int64_t k = 0;
+  while (c->small.blocks > 0 && !c->timing && k < nsteps) {
+    StepArgs& a = c->args;
+    a.f_in = c->fA;
+    a.f_out = c->fB;
+    const int m = (int)std::min<int64_t>(nsteps - k, kClusterSteps);
+    launch_cluster_steps(a, c->small, m, c->stream);
+    if (m & 1) std::swap(c->fA, c->fB);
+    k += m;
+  }
+  for (; k < nsteps; ++k) {
     StepArgs& a = c->args;
     a.f_in = c->fA;
     a.f_out = c->fB;

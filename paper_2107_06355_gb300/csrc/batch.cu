@@ -9,7 +9,8 @@
 // step, chosen by the autotuner:
 //   PLAN_LAUNCHES   two launches per step covering every instance;
 //   PLAN_GRAPH      the same two launches, two steps captured in a CUDA graph that
-//                   is replayed;
+//                   is replayed; a batch of small lattices runs all steps of a call as
+//                   one launch with a cluster per lattice under either (cluster_steps.cuh);
 //   PLAN_PERSISTENT one cooperative launch for all steps of a call: a grid-stride
 //                   loop over work items with a grid barrier between the passes.
 //                   Every barrier wait is bounded: after the spin limit the block
@@ -111,6 +112,7 @@ struct pplbm_batch {
   double* d_gout;                   // guard output, 4 per instance
   bool isolate;                     // diverged instances do not stop the batch
   std::vector<int> diverged;
+  ClusterShape small;               // launches and graph plans of small lattices (cluster_steps.cuh)
   int persistent_grid;
   pplbm_batch_plan plan;
   cudaGraphExec_t graph[2];  // graph[p]: two steps starting from parity p
@@ -460,6 +462,13 @@ pplbm_status issue_steps(pplbm_batch* b, int64_t nsteps, cudaStream_t s) {
     b->parity = (int)((b->parity + nsteps) & 1);
     return PPLBM_OK;
   }
+  while (b->small.blocks > 0 && k < nsteps) {
+    int m = (int)std::min<int64_t>(nsteps - k, kClusterSteps);
+    void* args[] = {(void*)&b->d_inst, (void*)&b->parity, (void*)&m};
+    BTRY(b, launch_clusters(batch_cluster_kernel(b->kind, b->st), b->n, b->small, args, s));
+    b->parity ^= m & 1;
+    k += m;
+  }
   if (b->plan.mode == PPLBM_PLAN_GRAPH) {
     for (; k + 2 <= nsteps; k += 2) BTRY(b, cudaGraphLaunch(b->graph[b->parity], s));
   }
@@ -610,6 +619,13 @@ pplbm_status pplbm_batch_create(pplbm_batch** out, int32_t n, const pplbm_lattic
   occ = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mixed_kernel(b->kind, b->st), kThreads, 0);
   b->mixed_grid = std::max(1, occ * sms);
+  int64_t most = 0, all = 0;
+  for (int i = 0; i < n; ++i) {
+    most = std::max(most, b->host_inst[i].a[0].n);
+    all += b->host_inst[i].a[0].n;
+  }
+  b->small = cluster_shape(batch_cluster_kernel(b->kind, b->st),
+                           b->kind == kFullMrt ? kClusterNodes : kClusterBatchNodes, most, all, n);
   pplbm_status s = apply_plan(b, PPLBM_PLAN_LAUNCHES, 0);
   if (s != PPLBM_OK) {
     pplbm_batch_destroy(b);

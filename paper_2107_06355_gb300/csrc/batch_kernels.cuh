@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include "cluster_steps.cuh"
 #include "dependent_launch.cuh"
 #include "step_device.cuh"
 
@@ -264,6 +265,31 @@ __global__ void __launch_bounds__(kThreads) k_batch_persistent(const BatchInst* 
       batch_collide_item<KIND, ST, true>(inst, owner2, w, parity, &sa, org);
     if (!grid_barrier(bar, err, spin_limit)) return;
   }
+}
+
+// All steps of a call for a batch of small lattices: one cluster per instance.
+template <int KIND, bool ST>
+__global__ void __launch_bounds__(kClusterThreads) k_batch_cluster(const BatchInst* inst, int parity0, int nsteps) {
+  __shared__ StepArgs sa[2];
+  const unsigned long long* src =
+      reinterpret_cast<const unsigned long long*>(inst[blockIdx.x / cluster_blocks()].a);
+  unsigned long long* dst = reinterpret_cast<unsigned long long*>(sa);
+  for (int k = threadIdx.x; k < (int)(sizeof(sa) / 8); k += blockDim.x) dst[k] = src[k];
+  __syncthreads();
+  cluster_steps<KIND, ST>(sa, parity0, nsteps);
+}
+
+template <bool ST>
+const void* batch_cluster_kernel_t(int kind) {
+  switch (kind) {
+    case kUnitTau: return (const void*)k_batch_cluster<kUnitTau, ST>;
+    case kShearTau: return (const void*)k_batch_cluster<kShearTau, ST>;
+    default: return (const void*)k_batch_cluster<kFullMrt, ST>;
+  }
+}
+
+const void* batch_cluster_kernel(int kind, bool st) {
+  return st ? batch_cluster_kernel_t<true>(kind) : batch_cluster_kernel_t<false>(kind);
 }
 
 // Guard, pass 1: one block per 256-node work item of the density pass; per block

@@ -33,6 +33,7 @@ struct pplbm_ctx {
   pplbm_status sticky;
   std::string msg;
   StepArgs args;
+  pplbm::ClusterShape small;  // blocks > 0: steps run as one launch per call
   // kernel timing: event pairs recorded around each launch while enabled
   bool timing;
   std::vector<cudaEvent_t> ev[2];  // per kernel: start/stop interleaved

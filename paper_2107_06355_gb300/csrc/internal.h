@@ -68,6 +68,14 @@ void set_collision_args(StepArgs& a, int kind, const pplbm_relax& r, const pplbm
 // Launchers (step_kernels.cu); all asynchronous on `stream`.
 void launch_rho_psi(const StepArgs& a, void* stream);
 void launch_collide(const StepArgs& a, void* stream);
+// Small lattices (cluster_steps.cuh): the shape of the cluster that advances a lattice,
+// blocks = 0 if the two step kernels do; nsteps (at most kClusterSteps) steps in one launch.
+struct ClusterShape {
+  int blocks, threads;
+};
+constexpr int kClusterSteps = 1000;
+ClusterShape small_lattice_shape(const StepArgs& a);
+void launch_cluster_steps(const StepArgs& a, ClusterShape shape, int nsteps, void* stream);
 void launch_fields(const StepArgs& a, double* rho, double* ux, double* uy, double* psi_out, void* stream);
 void launch_init_eq(const StepArgs& a, double* f, const double* rho0, const double* ux0, const double* uy0,
                     void* stream);

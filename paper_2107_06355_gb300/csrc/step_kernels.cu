@@ -16,6 +16,7 @@
 //              with half-way bounce-back at walls (Sec. IV).
 #include <cuda_runtime.h>
 
+#include "cluster_steps.cuh"
 #include "dependent_launch.cuh"
 #include "step_device.cuh"
 
@@ -103,6 +104,28 @@ __global__ void __launch_bounds__(kGuardThreads) k_guard_final(const double* par
   }
 }
 
+template <int KIND, bool ST>
+__global__ void __launch_bounds__(kClusterThreads) k_cluster_steps(const __grid_constant__ StepArgs a, int nsteps) {
+  __shared__ StepArgs sa[2];
+  if (threadIdx.x == 0) {
+    sa[0] = a;
+    sa[1] = a;
+    sa[1].f_in = a.f_out;
+    sa[1].f_out = const_cast<double*>(a.f_in);
+  }
+  __syncthreads();
+  cluster_steps<KIND, ST>(sa, 0, nsteps);
+}
+
+const void* cluster_kernel(int kind, bool st) {
+  switch (kind) {
+    case kUnitTau: return st ? (const void*)k_cluster_steps<kUnitTau, true> : (const void*)k_cluster_steps<kUnitTau, false>;
+    case kShearTau:
+      return st ? (const void*)k_cluster_steps<kShearTau, true> : (const void*)k_cluster_steps<kShearTau, false>;
+    default: return st ? (const void*)k_cluster_steps<kFullMrt, true> : (const void*)k_cluster_steps<kFullMrt, false>;
+  }
+}
+
 dim3 collide_grid(const StepArgs& a) { return tile_grid((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY); }
 
 }  // namespace
@@ -134,6 +157,15 @@ void launch_collide(const StepArgs& a, void* stream) {
     case kShearTau: launch_dependent(k_collide<kShearTau, false>, collide_grid(a), block, s, a, none, none, none, none); break;
     default: launch_dependent(k_collide<kFullMrt, false>, collide_grid(a), block, s, a, none, none, none, none); break;
   }
+}
+
+ClusterShape small_lattice_shape(const StepArgs& a) {
+  return cluster_shape(cluster_kernel(a.kind, a.kappa_q != 0.0), kClusterNodes, a.n, a.n, 1);
+}
+
+void launch_cluster_steps(const StepArgs& a, ClusterShape shape, int nsteps, void* stream) {
+  void* args[] = {(void*)&a, (void*)&nsteps};
+  launch_clusters(cluster_kernel(a.kind, a.kappa_q != 0.0), 1, shape, args, (cudaStream_t)stream);
 }
 
 void launch_fields(const StepArgs& a, double* rho, double* ux, double* uy, double* psi_out, void* stream) {
