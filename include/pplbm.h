@@ -255,7 +255,7 @@ pplbm_status pplbm_run_host(pplbm_ctx* ctx, const double* rho0, const double* ux
  * are device memory unless noted. */
 #define PPLBM_NGRAD 15
 
-/* Bytes of the adjoint workspace (adjoint planes, lambda ping-pong, per-block partials). */
+/* Bytes of the adjoint workspace (adjoint planes, lambda ping-pong, per-warp partials). */
 size_t pplbm_adjoint_workspace_bytes(const pplbm_lattice* lattice);
 /* One adjoint step at the state f_t (9 planes): lambda_t = (d f^{t+1}/d f^t)^T lambda_next,
  * grad += (d f^{t+1}/d constants)^T lambda_next. Uses the context's psi/moment planes.

@@ -19,10 +19,10 @@
 //      through psi = sqrt(psi^2(rho; constants)) to rho_bar and the constants'
 //      adjoints; lambda^t_i = rho_bar + c_i . j_bar (+ the rows 7, 8 of Eq. MatrixMRT
 //      times the stress moments' adjoints with the two-phase set).
-// Constant adjoints are reduced per block and summed in a fixed order
-// (deterministic); over a checkpointed rollout each block's sums accumulate
-// across the steps and are reduced once at the end. Blocks with no node on a
-// branch whose constants depend on alpha skip those reductions. The host maps
+// Constant adjoints are summed per warp in a fixed order (deterministic, no block
+// barriers); over a rollout each warp's sums accumulate across the steps and are reduced
+// once at the end. Warps with no node on a branch whose constants depend on alpha skip those
+// sums. The host maps
 // the adjoints to d/d alpha with dconstants/dalpha.
 #include <cuda_runtime.h>
 
@@ -31,6 +31,7 @@
 #include <cstring>
 
 #include "../../include/pplbm.h"
+#include "adjoint_fixed.cuh"
 #include "ctx.h"
 #include "dependent_launch.cuh"
 #include "step_device.cuh"
@@ -38,8 +39,9 @@
 namespace pplbm {
 namespace {
 
-constexpr int kTX = 32, kTY = 8, kNT = kTX * kTY;
-// adjoint workspace: kBarPlanes adjoint planes, two 9-plane lambda buffers, per-block partials
+// blocks of two rows of one warp each: with 8 rows 256^2 nodes are 256 blocks for 152 SMs
+constexpr int kTX = 32, kTY = 2, kNT = kTX * kTY;
+// adjoint workspace: kBarPlanes adjoint planes, two 9-plane lambda buffers, per-warp partials
 constexpr int kBarPlanes = 11;
 constexpr int kLamOffset = kBarPlanes;            // in planes of n values
 constexpr int kPartialOffset = kBarPlanes + 18;
@@ -50,10 +52,7 @@ enum {
   G_PMAX = 0, G_B1, G_IA1, G_A2, G_B2, G_PMIN, G_B3, G_IA3, G_ZZ, G_K1V, G_K2V, G_K1L, G_K2L, G_K4L, G_KAPPA, kNGrad
 };
 static_assert(kNGrad == PPLBM_NGRAD, "gradient slot count");
-// A1 reduces G_ZZ and G_KAPPA (two values per block), A2 every other slot; A2's
-// local index of slot k (k != G_ZZ, k < G_KAPPA)
-constexpr int kA2 = kNGrad - 2;
-__host__ __device__ constexpr int a2_index(int k) { return k < G_ZZ ? k : k - 1; }
+// (A1 sums G_ZZ and G_KAPPA, A2 every other slot)
 
 struct AdjArgs {
   StepArgs a;            // forward arguments of step t (psi, mom filled by K1 on f^t)
@@ -62,10 +61,12 @@ struct AdjArgs {
   double* bar;           // kBarPlanes planes: rho_bar, jx_bar, jy_bar, psi_bar (own), gx_bar, gy_bar,
                          // the surface-tension sums' t_bar, sd_bar, xd_bar, and (two-phase set)
                          // the stress moments' m7_bar, m8_bar
-  double* partial1;      // per A1 block: the zz-scale and kappa adjoints
-  double* partial2;      // per A2 block: kA2 constant adjoints (slot order without G_ZZ, G_KAPPA)
-  int accumulate;        // add this step's block sums to the partials (a rollout) instead of storing them
-  unsigned slots;        // bit k set: gradient slot k is accumulated (others stay 0)
+  double* partial;       // the constants' adjoints summed per warp: slot k of warp w at k nw + w
+  int nw;                // warps: rows of 32 nodes
+  int accumulate;        // add this step's sums to the partials (a rollout) instead of storing them
+  unsigned slots;        // bit k set: gradient slot k is accumulated (others are not touched)
+  double q1, q3;         // ellipses: dp/drho 2/G = q d / s
+  double h1, h3;         // a^2 / 2
 };
 
 // bits of the slots [k0, k1] of a group
@@ -354,316 +355,368 @@ __device__ __forceinline__ void collide_reduced_reverse(const StepArgs& a, doubl
   *jy_b = jyb;
 }
 
-// psi^2(rho) and its derivatives w.r.t. rho and the alpha-dependent constants (eos_dev.cuh);
-// the C-S branch constants' derivatives only when bulk_slots (a uniform flag)
-__device__ __forceinline__ double psi2_grad(const EosConst& e, double rho, bool bulk_slots, double* dc) {
-  for (int k = 0; k < kA2; ++k) dc[k] = 0.0;
+// d psi^2 / d rho on the C-S branches and the Peng loop in double precision (eos_dev.cuh):
+// densities outside cs_slope_fixed's domain.
+__device__ __noinline__ double slope_general(const EosConst& e, double rho) {
   const long long rb = dbits(rho);
   const bool vap = rb <= e.bits_rho_v, liq = rb >= e.bits_rho_l;
-  if (e.mode == 2 && !vap && !liq) {  // Peng cubic loop: no alpha-dependent constants
+  if (e.mode == 2 && !vap && !liq) {
     const double dv = rho - e.rho_v, dl = rho - e.rho_l, dm = rho - e.rho_m;
     const double dp = e.theta * (dl * dm + dv * dm + dv * dl);
     return e.psi2_scale * (dp - 1.0 / 3.0);
   }
-  if (e.mode != 1 || vap || liq) {
-    const bool use_v = (e.mode == 1) && vap;
-    const double k1 = use_v ? e.k1_v : e.k1_l, k2 = use_v ? e.k2_v : e.k2_l;
-    const double eta = e.b4 * rho, om = 1.0 - eta;
-    const double r = fast_rcp(om), r2 = r * r;
-    // psi^2 = rho (k1 Z + k2 rho + k3) + k4 (k4 of the vapour branch is 0), Z of Eq. CS;
-    // d(rho Z)/drho = Z + eta Z'(eta) = (1 + 4 eta + 4 eta^2 - 4 eta^3 + eta^4) / (1 - eta)^4
-    const double P = fma(eta, fma(eta, fma(eta, eta - 4.0, 4.0), 4.0), 1.0);
-    if (bulk_slots) {  // constant indices only, so dc stays in registers
-      const double Z = fma(eta, fma(eta, om, 1.0), 1.0) * (r2 * r);
-      const double rz = rho * Z, rr = rho * rho;
-      dc[a2_index(G_K1V)] = use_v ? rz : 0.0;
-      dc[a2_index(G_K2V)] = use_v ? rr : 0.0;
-      dc[a2_index(G_K1L)] = use_v ? 0.0 : rz;
-      dc[a2_index(G_K2L)] = use_v ? 0.0 : rr;
-      dc[a2_index(G_K4L)] = use_v ? 0.0 : 1.0;
+  const bool use_v = (e.mode == 1) && vap;
+  const double k1 = use_v ? e.k1_v : e.k1_l, k2 = use_v ? e.k2_v : e.k2_l;
+  const double eta = e.b4 * rho, om = 1.0 - eta;
+  const double r = fast_rcp(om), r2 = r * r;
+  // psi^2 = rho (k1 Z + k2 rho + k3) + k4 (k4 of the vapour branch is 0), Z of Eq. CS;
+  // d(rho Z)/drho = Z + eta Z'(eta) = (1 + 4 eta + 4 eta^2 - 4 eta^3 + eta^4) / (1 - eta)^4
+  const double P = fma(eta, fma(eta, fma(eta, eta - 4.0, 4.0), 4.0), 1.0);
+  return fma(k1 * (r2 * r2), P, fma(2.0 * k2, rho, e.k3));
+}
+
+// Sums over a warp, in a fixed order.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(~0u, v, m);
+  return v;
+}
+
+// Eight sums at once: each exchange halves the values a lane holds, so they cost 9 FP64
+// additions instead of 40. Lanes 4 j hold the sum of v[j].
+__device__ __forceinline__ double warp_sum8(double (&v)[8]) {
+  const int lane = threadIdx.x;
+#pragma unroll
+  for (int m = 16, h = 4; h > 0; m >>= 1, h >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double keep = up ? v[i + h] : v[i], send = up ? v[i] : v[i + h];
+      v[i] = keep + __shfl_xor_sync(~0u, send, m);
     }
-    return fma(k1 * (r2 * r2), P, fma(2.0 * k2, rho, e.k3));
   }
-  const double s = e.psi2_scale;
-  double dp;
-  if (rb <= e.bits_rho_max) {
-    const double d = rho - e.rho_max;
-    const double s1 = fast_sqrt(fma(-d * d, e.inv_a1sq, 1.0));
-    const double q = e.b1 * d * fast_rcp(s1);
-    dp = -q * e.inv_a1sq;
-    dc[a2_index(G_PMAX)] = s;
-    dc[a2_index(G_B1)] = s * (s1 - 1.0);
-    dc[a2_index(G_IA1)] = -0.5 * s * q * d;
-  } else if (rb < e.bits_rho_min) {
-    const double t = (rho - e.rho_max) * e.inv_span;
-    dp = (3.0 * e.a2 * t + 2.0 * e.b2) * t * e.inv_span;
-    dc[a2_index(G_PMAX)] = s;
-    dc[a2_index(G_A2)] = s * t * t * t;
-    dc[a2_index(G_B2)] = s * t * t;
-  } else {
-    const double d = rho - e.rho_min;
-    const double s3 = fast_sqrt(fma(-d * d, e.inv_a3sq, 1.0));
-    const double q = e.b3 * d * fast_rcp(s3);
-    dp = q * e.inv_a3sq;
-    dc[a2_index(G_PMIN)] = s;
-    dc[a2_index(G_B3)] = s * (1.0 - s3);
-    dc[a2_index(G_IA3)] = 0.5 * s * q * d;
-  }
-  return s * (dp - 1.0 / 3.0);
+  v[0] += __shfl_xor_sync(~0u, v[0], 2);
+  return v[0] + __shfl_xor_sync(~0u, v[0], 1);
 }
 
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  red[threadIdx.y * kTX + threadIdx.x] = v;
-  __syncthreads();
-  for (int w = kNT / 2; w > 0; w >>= 1) {
-    const int t = threadIdx.y * kTX + threadIdx.x;
-    if (t < w) red[t] += red[t + w];
-    __syncthreads();
-  }
-  const double r = red[0];
-  __syncthreads();
-  return r;
+// the warp's row of 32 nodes (x0 .. x0 + 31, y)
+__device__ __forceinline__ int warp_index(int y) { return y * gridDim.x + blockIdx.x; }
+
+// one warp's share of slot k; a warp has its own place, so the additions' order is the steps'
+__device__ __forceinline__ void add_partial(const AdjArgs& g, int k, int w, double v) {
+  double* dst = g.partial + (int64_t)k * g.nw + w;
+  if (g.accumulate)
+    atomicAdd(dst, v);
+  else
+    *dst = v;
 }
 
+// mu_i(x) = lambda^{t+1} at the node the push sent f*_i to
+__device__ __forceinline__ void gather_mu(const AdjArgs& g, const Place& pl, double (&mu)[9]) {
+  const int N = (int)g.a.n, x = pl.x, node = pl.r + x;
+  const double* L1 = g.lam1;
+  mu[0] = L1[node];
+  mu[1] = L1[N + pl.r + pl.xe];
+  mu[3] = L1[3 * N + pl.r + pl.xw];
+  mu[2] = pl.up ? L1[4 * N + node] : L1[2 * N + pl.rn + x];
+  mu[5] = pl.up ? L1[7 * N + node] : L1[5 * N + pl.rn + pl.xe];
+  mu[6] = pl.up ? L1[8 * N + node] : L1[6 * N + pl.rn + pl.xw];
+  mu[4] = pl.down ? L1[2 * N + node] : L1[4 * N + pl.rs + x];
+  mu[7] = pl.down ? L1[5 * N + node] : L1[7 * N + pl.rs + pl.xw];
+  mu[8] = pl.down ? L1[6 * N + node] : L1[8 * N + pl.rs + pl.xe];
+}
+
+// A1 of a node in double precision (with the forward's integer stages): nodes outside the
+// fixed-point path's domain.
 template <int KIND, bool ST>
-__global__ void __launch_bounds__(kNT) k_adj_collide(const __grid_constant__ AdjArgs g) {
-  begin_dependent();
-  __shared__ double sp[(kTY + 2) * (kTX + 2)];
-  __shared__ double red[kNT];
+__device__ __noinline__ void adj_collide_general(const AdjArgs& g, int x, int y, double* zs_b, double* kap_b) {
   const StepArgs& a = g.a;
-  const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * kTY;
-  load_psi_tile(a, sp, x0, y0, kTX, kTY, threadIdx.x, threadIdx.y, threadIdx.y * kTX + threadIdx.x, kNT);
-  __syncthreads();
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-  double zs_b = 0.0, kap_b = 0.0;
-  if (x < a.nx && y < a.ny) {
-    const int c = (threadIdx.y + 1) * (kTX + 2) + threadIdx.x + 1, sw = kTX + 2;
-    const double p0 = sp[c];
-    // the forward collision pass's stencil sums (same arithmetic, same force)
-    double gx, gy;
-    fx::shan_chen_stencil(sp[c + 1], sp[c - 1], sp[c + sw], sp[c - sw], sp[c + sw + 1], sp[c + sw - 1],
-                          sp[c - sw - 1], sp[c - sw + 1], &gx, &gy);
-    const int64_t N = a.n, node = (int64_t)y * a.nx + x;
-    const int nx = a.nx, ny = a.ny;
-    const int xe = (x + 1 == nx) ? 0 : x + 1, xw = (x == 0) ? nx - 1 : x - 1;
-    int yn = y + 1, ys = y - 1;
-    bool up = false, down = false;
-    if (a.walls) {
-      up = (yn == ny);
-      down = (ys < 0);
-    } else {
-      if (yn == ny) yn = 0;
-      if (ys < 0) ys = ny - 1;
-    }
-    const int64_t row = (int64_t)y * nx, rn = (int64_t)yn * nx, rs = (int64_t)ys * nx;
-    const double* L1 = g.lam1;
-    // mu_i(x) = lambda^{t+1} at the node the push sent f*_i to
-    double mu[9];
-    mu[0] = L1[node];
-    mu[1] = L1[N + row + xe];
-    mu[3] = L1[3 * N + row + xw];
-    mu[2] = up ? L1[4 * N + node] : L1[2 * N + rn + x];
-    mu[5] = up ? L1[7 * N + node] : L1[5 * N + rn + xe];
-    mu[6] = up ? L1[8 * N + node] : L1[6 * N + rn + xw];
-    mu[4] = down ? L1[2 * N + node] : L1[4 * N + rs + x];
-    mu[7] = down ? L1[5 * N + node] : L1[7 * N + rs + xw];
-    mu[8] = down ? L1[6 * N + node] : L1[8 * N + rs + xe];
-    double rb, jxb, jyb, pb, gxb, gyb;
-    double st_b[4] = {0.0, 0.0, 0.0, 0.0};  // the source's k_b, t_b, sd_b, xd_b
-    SurfQ sq = {0.0, 0.0, 0.0, 0.0};
-    if (ST)
-      sq = surface_q(a, p0, sp[c + 1], sp[c - 1], sp[c + sw], sp[c - sw], sp[c + sw + 1], sp[c + sw - 1],
-                     sp[c - sw - 1], sp[c - sw + 1]);
-    double* B = g.bar;
-    if (!ST || a.kappa_q == 0.0) {
-      // the forward ran collide_reduced_fx (no source, or kappa = 0 in a kernel with it)
-      double m7b = 0.0, m8b = 0.0, src[4] = {0.0, 0.0, 0.0, 0.0};
-      const bool shear = KIND == kShearTau;
-      collide_reduced_reverse<KIND == kShearTau, ST>(a, a.mom[node], a.mom[N + node], a.mom[2 * N + node],
-                                                     shear ? a.mom[3 * N + node] : 0.0,
-                                                     shear ? a.mom[4 * N + node] : 0.0, p0, gx, gy, mu, &rb, &jxb,
-                                                     &jyb, &m7b, &m8b, &pb, &gxb, &gyb, &zs_b, src);
-      if (shear) {
-        B[9 * N + node] = m7b;
-        B[10 * N + node] = m8b;
-      }
-      if (ST) {
-        // the source's adjoints at k = kappa_q psi = 0 (forward: zz += k t; unit: the
-        // axis populations' m7*/4 parts -= +-k sd, Pxy -= k xd; two-phase: m7* -= 4 omega
-        // k sd, m8* -= omega k xd): only the k adjoint is non-zero
-        if (shear)
-          st_b[0] = fma(src[0], sq.t, -src[3] * fma(4.0 * sq.sd, src[1], sq.xd * src[2]));
-        else
-          st_b[0] = fma(src[0], sq.t, -fma(4.0 * src[1], sq.sd, src[2] * sq.xd));
-      }
-    } else if (KIND == kShearTau) {
-      double m7b, m8b;
-      collide_shear_reverse(a, a.mom[node], a.mom[N + node], a.mom[2 * N + node], a.mom[3 * N + node],
-                            a.mom[4 * N + node], p0, gx, gy, mu, ST ? &sq : nullptr, &rb, &jxb, &jyb, &m7b, &m8b, &pb,
-                            &gxb, &gyb, &zs_b, st_b);
+  const Place pl = place_of(a, x, y);
+  fx::u64 v[9];
+  load_psi(a, pl, v);
+  double p[9];
+  for (int k = 0; k < 9; ++k) p[k] = fx::double_of(v[k]);
+  const double p0 = p[0];
+  // the forward collision pass's stencil sums
+  double gx, gy;
+  fx::shan_chen_stencil(p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8], &gx, &gy);
+  const int64_t N = a.n, node = pl.r + x;
+  double mu[9];
+  gather_mu(g, pl, mu);
+  double rb, jxb, jyb, pb, gxb, gyb;
+  double st_b[4] = {0.0, 0.0, 0.0, 0.0};  // the source's k_b, t_b, sd_b, xd_b
+  SurfQ sq = {0.0, 0.0, 0.0, 0.0};
+  if (ST)
+    sq = surface_q(a, p0, p[1], p[2], p[3], p[4], p[5], p[6], p[7], p[8]);
+  double* B = g.bar;
+  if (!ST || a.kappa_q == 0.0) {
+    // the forward ran collide_reduced_fx (no source, or kappa = 0 in a kernel with it)
+    double m7b = 0.0, m8b = 0.0, src[4] = {0.0, 0.0, 0.0, 0.0};
+    const bool shear = KIND == kShearTau;
+    collide_reduced_reverse<KIND == kShearTau, ST>(a, a.mom[node], a.mom[N + node], a.mom[2 * N + node],
+                                                   shear ? a.mom[3 * N + node] : 0.0,
+                                                   shear ? a.mom[4 * N + node] : 0.0, p0, gx, gy, mu, &rb, &jxb,
+                                                   &jyb, &m7b, &m8b, &pb, &gxb, &gyb, zs_b, src);
+    if (shear) {
       B[9 * N + node] = m7b;
       B[10 * N + node] = m8b;
-    } else {
-      double zq_b[4];
-      collide_unit_reverse(a, a.mom[node], a.mom[N + node], a.mom[2 * N + node], p0, gx, gy, mu, &rb, &jxb, &jyb,
-                           &pb, &gxb, &gyb, &zs_b, ST ? zq_b : nullptr);
-      if (ST) {
-        // forward: zz += k t, axp -= k sd, ayp += k sd, Pxy -= k xd, k = kappa_q psi(x)
-        const double dsd = zq_b[2] - zq_b[1];
-        st_b[0] = fma(zq_b[0], sq.t, fma(dsd, sq.sd, -zq_b[3] * sq.xd));
-        st_b[1] = zq_b[0] * sq.k;
-        st_b[2] = dsd * sq.k;
-        st_b[3] = -zq_b[3] * sq.k;
-      }
     }
     if (ST) {
-      // own node: k = kappa_q psi(x), and t carries -psi(x); kappa_q = kappa G / 24
-      pb += fma(st_b[0], a.kappa_q, -st_b[1]);
-      kap_b = st_b[0] * p0 * (a.G / 24.0);
-      B[6 * N + node] = st_b[1];
-      B[7 * N + node] = st_b[2];
-      B[8 * N + node] = st_b[3];
+      // the source's adjoints at k = kappa_q psi = 0 (forward: zz += k t; unit: the
+      // axis populations' m7*/4 parts -= +-k sd, Pxy -= k xd; two-phase: m7* -= 4 omega
+      // k sd, m8* -= omega k xd): only the k adjoint is non-zero
+      if (shear)
+        st_b[0] = fma(src[0], sq.t, -src[3] * fma(4.0 * sq.sd, src[1], sq.xd * src[2]));
+      else
+        st_b[0] = fma(src[0], sq.t, -fma(4.0 * src[1], sq.sd, src[2] * sq.xd));
     }
-    B[node] = rb;
-    B[N + node] = jxb;
-    B[2 * N + node] = jyb;
-    B[3 * N + node] = pb;
-    B[4 * N + node] = gxb;
-    B[5 * N + node] = gyb;
+  } else if (KIND == kShearTau) {
+    double m7b, m8b;
+    collide_shear_reverse(a, a.mom[node], a.mom[N + node], a.mom[2 * N + node], a.mom[3 * N + node],
+                          a.mom[4 * N + node], p0, gx, gy, mu, ST ? &sq : nullptr, &rb, &jxb, &jyb, &m7b, &m8b, &pb,
+                          &gxb, &gyb, zs_b, st_b);
+    B[9 * N + node] = m7b;
+    B[10 * N + node] = m8b;
+  } else {
+    double zq_b[4];
+    collide_unit_reverse(a, a.mom[node], a.mom[N + node], a.mom[2 * N + node], p0, gx, gy, mu, &rb, &jxb, &jyb,
+                         &pb, &gxb, &gyb, zs_b, ST ? zq_b : nullptr);
+    if (ST) {
+      // forward: zz += k t, axp -= k sd, ayp += k sd, Pxy -= k xd, k = kappa_q psi(x)
+      const double dsd = zq_b[2] - zq_b[1];
+      st_b[0] = fma(zq_b[0], sq.t, fma(dsd, sq.sd, -zq_b[3] * sq.xd));
+      st_b[1] = zq_b[0] * sq.k;
+      st_b[2] = dsd * sq.k;
+      st_b[3] = -zq_b[3] * sq.k;
+    }
+  }
+  if (ST) {
+    // own node: k = kappa_q psi(x), and t carries -psi(x); kappa_q = kappa G / 24
+    pb += fma(st_b[0], a.kappa_q, -st_b[1]);
+    *kap_b = st_b[0] * p0 * (a.G / 24.0);
+    B[6 * N + node] = st_b[1];
+    B[7 * N + node] = st_b[2];
+    B[8 * N + node] = st_b[3];
+  }
+  B[node] = rb;
+  B[N + node] = jxb;
+  B[2 * N + node] = jyb;
+  B[3 * N + node] = pb;
+  B[4 * N + node] = gxb;
+  B[5 * N + node] = gyb;
+}
+
+// A1. What bounds it: integer issue on large lattices (1,090 instructions per node, 590 on
+// the ALU pipe; with the two-phase set and the source 1,780, 890), latency on small ones. With
+// its products on the FP64 pipe (41 to 122 instructions per node) and every stage's sums
+// rounded to doubles in integer code it was bound by both pipes: 1024^2 108 us, now 50 (with
+// the two-phase set and the source 256, now 113). In fixed point with blocks of 256 threads
+// and a block-wide sum it took 68 (141) there, but 35 us against 23 before on 300 x 125.
+// 10 resident blocks (96 registers), 8 for the two-phase set (128), without spills.
+template <int KIND, bool ST>
+__global__ void __launch_bounds__(kNT, KIND == kShearTau ? 8 : 10) k_adj_collide(const __grid_constant__ AdjArgs g) {
+  begin_dependent();
+  const StepArgs& a = g.a;
+  const int x = blockIdx.x * kTX + threadIdx.x, y = tile_row() * kTY + threadIdx.y;
+  if (y >= a.ny) return;
+  double zs_b = 0.0, kap_b = 0.0;
+  if (x < a.nx) {
+    constexpr bool kShear = KIND == kShearTau;
+    const Place pl = place_of(a, x, y);
+    const int N = (int)a.n, node = pl.r + x;
+    fx::u64 psi[9];
+    load_psi(a, pl, psi);
+    double mu[9];
+    gather_mu(g, pl, mu);
+    fx::ReverseOut o;
+    if (fx::collide_reverse_fixed<kShear, ST>(a.fix, psi, a.mom[node], a.mom[N + node], a.mom[2 * N + node],
+                                              kShear ? a.mom[3 * N + node] : 0.0, kShear ? a.mom[4 * N + node] : 0.0,
+                                              mu, &o)) {
+      double* B = g.bar;
+      double rb = o.rho_b, pb = o.psi_b;
+      if (ST) {
+        // the source: zz += k t, p7 -= 4 omega k sd / 36, p8 -= omega k xd / 36
+        const double p0 = fx::double_of(psi[0]);
+        const SurfQ sq = {a.kappa_q * p0, o.t6 * (1.0 / 6.0), o.sd, o.xd};
+        const double u7 = o.u7 * (1.0 / 36.0), u8 = o.u8 * (1.0 / 36.0), om = kShear ? o.om : 1.0;
+        const double w = fma(4.0 * sq.sd, u7, sq.xd * u8);
+        const double k_b = fma(o.u6, sq.t, -om * w);
+        double t_b = 0.0, sd_b = 0.0, xd_b = 0.0;
+        if (a.kappa_q != 0.0) {
+          t_b = o.u6 * sq.k;
+          sd_b = -4.0 * om * sq.k * u7;
+          xd_b = -om * sq.k * u8;
+          if (kShear) rb = fma(sq.k * w * om, om * a.tau_b, rb);  // d omega / d rho = -tau_b omega^2
+        }
+        // own node: k = kappa_q psi(x), and t carries -psi(x); kappa_q = kappa G / 24
+        pb += fma(k_b, a.kappa_q, -t_b);
+        kap_b = k_b * p0 * (a.G / 24.0);
+        B[6 * N + node] = t_b;
+        B[7 * N + node] = sd_b;
+        B[8 * N + node] = xd_b;
+      }
+      if (kShear) {
+        B[9 * N + node] = o.m7_b;
+        B[10 * N + node] = o.m8_b;
+      }
+      zs_b = o.zs_b;
+      B[node] = rb;
+      B[N + node] = o.jx_b;
+      B[2 * N + node] = o.jy_b;
+      B[3 * N + node] = pb;
+      B[4 * N + node] = o.gx_b;
+      B[5 * N + node] = o.gy_b;
+    } else {
+      double z = 0.0, k = 0.0;
+      adj_collide_general<KIND, ST>(g, x, y, &z, &k);
+      zs_b = z;
+      kap_b = k;
+    }
   }
   // grid-uniform tests
-  const double s = (g.slots >> G_ZZ) & 1u ? block_sum(zs_b, red) : 0.0;
-  const double sk = ST && ((g.slots >> G_KAPPA) & 1u) ? block_sum(kap_b, red) : 0.0;
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    double* dst = g.partial1 + 2 * (blockIdx.y * gridDim.x + blockIdx.x);
-    dst[0] = g.accumulate ? dst[0] + s : s;
-    dst[1] = g.accumulate ? dst[1] + sk : sk;
+  const int w = warp_index(y);
+  if ((g.slots >> G_ZZ) & 1u) {
+    const double v = warp_sum(zs_b);
+    if (threadIdx.x == 0) add_partial(g, G_ZZ, w, v);
+  }
+  if (ST && ((g.slots >> G_KAPPA) & 1u)) {
+    const double v = warp_sum(kap_b);
+    if (threadIdx.x == 0) add_partial(g, G_KAPPA, w, v);
   }
 }
 
-// tiles of adjoint planes p0 .. p0 + NP - 1 with a one-node halo (zero beyond a wall:
-// ghosts carry no adjoint); tile j at s + j * (kTY + 2) * (kTX + 2)
-template <int NP>
-__device__ __forceinline__ void load_bar_tiles(const AdjArgs& g, int p0, double* s, int x0, int y0) {
-  const StepArgs& a = g.a;
-  const int sw = kTX + 2, ts = (kTY + 2) * sw;
-  for (int k = threadIdx.y * kTX + threadIdx.x; k < ts; k += kNT) {
-    const int ty = k / sw, tx = k - ty * sw;
-    const int gx = wrap_index(x0 + tx - 1, a.nx);
-    int gy = y0 + ty - 1;
-    const bool in = !a.walls || (gy >= 0 && gy < a.ny);
-    if (!a.walls) gy = wrap_index(gy, a.ny);
-#pragma unroll
-    for (int j = 0; j < NP; ++j) s[j * ts + k] = in ? g.bar[(p0 + j) * a.n + (int64_t)gy * a.nx + gx] : 0.0;
-  }
-}
-
-// 4 resident blocks per SM (64 registers, 8-16 bytes spilled): at 71 registers and 3
-// blocks the pass's FP64 pipe waits on latency (125 against 109 us on 1024^2)
+// A2. What bounds it: integer issue (1,440 instructions per node, 890 on the ALU pipe, 38
+// on the FP64 pipe with alpha's slots; 22 without). With the C-S slope, the reciprocals and
+// the block-wide sums on the FP64 pipe (121 instructions per warp and node, 12 additions per
+// slot in each block's trees, up to 90 block barriers) that pipe was 81 % busy: 1024^2 248
+// us, now 85 (two-phase with the source 156, now 82). A gradient's step in all, 256^2 60 us
+// -> 28, 1024^2 466 -> 180, 300 x 125 with the source 64 -> 31, 60^2 46 -> 16. 12 resident
+// blocks (80 registers); 16 (64 registers) gain 1 % at 1024^2 and lose 10 % at 256^2.
 template <int KIND, bool ST>
-__global__ void __launch_bounds__(kNT, 4) k_adj_rho_psi(const __grid_constant__ AdjArgs g) {
+__global__ void __launch_bounds__(kNT, 12) k_adj_rho_psi(const __grid_constant__ AdjArgs g) {
   begin_dependent();
-  constexpr int ts = (kTY + 2) * (kTX + 2);
-  __shared__ double tiles[(ST ? 5 : 2) * ts];  // gx_bar, gy_bar (and t_bar, sd_bar, xd_bar)
-  __shared__ double red[kNT];
-  double* sx = tiles;
-  double* sy = tiles + ts;
   const StepArgs& a = g.a;
-  const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * kTY;
-  load_bar_tiles<ST ? 5 : 2>(g, 4, tiles, x0, y0);
-  __syncthreads();
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-  double dcsum[kA2];
-  for (int k = 0; k < kA2; ++k) dcsum[k] = 0.0;
-  // which constants this node's branch uses: the shaped loop's, the vapour C-S's
-  // or the liquid C-S's
-  bool shaped = false, vap_side = false, liq_side = false;
-  if (x < a.nx && y < a.ny) {
-    const int c = (threadIdx.y + 1) * (kTX + 2) + threadIdx.x + 1, sw = kTX + 2;
-    // transpose of g = 12 sum_c w_c psi(x + c) c, gathered at this node y, plus the
-    // node's own psi adjoint (one fixed-point frame, fixsum.cuh)
-    const int64_t N = a.n, node = (int64_t)y * a.nx + x;
-    const double gv[13] = {g.bar[3 * N + node], sx[c - 1], sx[c + 1], sy[c - sw], sy[c + sw],
-                           sx[c - sw - 1], sy[c - sw - 1], sx[c + sw + 1], sy[c + sw + 1],
-                           sx[c + sw - 1], sy[c + sw - 1], sx[c - sw + 1], sy[c - sw + 1]};
-    double psi_b = fx::psi_adjoint_gather(gv);
-    if constexpr (ST) {
-      // transposes of t = (axis sum)/6 + (diagonal sum)/12 - psi(x), sd = (pE + pW) - (pN + pS),
-      // xd = (pNE + pSW) - (pNW + pSE) at the neighbours (the -psi(x) term is A1's)
-      const double* st = tiles + 2 * ts;
-      const double* sd = tiles + 3 * ts;
-      const double* sq = tiles + 4 * ts;
-      const double ta = (st[c + 1] + st[c - 1]) + (st[c + sw] + st[c - sw]);
-      const double tg = (st[c + sw + 1] + st[c - sw - 1]) + (st[c + sw - 1] + st[c - sw + 1]);
-      psi_b += fma(1.0 / 6.0, ta, fma(1.0 / 12.0, tg, ((sd[c + 1] + sd[c - 1]) - (sd[c + sw] + sd[c - sw])) +
-                                                      ((sq[c + sw + 1] + sq[c - sw - 1]) - (sq[c + sw - 1] + sq[c - sw + 1]))));
-    }
-    const double rho = a.mom[node];
-    const double psi = a.psi[node];
-    double dc[kA2];
-    const double dpsi2 = psi2_grad(a.eos, rho, (g.slots & slot_bits(G_K1V, G_K4L)) != 0u, dc);
-    const double psi2_b = 0.5 * psi_b * fast_rcp(psi);  // psi = sqrt(psi^2) > 0 (checked by the step)
-    const double rho_b = g.bar[node] + psi2_b * dpsi2;
-    const long long rb = dbits(rho);
-    const bool vap = rb <= a.eos.bits_rho_v, liq = rb >= a.eos.bits_rho_l;
-    // as in psi2_grad: C-S (shape 0) uses the liquid constants everywhere, the Peng
-    // loop (2) outside (rho_v, rho_l), the shaped EOS (1) on its liquid branch
-    const int m = a.eos.mode;
-    shaped = m == 1 && !vap && !liq && (g.slots & slot_bits(G_PMAX, G_IA3));
-    vap_side = m == 1 && vap && (g.slots & slot_bits(G_K1V, G_K2V));
-    liq_side = (m == 0 || (m == 2 && (vap || liq)) || (m == 1 && liq)) && (g.slots & slot_bits(G_K1L, G_K4L));
-    // only the group this node's branch uses is non-zero (constant loop bounds)
-    if (shaped)
-      for (int k = a2_index(G_PMAX); k <= a2_index(G_IA3); ++k) dcsum[k] = psi2_b * dc[k];
-    if (vap_side)
-      for (int k = a2_index(G_K1V); k <= a2_index(G_K2V); ++k) dcsum[k] = psi2_b * dc[k];
-    if (liq_side)
-      for (int k = a2_index(G_K1L); k <= a2_index(G_K4L); ++k) dcsum[k] = psi2_b * dc[k];
-    const double jxb = g.bar[N + node], jyb = g.bar[2 * N + node];
-    // lambda^t_i = rho_bar + c_i . j_bar (+ rows 7, 8 of Eq. MatrixMRT times the stress
-    // moments' adjoints with the two-phase set), exact in one frame (fixsum.cuh)
-    constexpr bool kShear = KIND == kShearTau;
-    double l[9];
-    fx::lambda_assembly<kShear>(rho_b, jxb, jyb, kShear ? g.bar[9 * N + node] : 0.0,
-                                kShear ? g.bar[10 * N + node] : 0.0, l);
-    double* L0 = g.lam0;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) L0[k * N + node] = l[k];
+  const int x = blockIdx.x * kTX + threadIdx.x, y = tile_row() * kTY + threadIdx.y;
+  if (y >= a.ny) return;
+  const bool in = x < a.nx;  // the others repeat the last node, without results
+  const Place pl = place_of(a, in ? x : a.nx - 1, y);
+  const int64_t N = a.n;
+  const int node = pl.r + pl.x;
+  // neighbours in the rows above and below; beyond a wall they are ghosts with no adjoint
+  auto above = [&](const double* p, int c) { return pl.up ? 0.0 : p[pl.rn + c]; };
+  auto below = [&](const double* p, int c) { return pl.down ? 0.0 : p[pl.rs + c]; };
+  // transpose of g = 12 sum_c w_c psi(x + c) c, gathered at this node, plus the node's own
+  // psi adjoint (one fixed-point frame, fixsum.cuh)
+  const double *X = g.bar + 4 * N, *Y = g.bar + 5 * N;
+  const double gv[13] = {g.bar[3 * N + node], X[pl.r + pl.xw], X[pl.r + pl.xe], below(Y, pl.x), above(Y, pl.x),
+                         below(X, pl.xw), below(Y, pl.xw), above(X, pl.xe), above(Y, pl.xe),
+                         above(X, pl.xw), above(Y, pl.xw), below(X, pl.xe), below(Y, pl.xe)};
+  double psi_b = fx::psi_adjoint_gather(gv);
+  if constexpr (ST) {
+    // transposes of t = (axis sum)/6 + (diagonal sum)/12 - psi(x), sd = (pE + pW) - (pN + pS),
+    // xd = (pNE + pSW) - (pNW + pSE) at the neighbours (the -psi(x) term is A1's)
+    const double *T = g.bar + 6 * N, *S = g.bar + 7 * N, *Q = g.bar + 8 * N;
+    const double sv[16] = {T[pl.r + pl.xe], T[pl.r + pl.xw], above(T, pl.x), below(T, pl.x),
+                           above(T, pl.xe), below(T, pl.xw), above(T, pl.xw), below(T, pl.xe),
+                           S[pl.r + pl.xe], S[pl.r + pl.xw], above(S, pl.x), below(S, pl.x),
+                           above(Q, pl.xe), below(Q, pl.xw), above(Q, pl.xw), below(Q, pl.xe)};
+    psi_b = fma(1.0 / 12.0, fx::surface_adjoint_gather(sv), psi_b);
   }
-  const int blk = blockIdx.y * gridDim.x + blockIdx.x;
-  double* dst = g.partial2 + (int64_t)blk * kA2;
-  // Block-uniform tests: a group of constants that no node of the block uses adds
-  // exact zeros, so its reductions are skipped.
-  const bool any_shaped = __syncthreads_or(shaped);
-  const bool any_vap = __syncthreads_or(vap_side);
-  const bool any_liq = __syncthreads_or(liq_side);
-  auto group = [&](int k0, int k1, bool used) {
-    for (int k = k0; k < k1; ++k) {
-      const int slot = k < G_ZZ ? k : k + 1;
-      const double s = used && ((g.slots >> slot) & 1u) ? block_sum(dcsum[k], red) : 0.0;
-      if (threadIdx.x == 0 && threadIdx.y == 0) dst[k] = g.accumulate ? dst[k] + s : s;
+  const double rho = a.mom[node];
+  const fx::u64 nb = fx::bits_of(rho), pb = fx::bits_of(a.psi[node]);
+  const EosConst& e = a.eos;
+  const long long rb = (long long)nb;
+  // the constants the node's branch uses: the shaped loop's, the vapour C-S's or the liquid's
+  const bool vap = rb <= e.bits_rho_v, liq = rb >= e.bits_rho_l;
+  const bool bulk_on = (g.slots & slot_bits(G_K1V, G_K4L)) != 0u;      // grid-uniform
+  const bool shape_on = (g.slots & slot_bits(G_PMAX, G_IA3)) != 0u;
+  const bool loop = e.mode == 1 && !vap && !liq;
+  // 1/(2 psi); psi > 0 (checked by the step)
+  const bool psi_ok = (fx::u32)(fx::hi32(pb) - 0x10000000u) < 0x60000000u;
+  const double half = psi_ok ? fx::half_reciprocal(pb) : 0.5 * fast_rcp(fx::double_of(pb));
+  double dpsi2;
+  // the loop's slots G_PMAX .. G_IA3 (with psi^2 = 2/G (p - rho/3))
+  double sh[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (loop) {
+    const bool first = rb <= e.bits_rho_max;
+    if (!first && rb < e.bits_rho_min) {
+      const double t = (rho - e.rho_max) * e.inv_span;
+      dpsi2 = fma(fma(3.0 * e.a2, t, 2.0 * e.b2) * t, e.inv_span * e.psi2_scale, e.k3);
+      sh[G_PMAX] = e.psi2_scale;
+      sh[G_A2] = e.psi2_scale * t * t * t;
+      sh[G_B2] = e.psi2_scale * t * t;
+    } else {
+      // s = sqrt(1 - d^2/a^2) and 1/s from one seed (see fast_sqrt)
+      const double d = rho - (first ? e.rho_max : e.rho_min);
+      const double z = fma(-d * d, first ? e.inv_a1sq : e.inv_a3sq, 1.0);
+      const double r = rsqrt_seed(z), zr = z * r;
+      const double er = fma(-zr, r, 1.0), c = fma(0.375, er, 0.5) * er;
+      const double q = (first ? g.q1 : g.q3) * d * fma(r, c, r);
+      dpsi2 = q + e.k3;
+      const double v1 = e.psi2_scale * (fma(zr, c, zr) - 1.0), v2 = (first ? g.h1 : g.h3) * d * q;
+      sh[first ? G_PMAX : G_PMIN] = e.psi2_scale;
+      sh[G_B1] = first ? v1 : 0.0;
+      sh[G_B3] = first ? 0.0 : -v1;
+      sh[G_IA1] = first ? v2 : 0.0;
+      sh[G_IA3] = first ? 0.0 : v2;
     }
-  };
-  group(a2_index(G_PMAX), a2_index(G_IA3) + 1, any_shaped);
-  group(a2_index(G_K1V), a2_index(G_K2V) + 1, any_vap);
-  group(a2_index(G_K1L), a2_index(G_K4L) + 1, any_liq);
+  } else if (!((fx::u32)(fx::hi32(nb) - 0x00100000u) < 0x7FE00000u && (e.mode != 2 || vap || liq) &&
+               fx::cs_slope_fixed(a.efix, a.efix.cs[e.mode == 1 && vap ? 0 : 1], fx::significand(nb), (int)(nb >> 52),
+                                  &dpsi2))) {
+    dpsi2 = slope_general(e, rho);
+  }
+  const double psi2_b = psi_b * half;  // psi = sqrt(psi^2)
+  const double rho_b = fma(psi2_b, dpsi2, g.bar[node]);
+  // lambda^t_i = rho_bar + c_i . j_bar (+ rows 7, 8 of Eq. MatrixMRT times the stress
+  // moments' adjoints with the two-phase set), exact in one frame (fixsum.cuh)
+  constexpr bool kShear = KIND == kShearTau;
+  double l[9];
+  fx::lambda_assembly<kShear>(rho_b, g.bar[N + node], g.bar[2 * N + node], kShear ? g.bar[9 * N + node] : 0.0,
+                              kShear ? g.bar[10 * N + node] : 0.0, l);
+  if (in) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) g.lam0[k * N + node] = l[k];
+  }
+  // a warp without a node on the loop adds nothing to its constants
+  const int w = warp_index(y), lane = threadIdx.x;
+  const double m = in ? psi2_b : 0.0;
+  if (shape_on && (__any_sync(~0u, in && loop) || !g.accumulate)) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sh[k] = loop && in ? sh[k] * m : 0.0;
+    const double v = warp_sum8(sh);
+    if ((lane & 3) == 0 && ((g.slots >> (lane >> 2)) & 1u)) add_partial(g, lane >> 2, w, v);
+  }
+  if (bulk_on) {
+    // K1V, K2V, K1L, K2L, K4L: psi^2 = rho (k1 Z + k2 rho + k3) + k4, Z of Eq. CS
+    const bool use_v = e.mode == 1 && vap, cs = in && !loop && (e.mode != 2 || vap || liq);
+    const double eta = e.b4 * rho, om = 1.0 - eta;
+    const double r = fast_rcp(om);
+    const double rz = rho * (fma(eta, fma(eta, om, 1.0), 1.0) * (r * r * r)) * m, rr = rho * rho * m;
+    double v8[8] = {cs && use_v ? rz : 0.0, cs && use_v ? rr : 0.0, cs && !use_v ? rz : 0.0,
+                    cs && !use_v ? rr : 0.0, cs && !use_v ? m : 0.0, 0.0, 0.0, 0.0};
+    const double v = warp_sum8(v8);
+    const int slot = G_K1V + (lane >> 2);
+    if ((lane & 3) == 0 && slot <= G_K4L && ((g.slots >> slot) & 1u)) add_partial(g, slot, w, v);
+  }
 }
 
-// grad[k] += sum over blocks, in a fixed order; one block per gradient slot
-__global__ void __launch_bounds__(256) k_adj_reduce(const double* partial1, const double* partial2, int nblocks,
-                                                    double* grad) {
-  __shared__ double red[256];
+// grad[k] += sum over the warps' partials, in a fixed order; one block per gradient slot
+constexpr int kReduceThreads = 1024;
+
+__global__ void __launch_bounds__(kReduceThreads) k_adj_reduce(const double* partial, int nw, unsigned slots, double* grad) {
+  __shared__ double red[kReduceThreads / 32];
   const int k = blockIdx.x;
+  if (!((slots >> k) & 1u)) return;
   double acc = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += 256)
-    acc += k == G_ZZ ? partial1[2 * b] : k == G_KAPPA ? partial1[2 * b + 1] : partial2[(int64_t)b * kA2 + a2_index(k)];
-  red[threadIdx.x] = acc;
+#pragma unroll 4
+  for (int w = threadIdx.x; w < nw; w += kReduceThreads) acc += partial[(int64_t)k * nw + w];
+  acc = warp_sum(acc);
+  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = acc;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    const double v = warp_sum(red[threadIdx.x]);
+    if (threadIdx.x == 0) grad[k] += v;
   }
-  if (threadIdx.x == 0) grad[k] += red[0];
 }
 
 // f_i = w_i rho0 is f^eq at rest; its transpose: rho0_bar = sum_i w_i lambda_i
@@ -676,7 +729,8 @@ __global__ void k_adj_init(int64_t n, const double* lam, double* rho_bar) {
   rho_bar[i] = s;
 }
 
-int nblocks(const StepArgs& a) { return ((a.nx + kTX - 1) / kTX) * ((a.ny + kTY - 1) / kTY); }
+// warps of the two passes: rows of 32 nodes
+int64_t warps_of(int nx, int ny) { return (int64_t)((nx + kTX - 1) / kTX) * ny; }
 
 }  // namespace
 }  // namespace pplbm
@@ -687,8 +741,7 @@ namespace {
 
 size_t adj_bytes(const pplbm_lattice* l) {
   const size_t n = (size_t)l->nx * l->ny;
-  const size_t nb = (size_t)((l->nx + kTX - 1) / kTX) * ((l->ny + kTY - 1) / kTY);
-  return sizeof(double) * (kPartialOffset * n + nb * kNGrad + 64);
+  return sizeof(double) * (kPartialOffset * n + (size_t)warps_of(l->nx, l->ny) * kNGrad + 64);
 }
 
 // one adjoint step given the forward arguments of step t whose psi and moment
@@ -700,12 +753,15 @@ pplbm_status adjoint_core(pplbm_ctx* c, const StepArgs& a, const double* lam1, d
   g.lam1 = lam1;
   g.lam0 = lam0;
   g.bar = ws;
-  const int nb = nblocks(a);
-  g.partial1 = ws + kPartialOffset * c->n;
-  g.partial2 = g.partial1 + 2 * nb;
+  g.partial = ws + kPartialOffset * c->n;
+  g.nw = (int)warps_of(a.nx, a.ny);
+  g.q1 = -a.eos.psi2_scale * a.eos.b1 * a.eos.inv_a1sq;
+  g.q3 = a.eos.psi2_scale * a.eos.b3 * a.eos.inv_a3sq;
+  g.h1 = 0.5 / a.eos.inv_a1sq;
+  g.h3 = 0.5 / a.eos.inv_a3sq;
   g.accumulate = accumulate ? 1 : 0;
   g.slots = c->adj_slots;
-  const dim3 grid((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY), block(kTX, kTY);
+  const dim3 grid = tile_grid((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY), block(kTX, kTY);
   const bool st = a.kappa_q != 0.0 || ((g.slots >> G_KAPPA) & 1u);  // with the source (kappa_q may be 0)
   if (a.kind == kShearTau) {
     if (st) {
@@ -722,7 +778,7 @@ pplbm_status adjoint_core(pplbm_ctx* c, const StepArgs& a, const double* lam1, d
     launch_dependent(k_adj_collide<kUnitTau, false>, grid, block, c->stream, g);
     launch_dependent(k_adj_rho_psi<kUnitTau, false>, grid, block, c->stream, g);
   }
-  if (reduce) k_adj_reduce<<<kNGrad, 256, 0, c->stream>>>(g.partial1, g.partial2, nb, grad);
+  if (reduce) k_adj_reduce<<<kNGrad, kReduceThreads, 0, c->stream>>>(g.partial, g.nw, g.slots, grad);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     c->msg = cudaGetErrorString(e);
@@ -814,10 +870,10 @@ pplbm_status pplbm_backward_checkpointed(pplbm_ctx* c, int64_t nsteps, int64_t i
     return PPLBM_ERR_CUDA;
   double* cur = lamA;
   double* nxt = lamB;
-  // per-block constant adjoints are summed over the whole rollout, then reduced once
-  const size_t nb = (size_t)nblocks(c->args);
+  // per-warp constant adjoints are summed over the whole rollout, then reduced once
+  const int nw = (int)warps_of(c->args.nx, c->args.ny);
   double* partials = ws + kPartialOffset * c->n;
-  if (cudaMemsetAsync(partials, 0, sizeof(double) * nb * kNGrad, s) != cudaSuccess) return PPLBM_ERR_CUDA;
+  if (cudaMemsetAsync(partials, 0, sizeof(double) * nw * kNGrad, s) != cudaSuccess) return PPLBM_ERR_CUDA;
   if (nsteps > 0) {
     const int64_t nseg = (nsteps + interval - 1) / interval;
     // With interval >= 4 the segment buffer (interval x 9 planes) holds two f
@@ -864,7 +920,7 @@ pplbm_status pplbm_backward_checkpointed(pplbm_ctx* c, int64_t nsteps, int64_t i
       }
     }
   }
-  k_adj_reduce<<<kNGrad, 256, 0, s>>>(partials, partials + 2 * nb, (int)nb, grad);
+  k_adj_reduce<<<kNGrad, kReduceThreads, 0, s>>>(partials, nw, c->adj_slots, grad);
   if (cudaGetLastError() != cudaSuccess) return PPLBM_ERR_CUDA;
   if (cudaMemcpyAsync(lambda_0, cur, sizeof(double) * stride, cudaMemcpyDefault, s) != cudaSuccess)
     return PPLBM_ERR_CUDA;
@@ -906,9 +962,9 @@ pplbm_status pplbm_backward_stored(pplbm_ctx* c, int64_t nsteps, const double* f
   cudaStream_t s = c->stream;
   if (cudaMemcpyAsync(cur, lambda_N, sizeof(double) * stride, cudaMemcpyDefault, s) != cudaSuccess)
     return PPLBM_ERR_CUDA;
-  const size_t nb = (size_t)nblocks(c->args);
+  const int nw = (int)warps_of(c->args.nx, c->args.ny);
   double* partials = ws + kPartialOffset * n;
-  if (cudaMemsetAsync(partials, 0, sizeof(double) * nb * kNGrad, s) != cudaSuccess) return PPLBM_ERR_CUDA;
+  if (cudaMemsetAsync(partials, 0, sizeof(double) * nw * kNGrad, s) != cudaSuccess) return PPLBM_ERR_CUDA;
   for (int64_t t = nsteps - 1; t >= 0; --t) {
     StepArgs a = c->args;
     a.psi = const_cast<double*>(fields) + t * field_planes(c) * n;
@@ -916,7 +972,7 @@ pplbm_status pplbm_backward_stored(pplbm_ctx* c, int64_t nsteps, const double* f
     if (pplbm_status st = adjoint_core(c, a, cur, nxt, grad, ws, true, false)) return st;
     std::swap(cur, nxt);
   }
-  k_adj_reduce<<<kNGrad, 256, 0, s>>>(partials, partials + 2 * nb, (int)nb, grad);
+  k_adj_reduce<<<kNGrad, kReduceThreads, 0, s>>>(partials, nw, c->adj_slots, grad);
   if (cudaGetLastError() != cudaSuccess) return PPLBM_ERR_CUDA;
   if (cudaMemcpyAsync(lambda_0, cur, sizeof(double) * stride, cudaMemcpyDefault, s) != cudaSuccess)
     return PPLBM_ERR_CUDA;

@@ -385,6 +385,27 @@ PPLBM_FX double psi_adjoint_gather(const double (&v)[13]) {
   return double_of(mx >= kFrameMaxHi ? kNaN : round_frame_s((i64)s, eg));
 }
 
+// The transposes of the surface-tension source's stencil sums, gathered: 12 times
+// (ta/6 + tg/12 + sd + xd) with ta the t adjoints of the axis neighbours (v[0..3]), tg of
+// the diagonal ones (v[4..7]), sd = (E + W) - (N + S) (v[8..11]) and xd = (NE + SW) - (NW +
+// SE) (v[12..15]), exact in one frame (coefficients summing to 108: headroom 8).
+PPLBM_FX double surface_adjoint_gather(const double (&v)[16]) {
+  u64 b[16];
+  unsigned mx = 0;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    b[k] = bits_of(v[k]);
+    mx = mx > mag_hi(b[k]) ? mx : mag_hi(b[k]);
+  }
+  const int eg = (int)(mx >> 20) + 8;
+  u64 t[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) t[k] = (u64)sterm(b[k], eg);
+  const u64 ta = (t[0] + t[1]) + (t[2] + t[3]), tg = (t[4] + t[5]) + (t[6] + t[7]);
+  const u64 sx = ((t[8] + t[9]) - (t[10] + t[11])) + ((t[12] + t[13]) - (t[14] + t[15]));
+  return double_of(mx >= kFrameMaxHi ? kNaN : round_frame_s((i64)(2 * ta + tg + 12 * sx), eg));
+}
+
 // The adjoint's lambda^t_i = rho_bar + c_i . j_bar (+ with SHEAR the rows 7, 8 of Eq.
 // MatrixMRT times the stress moments' adjoints m7_bar, m8_bar: +-1 on the axes,
 // +-1 on the diagonals), i = 1..8 (lambda_0 = rho_bar), exact in one frame
