@@ -2,9 +2,10 @@
 // kernels (step_kernels.cu) and the batched multi-lattice kernels (batch.cu) so
 // that both perform identical arithmetic.
 //
-// The GB300 FP64 pipe issues about 0.6e12 instructions/s, some 60x below FP32,
-// so these kernels are bound by FP64 issue rather than HBM: the arithmetic is
-// arranged to minimise FP64 instructions per node.
+// The GB300 FP64 pipe issues about 0.53e12 instructions/s, a 38th of the integer pipes, so
+// the per-node arithmetic runs on the integer pipes in fixed point (fixsum.cuh, fixmul.cuh,
+// eos_fixed.cuh, collide_fixed.cuh), bound by their issue rather than by HBM; the
+// double-precision forms below run the nodes that the frames cannot hold, and the fields.
 //  * K1 hands K2 the moments instead of the populations, so K2 never re-sums f.
 //  * With Lambda = I or with only the shear rates relaxing, f* is rebuilt
 //    directly as w_i [rho + 3 c.P + 4.5 (c c - I/3) : Pi] plus the sigma term of
@@ -14,8 +15,7 @@
 //    Li term needs no division by psi^2.
 //  * The optional surface-tension control (template flag ST) adds Li & Luo's
 //    source C to m*; in population space it joins the Li term's z and the rows
-//    7, 8 terms, so it costs about 15 FP64 instructions per node, and nothing when
-//    the flag is off.
+//    7, 8 terms, and costs nothing when the flag is off.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -154,51 +154,6 @@ __device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __
 __device__ __forceinline__ int wrap_index(int v, int n) {
   v %= n;
   return v < 0 ? v + n : v;
-}
-
-// v mod n for v in [-n, 2n) by one conditional add or subtract (no division); other
-// values (a lattice narrower than a tile) through the remainder
-__device__ __forceinline__ int wrap_near(int v, int n) {
-  v += v < 0 ? n : 0;
-  v -= v >= n ? n : 0;
-  return (v >= 0 && v < n) ? v : wrap_index(v, n);
-}
-
-// psi at lattice column gx (any integer: periodic wrap) and row gy in [-1, ny]
-// (periodic, or the wall ghost values beyond the walls)
-__device__ __forceinline__ double psi_wrapped(const StepArgs& a, int gx, int gy) {
-  gx = wrap_near(gx, a.nx);
-  if (a.walls) {
-    if (gy < 0) return a.psi_ghost_bottom;
-    if (gy >= a.ny) return a.psi_ghost_top;
-  } else {
-    gy = wrap_near(gy, a.ny);
-  }
-  return a.psi[(int64_t)gy * a.nx + gx];
-}
-
-// psi of the tile [x0 - 1, x0 + tw] x [y0 - 1, y0 + th] into sp (row stride tw + 2):
-// periodic wrap in x; periodic in y, or the wall ghost values beyond the walls. The
-// block has tw * th threads: thread (lx, ly) loads its own node, then the 2 (tw + 2)
-// + 2 th halo values are shared out, rows first (no division by the tile width).
-__device__ __forceinline__ void load_psi_tile(const StepArgs& a, double* sp, int x0, int y0, int tw, int th, int lx,
-                                              int ly, int tid, int nthreads) {
-  const int sw = tw + 2;
-  sp[(ly + 1) * sw + lx + 1] = psi_wrapped(a, x0 + lx, y0 + ly);
-  const int nh = 2 * sw + 2 * th;
-  for (int k = tid; k < nh; k += nthreads) {
-    int tx, ty;
-    if (k < 2 * sw) {
-      const bool top = k >= sw;
-      ty = top ? th + 1 : 0;
-      tx = top ? k - sw : k;
-    } else {
-      const int j = k - 2 * sw;
-      ty = 1 + (j >> 1);
-      tx = (j & 1) ? tw + 1 : 0;
-    }
-    sp[ty * sw + tx] = psi_wrapped(a, x0 + tx - 1, y0 + ty - 1);
-  }
 }
 
 struct Post {
