@@ -16,7 +16,8 @@ batch's stream, repeated until at least 1.5 s and 5 blocks have run (nvidia-smi
 samples the clocks meanwhile); `value` is from the median block, the max over
 ranks. Each pass's launches are bracketed by their own CUDA events inside the
 same blocks, which gives the dominant kernel's live launch duration for the
-roofline. Its peak is the FP64 issue rate measured here by pplbm_fp64_peak.
+roofline: integer instructions against the ALU pipe's rate, FP64 instructions against
+the issue rate measured here by pplbm_fp64_peak, whichever is closer.
 
 Also reported: the 2048 x 1024 droplet impact (walls, two-phase tau, T_r = 0.35,
 Re = 300) as a single lattice; per-plan times of the 64-lattice batch over 1,000
@@ -50,24 +51,18 @@ E2E_INNER = 100  # LBM steps per end-to-end call
 MIN_TIMED_S = 1.5
 MIN_BLOCKS = 5
 
-# FP64 instructions of one node update per kernel, from the kernels' arithmetic on
-# bulk nodes (unit relaxation times, Li forcing), counting what runs on the FP64 pipe:
-# the density pass 15 (the C-S branch 9 with v = 1/(1 - eta), sqrt 5; its moments are
-# integer sums in one fixed-point frame), the collision pass 19 (products, the
-# reciprocal and the Li term; its force stencil, the sums j + h, j + 2h, j + 3h and
-# the nine output populations are exact integer combinations in fixed-point frames).
-# These are the fallback; the roofline uses the counts ncu measured on the workload
-# (COUNTS).
-FP64_PER_NODE = {"rho_psi": 15, "collide": 19}
-# integer-pipe (ALU) instructions per node of the same passes (ncu; fallback figures)
-ALU_PER_NODE = {"rho_psi": 223, "collide": 1020}
+# FP64-pipe and integer-pipe (ALU) instructions per node of the two passes with unit
+# relaxation times on the headline workload (ncu, sm__inst_executed_pipe_fp64 / _alu x 32 per
+# node). The passes run in fixed point: the FP64 pipe only converts results (the moments; six
+# of the nine populations). These are the fallback for sources other than those of COUNTS.
+FP64_PER_NODE = {"rho_psi": 3.2, "collide": 6.8}
+ALU_PER_NODE = {"rho_psi": 241, "collide": 361}
 # ALU pipe issue rate: 64 thread instructions per SM per clock (ncu's
 # sm__pipe_alu_cycles_active scale: 82.7 % active at 16.6e12 instructions/s)
 ALU_PER_SM_CLK = 64
-# the two-phase relaxation (rows 7, 8 relax with 1/tau(rho)), walls: pass 1 adds the
-# two stress moments to its fixed-point frame, pass 2 tau(rho), its reciprocal and the
-# rows 7, 8 corrections (two more terms of its output frame)
-FP64_PER_NODE_SHEAR = {"rho_psi": 14.4, "collide": 32}  # ncu on the impact lattice: 14.42, 32.00
+# the two-phase relaxation (rows 7, 8 relax with 1/tau(rho)), walls (ncu on the impact lattice)
+FP64_PER_NODE_SHEAR = {"rho_psi": 5.0, "collide": 6.5}
+ALU_PER_NODE_SHEAR = {"rho_psi": 248, "collide": 444}
 # algorithmic bytes per node of each pass as built (moments handed from pass 1 to
 # pass 2): pass 1 reads 9 f and writes psi + 3 moments (5 with tau(rho)); pass 2
 # reads the moments and the psi tile and writes 9 f
@@ -78,29 +73,27 @@ BYTES_PER_NODE_SHEAR = {"rho_psi": 72 + 48, "collide": 40 + 8 + 72}
 BYTES_PER_NODE_SCOPE = 232
 # FP64-pipe and integer-pipe (ALU) instructions of one MacCormack step per grid point
 # (ncu, sm__inst_executed_pipe_fp64 / _alu x 32 per point, one kernel per capture, the
-# 2048 x 1024 grid of fd_throughput): predictor 54.0 / 1,947, corrector 60.0 / 1,963,
-# two EOS passes of 24.9 / 11; the update kernels' stencil differences are integer
-# combinations in fixed-point frames (at 3 blocks per SM: ALU 89 % / 86 %, FP64 79 % /
-# 84 % active)
-FD_FP64_PER_POINT = 54.0 + 60.0 + 2 * 24.9
-FD_ALU_PER_POINT = 1947 + 1963 + 2 * 11
+# 2048 x 1024 grid of fd_throughput): predictor 6.0 / 826, corrector 12.0 / 826, two EOS
+# passes of 1.0 / 154
+FD_FP64_PER_POINT = 6.0 + 12.0 + 2 * 1.0
+FD_ALU_PER_POINT = 826 + 826 + 2 * 154
 
 # Per launch of each batched pass on the headline workload (all 64 lattices), from
 # one ncu capture per kernel (--metrics dram__bytes_read.sum, dram__bytes_write.sum,
-# the thread-level DFMA/DADD/DMUL counts and sm__inst_executed_pipe_alu.sum;
+# sm__inst_executed_pipe_fp64.sum and sm__inst_executed_pipe_alu.sum;
 # bench.py --profile-sweep 64): DRAM bytes per launch, FP64 and ALU instructions per
 # node. They hold for the device code whose digest is recorded with them; once it
 # changes, traffic is null and the source counts above are used until the capture is
 # repeated.
-COUNTS = {"sources": "d5b0fa9fdc3eb98c",
-          "rho_psi": {"dram_bytes": 1316718336, "fp64_per_node": 14.542, "alu_per_node": 222.7},
-          "collide": {"dram_bytes": 1302610432, "fp64_per_node": 19.000, "alu_per_node": 1020.1},
+COUNTS = {"sources": "c2ec4fc6a7c6de15",
+          "rho_psi": {"dram_bytes": 1320026880, "fp64_per_node": 3.156, "alu_per_node": 240.8},
+          "collide": {"dram_bytes": 1334366208, "fp64_per_node": 6.780, "alu_per_node": 360.8},
           # the pipelined plan's mixed kernel: one launch runs the density pass of one
           # group and the collision pass of the other (half the nodes each); a step is
           # two launches
-          "mixed": {"dram_bytes": 1399193600}}
+          "mixed": {"dram_bytes": 1356397568}}
 KERNEL_SOURCES = ("batch_kernels.cuh", "step_device.cuh", "eos_dev.cuh", "eos.cuh", "fp64.cuh", "fixsum.cuh",
-                  "internal.h")
+                  "fixmul.cuh", "eos_fixed.cuh", "collide_fixed.cuh", "internal.h")
 
 
 def kernel_sources_digest():
@@ -128,8 +121,8 @@ def pass_traffic(name):
 def pass_fp64(name):
     """(FP64 instructions per node, where the figure comes from)."""
     if counts_valid():
-        return COUNTS[name]["fp64_per_node"], "ncu on this workload (thread-level DFMA + DADD + DMUL per node)"
-    return FP64_PER_NODE[name], "the kernel's arithmetic on bulk nodes"
+        return COUNTS[name]["fp64_per_node"], "ncu on this workload (FP64 pipe, per node)"
+    return FP64_PER_NODE[name], "ncu on an earlier build of this workload"
 
 
 def pass_alu(name):
@@ -382,7 +375,7 @@ def impact_2048(torch, stream, barrier, steps=1000):
         "built_bytes_per_node": sum(BYTES_PER_NODE_SHEAR.values()),
         "frac_built": sum(BYTES_PER_NODE_SHEAR.values()) * nodes / step_s / 1e9 / hbm_gbs,
         "peak": hbm_gbs, "unit": "GB/s", "peak_source": peak_src}
-    out["fp64_per_node"] = FP64_PER_NODE_SHEAR
+    out["fp64_per_node"], out["alu_per_node"] = FP64_PER_NODE_SHEAR, ALU_PER_NODE_SHEAR
     return out
 
 
@@ -570,7 +563,7 @@ def eos_variant_throughput(torch, steps=1000):
     return out
 
 
-def impact_sweep_throughput(torch, fp64_peak, steps=2000):
+def impact_sweep_throughput(torch, sm_mhz, steps=2000):
     """A slice of the stability study (Sec. IV.D) on the batched engine: droplet
     impact at Re = 300 on (600, 250) lattices with walls, C-S a = 0.363, Li forcing,
     two-phase tau(rho), T_r in {0.45, ..., 0.75} x v_r in {2, ..., 10}: 35 instances,
@@ -586,10 +579,10 @@ def impact_sweep_throughput(torch, fp64_peak, steps=2000):
     mlups = nodes * steps / (ms / 1e3) / 1e6 if stable == n_inst else None
     out = {"instances": n_inst, "stable": stable, "nodes": nodes, "steps": steps, "mlups": mlups, "plan": plan}
     if mlups is not None:
-        per = sum(FP64_PER_NODE_SHEAR.values())
-        achieved = per * mlups * 1e6
-        out["roofline"] = {"bound": "alu", "achieved": achieved / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
-                           "frac": achieved / 1e12 / fp64_peak, "fp64_per_node": per}
+        per = sum(ALU_PER_NODE_SHEAR.values())
+        achieved, peak = per * mlups * 1e6, ALU_PER_SM_CLK * 152 * sm_mhz * 1e6
+        out["roofline"] = {"bound": "alu", "pipe": "integer", "achieved": achieved / 1e12, "peak": peak / 1e12,
+                           "unit": "T integer instr/s", "frac": achieved / peak, "alu_per_node": per}
     return out
 
 
@@ -644,7 +637,7 @@ def fd_throughput(torch, fp64_peak, sm_mhz, steps=200):
     alu_peak = ALU_PER_SM_CLK * 152 * sm_mhz * 1e6
     return {"grid": f"{nx}x{ny}, dx=1, dt=0.4", "mlups": pts / 1e6,
             "ms_per_step": ms / steps, "finite": ok, "launches_per_step": 4,
-            "roofline": {"bound": "alu", "pipe": "integer (the update kernels' stencil sums)",
+            "roofline": {"bound": "alu", "pipe": "integer",
                          "achieved": alu / 1e12, "peak": alu_peak / 1e12, "unit": "T integer instr/s",
                          "frac": alu / alu_peak, "alu_per_point_step": FD_ALU_PER_POINT},
             "fp64_pipe": {"achieved": achieved / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
@@ -1027,7 +1020,7 @@ def main():
     alu_peak = ALU_PER_SM_CLK * 152 * mhz * 1e6 / 1e12
     fp64_pipe = {"pipe": "fp64", "kernel": dom_name, "achieved": achieved, "peak": fp64_peak,
                  "unit": "TFLOP/s", "frac": achieved / fp64_peak,
-                 "flop_convention": "1 per FP64 add/mul/fma instruction (per thread); "
+                 "flop_convention": "1 per FP64-pipe instruction (per thread); "
                                     f"{fp64_node.get(dom, sum(fp64_node.values()))} per node ({fp64_src})",
                  "peak_source": "measured: pplbm_fp64_peak in this run (fp64_peak_measured)"}
     alu_node = pass_alu(dom) if per_pass else sum(pass_alu(k) for k in ("rho_psi", "collide"))
@@ -1036,7 +1029,7 @@ def main():
                 "peak": alu_peak, "unit": "T integer instr/s",
                 "frac": alu_node * nodes / dom_s / 1e12 / alu_peak,
                 "peak_source": f"derived: 64 integer lanes per SM x 152 SMs x {mhz:.0f} MHz (sampled)",
-                "note": "the pass's sums run on the integer pipe (fixed-point frames and software IEEE adds)"}
+                "note": "the arithmetic runs in fixed point on the integer pipes"}
     if int_pipe["frac"] > fp64_pipe["frac"]:
         roof, other = dict(int_pipe), fp64_pipe
     else:
@@ -1118,7 +1111,7 @@ def main():
         line["adjoint"] = adjoint_cost(torch)
         line["eos_variants_mlups"] = eos_variant_throughput(torch)
         line["fd_solver"] = fd_throughput(torch, fp64_peak, clk.get("sm_mhz") or sm_max)
-        line["impact_sweep"] = impact_sweep_throughput(torch, fp64_peak)
+        line["impact_sweep"] = impact_sweep_throughput(torch, clk.get("sm_mhz") or sm_max)
     else:
         batch.close()
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:

@@ -389,8 +389,8 @@ typedef struct pplbm_batch pplbm_batch;
 #define PPLBM_PLAN_PIPELINED 3   /* the instances in two groups of about equal node counts, the
                                     second half a step behind the first within a call: every
                                     launch runs one group's density pass with the other's
-                                    collision pass (the FP64-bound and the integer-bound pass
-                                    share the SMs); 2 nsteps + 1 launches per call, two-step
+                                    collision pass (one's memory latency behind the other's
+                                    arithmetic); 2 nsteps + 1 launches per call, two-step
                                     CUDA graphs in between; every instance ends the call at the
                                     same step; each launch is a resident grid whose blocks take
                                     the work items in order from a device counter */
@@ -569,7 +569,7 @@ pplbm_status pplbm_fixsum_adjoint_eval(long long n, int32_t shear, const double*
 
 /* FP64 issue-rate probe, the denominator of the step's arithmetic roofline (the
  * step's per-node arithmetic is double precision throughout, Sec. II; on this GPU
- * the FP64 pipe, not memory, bounds it). Launches blocks_per_sm x (SM count)
+ * arithmetic issue, not memory, bounds it). Launches blocks_per_sm x (SM count)
  * blocks of 256 threads; each thread runs `iters` rounds of `chains` (1, 2, 4, 8,
  * 16 or 32) independent chains of one FP64 operation: op 0 fused multiply-add,
  * 1 add, 2 multiply; op 3 runs chains of the integer-pipe addition the step kernels
