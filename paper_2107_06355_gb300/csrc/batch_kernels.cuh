@@ -66,65 +66,71 @@ __device__ __forceinline__ void stage_args(const BatchInst* __restrict__ inst, i
   __syncthreads();
 }
 
-// density/psi pass over block `local` (256 nodes) of instance id; REUSE: the block
-// takes another item afterwards (persistent kernel), so it waits until every thread is
-// done with the shared arguments
-template <int KIND, bool REUSE>
-__device__ __forceinline__ void batch_rho_psi_local(const BatchInst* __restrict__ inst, int id, int local,
-                                                    int parity, StepArgs* sa) {
-  stage_args(inst, id, parity, sa);
-  const int i = local * kThreads + threadIdx.x;
-  if (i < (int)sa->n) rho_psi_node<KIND>(*sa, sa->f_in, i);
-  if (REUSE) __syncthreads();
-}
+// A work item is 256 nodes (or a tile of 256), shared by 256 / NT blocks of NT threads; block
+// `part` of them. LAUNCHED: one part per block of a dependent launch, which waits for its
+// predecessor after its arguments are in (no kernel writes them); otherwise the block takes
+// another item afterwards (persistent kernel), so it waits until every thread is done with
+// the shared arguments.
 
-template <int KIND, bool REUSE>
+// density/psi pass over item w
+template <int KIND, int NT, bool LAUNCHED>
 __device__ __forceinline__ void batch_rho_psi_item(const BatchInst* __restrict__ inst, const int* __restrict__ owner,
-                                                   int w, int parity, StepArgs* sa) {
-  const int id = owner[w];
-  batch_rho_psi_local<KIND, REUSE>(inst, id, w - inst[id].k1_start, parity, sa);
+                                                   int w, int part, int parity, StepArgs* sa) {
+  const int id = owner[w], local = w - inst[id].k1_start;
+  stage_args(inst, id, parity, sa);
+  if (LAUNCHED) begin_dependent();
+  const int i = local * kThreads + part * NT + threadIdx.x;
+  if (i < (int)sa->n) rho_psi_node<KIND>(*sa, sa->f_in, i);
+  if (!LAUNCHED) __syncthreads();
 }
 
-// collision pass over tile t of instance id; org: two shared ints for the tile
-// origin, which one thread computes per item; REUSE as for the density pass
-template <int KIND, bool ST, bool REUSE>
+// collision pass over item w; org: two shared ints for the tile origin, which one thread
+// computes per item
+template <int KIND, bool ST, int NT, bool LAUNCHED>
 __device__ __forceinline__ void batch_collide_item(const BatchInst* __restrict__ inst, const int* __restrict__ owner,
-                                                   int w, int parity, StepArgs* sa, int* org) {
+                                                   int w, int part, int parity, StepArgs* sa, int* org) {
   const int id = owner[w];
   const BatchInst& I = inst[id];
+  const int tw = I.tw, log2tw = I.log2tw;
   if (threadIdx.x == 0) {
     const int t = w - I.k2_start, tyi = t / I.tiles_x;
-    org[0] = (t - tyi * I.tiles_x) * I.tw;
+    org[0] = (t - tyi * I.tiles_x) * tw;
     org[1] = tyi * I.th;
   }
   stage_args(inst, id, parity, sa);  // ends with a barrier: org is visible
+  if (LAUNCHED) begin_dependent();
   const StepArgs& a = *sa;
-  const int x = org[0] + ((int)threadIdx.x & (I.tw - 1)), y = org[1] + ((int)threadIdx.x >> I.log2tw);
+  const int j = part * NT + (int)threadIdx.x;
+  const int x = org[0] + (j & (tw - 1)), y = org[1] + (j >> log2tw);
   if (x < a.nx && y < a.ny) collide_node<KIND, false, ST>(a, x, y, nullptr, nullptr, nullptr, nullptr);
-  if (REUSE) __syncthreads();
+  if (!LAUNCHED) __syncthreads();
 }
 
+// Blocks of the two passes' launches. us per step with 256 / 128 / 64 threads: 6 lattices of
+// 192^2 22.9 / 20.3 / 20.6 (with the source 26.6 / 22.8 / 22.7), 12 of 256^2 54.2 / 52.4 /
+// 53.6, 24 of 400^2 220 / 217 / 221, 35 two-phase 600 x 250 336 / 329 / 337: halves fill a
+// small batch's last wave, quarters copy their arguments too often.
+constexpr int kBlock = 128, kParts = kThreads / kBlock;
+
 template <int KIND>
-__global__ void __launch_bounds__(kThreads) k_batch_rho_psi(const BatchInst* inst, const int* owner, int parity) {
-  begin_dependent();
+__global__ void __launch_bounds__(kBlock) k_batch_rho_psi(const BatchInst* inst, const int* owner, int parity) {
   __shared__ StepArgs sa;
-  batch_rho_psi_item<KIND, false>(inst, owner, blockIdx.x, parity, &sa);
+  batch_rho_psi_item<KIND, kBlock, true>(inst, owner, blockIdx.x / kParts, blockIdx.x % kParts, parity, &sa);
 }
 
 // ST: some instance has the surface-tension source (kappa != 0); for the others
 // kappa_q = 0 makes the source exactly zero, so their results do not change
-// Unit relaxation times: 5 resident blocks per SM (at most 48 registers); the
+// Unit relaxation times: 40 resident warps per SM (at most 48 registers); the
 // integer-bound collision pass issues faster with the extra warps than it loses to
-// the 8-20 bytes of spilled registers. The other kinds keep 4 (they would spill more).
+// the 8-20 bytes of spilled registers. The other kinds keep 32 (they would spill more).
 constexpr int collide_min_blocks(int kind) { return kind == kUnitTau ? 5 : 4; }
 
 template <int KIND, bool ST>
-__global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
+__global__ void __launch_bounds__(kBlock, collide_min_blocks(KIND) * kParts)
     k_batch_collide(const BatchInst* inst, const int* owner, int parity) {
-  begin_dependent();
   __shared__ StepArgs sa;
   __shared__ int org[2];
-  batch_collide_item<KIND, ST, false>(inst, owner, blockIdx.x, parity, &sa, org);
+  batch_collide_item<KIND, ST, kBlock, true>(inst, owner, blockIdx.x / kParts, blockIdx.x % kParts, parity, &sa, org);
 }
 
 // ---- the pipelined plan's mixed kernel ----------------------------------------------
@@ -258,10 +264,10 @@ __global__ void __launch_bounds__(kThreads) k_batch_persistent(const BatchInst* 
   if ((int)blockIdx.x == absent_block) return;
   for (long long s = 0; s < nsteps; ++s) {
     const int parity = (int)((parity0 + s) & 1);
-    for (int w = blockIdx.x; w < n1; w += gridDim.x) batch_rho_psi_item<KIND, true>(inst, owner1, w, parity, &sa);
+    for (int w = blockIdx.x; w < n1; w += gridDim.x) batch_rho_psi_item<KIND, kThreads, false>(inst, owner1, w, 0, parity, &sa);
     if (!grid_barrier(bar, err, spin_limit)) return;
     for (int w = blockIdx.x; w < n2; w += gridDim.x)
-      batch_collide_item<KIND, ST, true>(inst, owner2, w, parity, &sa, org);
+      batch_collide_item<KIND, ST, kThreads, false>(inst, owner2, w, 0, parity, &sa, org);
     if (!grid_barrier(bar, err, spin_limit)) return;
   }
 }
@@ -353,16 +359,16 @@ void launch_pair_t(int kind, const BatchInst* inst, const int* o1, int n1, const
                    cudaStream_t s) {
   switch (kind) {
     case kUnitTau:
-      launch_dependent(k_batch_rho_psi<kUnitTau>, n1, kThreads, s, inst, o1, parity);
-      launch_dependent(k_batch_collide<kUnitTau, ST>, n2, kThreads, s, inst, o2, parity);
+      launch_dependent(k_batch_rho_psi<kUnitTau>, n1 * kParts, kBlock, s, inst, o1, parity);
+      launch_dependent(k_batch_collide<kUnitTau, ST>, n2 * kParts, kBlock, s, inst, o2, parity);
       break;
     case kShearTau:
-      launch_dependent(k_batch_rho_psi<kShearTau>, n1, kThreads, s, inst, o1, parity);
-      launch_dependent(k_batch_collide<kShearTau, ST>, n2, kThreads, s, inst, o2, parity);
+      launch_dependent(k_batch_rho_psi<kShearTau>, n1 * kParts, kBlock, s, inst, o1, parity);
+      launch_dependent(k_batch_collide<kShearTau, ST>, n2 * kParts, kBlock, s, inst, o2, parity);
       break;
     default:
-      launch_dependent(k_batch_rho_psi<kFullMrt>, n1, kThreads, s, inst, o1, parity);
-      launch_dependent(k_batch_collide<kFullMrt, ST>, n2, kThreads, s, inst, o2, parity);
+      launch_dependent(k_batch_rho_psi<kFullMrt>, n1 * kParts, kBlock, s, inst, o1, parity);
+      launch_dependent(k_batch_collide<kFullMrt, ST>, n2 * kParts, kBlock, s, inst, o2, parity);
       break;
   }
 }
@@ -402,9 +408,9 @@ void launch_collision_pass(int kind, bool st, const BatchInst* inst, const int* 
 #define PPLBM_K2(K)                                                                   \
   do {                                                                                \
     if (st)                                                                           \
-      launch_dependent(k_batch_collide<K, true>, n2, kThreads, s, inst, o2, parity); \
+      launch_dependent(k_batch_collide<K, true>, n2 * kParts, kBlock, s, inst, o2, parity); \
     else                                                                              \
-      launch_dependent(k_batch_collide<K, false>, n2, kThreads, s, inst, o2, parity); \
+      launch_dependent(k_batch_collide<K, false>, n2 * kParts, kBlock, s, inst, o2, parity); \
   } while (0)
   switch (kind) {
     case kUnitTau: PPLBM_K2(kUnitTau); break;
@@ -417,9 +423,9 @@ void launch_collision_pass(int kind, bool st, const BatchInst* inst, const int* 
 // the density/psi pass alone, over every instance (refreshes psi and the moments)
 void launch_density_pass(int kind, const BatchInst* inst, const int* o1, int n1, int parity, cudaStream_t s) {
   switch (kind) {
-    case kUnitTau: launch_dependent(k_batch_rho_psi<kUnitTau>, n1, kThreads, s, inst, o1, parity); break;
-    case kShearTau: launch_dependent(k_batch_rho_psi<kShearTau>, n1, kThreads, s, inst, o1, parity); break;
-    default: launch_dependent(k_batch_rho_psi<kFullMrt>, n1, kThreads, s, inst, o1, parity); break;
+    case kUnitTau: launch_dependent(k_batch_rho_psi<kUnitTau>, n1 * kParts, kBlock, s, inst, o1, parity); break;
+    case kShearTau: launch_dependent(k_batch_rho_psi<kShearTau>, n1 * kParts, kBlock, s, inst, o1, parity); break;
+    default: launch_dependent(k_batch_rho_psi<kFullMrt>, n1 * kParts, kBlock, s, inst, o1, parity); break;
   }
 }
 

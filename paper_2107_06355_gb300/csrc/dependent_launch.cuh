@@ -3,7 +3,7 @@
 //
 // The next kernel's blocks become resident while the previous one's last blocks run, so
 // its launch costs nothing on the critical path; each kernel waits for the launches before
-// it to complete before its first access to memory, which covers every hazard, and only
+// it to complete before its first access to memory that a kernel writes, and only
 // then lets its own successor start: with the two calls the other way round several
 // launches pile up on the SMs, and later ones find their places unevenly (33,700 nodes,
 // two-phase: 14.5 us per step against 10.0). Single lattice, us per step without / with:
@@ -23,7 +23,8 @@ inline dim3 tile_grid(int cols, int rows) {
 }
 __device__ __forceinline__ int tile_row() { return (int)(blockIdx.z * gridDim.y + blockIdx.y); }
 
-// at the start of a kernel launched by launch_dependent, before any memory access
+// at the start of a kernel launched by launch_dependent, before any access to memory that a
+// kernel writes
 __device__ __forceinline__ void begin_dependent() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
