@@ -617,7 +617,7 @@ pplbm_status pplbm_batch_create(pplbm_batch** out, int32_t n, const pplbm_lattic
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->persistent_grid = std::max(1, occ * sms);
   occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mixed_kernel(b->kind, b->st), kThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, mixed_kernel(b->kind, b->st), kBlock, 0);
   b->mixed_grid = std::max(1, occ * sms);
   int64_t most = 0, all = 0;
   for (int i = 0; i < n; ++i) {

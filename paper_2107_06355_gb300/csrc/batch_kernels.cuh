@@ -164,19 +164,20 @@ __device__ __forceinline__ void fetch_item_args(const BatchInst* __restrict__ in
   const unsigned long long* src =
       reinterpret_cast<const unsigned long long*>(&inst[id].a[is_collision_item(h) ? p2 : p1]);
   unsigned long long* d = reinterpret_cast<unsigned long long*>(dst);
-  for (int k = threadIdx.x; k < (int)(sizeof(StepArgs) / 8); k += kThreads) cp_async8(d + k, src + k);
+  for (int k = threadIdx.x; k < (int)(sizeof(StepArgs) / 8); k += kBlock) cp_async8(d + k, src + k);
 }
 
 // The item's pass from its staged arguments
 template <int KIND, bool ST>
-__device__ __forceinline__ void run_item(const StepArgs& a, const int4& h) {
+__device__ __forceinline__ void run_item(const StepArgs& a, const int4& h, int part) {
+  const int j = part * kBlock + (int)threadIdx.x;
   if (!is_collision_item(h)) {
-    const int i = h.y * kThreads + threadIdx.x;
+    const int i = h.y * kThreads + j;
     if (i < (int)a.n) rho_psi_node<KIND>(a, a.f_in, i);
     return;
   }
   const int log2tw = h.y, tw = 1 << log2tw;
-  const int lx = (int)threadIdx.x & (tw - 1), ly = (int)threadIdx.x >> log2tw;
+  const int lx = j & (tw - 1), ly = j >> log2tw;
   const int x = h.z + lx, y = h.w + ly;
   if (x < a.nx && y < a.ny) collide_node<KIND, false, ST>(a, x, y, nullptr, nullptr, nullptr, nullptr);
 }
@@ -184,19 +185,21 @@ __device__ __forceinline__ void run_item(const StepArgs& a, const int4& h) {
 // Work items of both passes in one launch (the pipelined plan): density items read
 // buffer p1, collision tiles p2. Lattices of one group run their density pass while
 // those of the other run their collision pass: both passes are bound by the integer pipe
-// (70 to 76 % busy run alone), and loads and stores of one overlap the other's arithmetic on
-// every SM. The grid is the resident block count G (at most n). Block b starts with item b;
-// later items come in table order from the queue counter queue[0] (item G + the
-// counter's old value), taken four items ahead: while a block computes item k it
-// copies in the arguments and headers of the next items (rings of 4), so that no item
-// waits on its set-up loads. The last block to finish resets queue[0]
-// and the finished-block count queue[1] for the next launch.
+// (60 % busy run alone), and loads and stores of one overlap the other's arithmetic on
+// every SM. The grid is the resident block count G (at most n, the number of parts: kParts
+// per item). Block b starts with part b; later parts come in table order from the queue
+// counter queue[0] (part G + the counter's old value), taken four ahead: while a block
+// computes part k it copies in the arguments and headers of the next ones (rings of 4), so
+// that no part waits on its set-up loads. The last block to finish resets queue[0] and the
+// finished-block count queue[1] for the next launch. ms per step on 12.9 M nodes with blocks
+// of 256 / 128 threads: 0.628 / 0.617; 35 two-phase 600 x 250 0.329 / 0.322.
 template <int KIND, bool ST>
-__global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
+__global__ void __launch_bounds__(kBlock, collide_min_blocks(KIND) * kParts)
     k_batch_mixed(const BatchInst* inst, const int4* items, int n, int p1, int p2, unsigned* queue) {
   __shared__ StepArgs sa[4];
   __shared__ int4 hdr[4];
-  __shared__ int qi[4];  // table index of the ring slot's item; -1: none
+  __shared__ int qi[4];    // the ring slot's part: table index times kParts plus part; -1: none
+  __shared__ int part[4];  // of the slot whose header is in hdr
   const int G = gridDim.x;
   if (threadIdx.x == 0) {
     const int t = G + (int)atomicAdd(&queue[0], 3u);
@@ -206,7 +209,10 @@ __global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
     qi[3] = t + 2 < n ? t + 2 : -1;
   }
   __syncthreads();
-  if (threadIdx.x < 3 && qi[threadIdx.x] >= 0) cp_async16(&hdr[threadIdx.x], items + qi[threadIdx.x]);
+  if (threadIdx.x < 3 && qi[threadIdx.x] >= 0) {
+    cp_async16(&hdr[threadIdx.x], items + qi[threadIdx.x] / kParts);
+    part[threadIdx.x] = qi[threadIdx.x] % kParts;
+  }
   cp_async_wait_all();
   __syncthreads();
   fetch_item_args(inst, hdr[0], p1, p2, &sa[0]);
@@ -221,11 +227,14 @@ __global__ void __launch_bounds__(kThreads, collide_min_blocks(KIND))
     if (qi[c2] >= 0) fetch_item_args(inst, hdr[c2], p1, p2, &sa[c2]);
     int next = -1;
     if (threadIdx.x == 0) {
-      if (qi[c3] >= 0) cp_async16(&hdr[c3], items + qi[c3]);
+      if (qi[c3] >= 0) {
+        cp_async16(&hdr[c3], items + qi[c3] / kParts);
+        part[c3] = qi[c3] % kParts;
+      }
       const int t = G + (int)atomicAdd(&queue[0], 1u);
       next = t < n ? t : -1;
     }
-    run_item<KIND, ST>(sa[c], hdr[c]);
+    run_item<KIND, ST>(sa[c], hdr[c], part[c]);
     if (threadIdx.x == 0) qi[c] = next;  // slot c now names item k + 4
     const bool more = qi[c1] >= 0;
     cp_async_wait_all();
@@ -386,13 +395,14 @@ void launch_pair(int kind, bool st, const BatchInst* inst, const int* o1, int n1
 void launch_mixed(int kind, bool st, const BatchInst* inst, const int4* items, int n, int grid, int p1, int p2,
                   unsigned* queue, cudaStream_t s) {
   if (n <= 0) return;
+  n *= kParts;
   grid = grid < n ? grid : n;
 #define PPLBM_KM(K)                                                                   \
   do {                                                                                \
     if (st)                                                                           \
-      k_batch_mixed<K, true><<<grid, kThreads, 0, s>>>(inst, items, n, p1, p2, queue);\
+      k_batch_mixed<K, true><<<grid, kBlock, 0, s>>>(inst, items, n, p1, p2, queue);\
     else                                                                              \
-      k_batch_mixed<K, false><<<grid, kThreads, 0, s>>>(inst, items, n, p1, p2, queue);\
+      k_batch_mixed<K, false><<<grid, kBlock, 0, s>>>(inst, items, n, p1, p2, queue);\
   } while (0)
   switch (kind) {
     case kUnitTau: PPLBM_KM(kUnitTau); break;
