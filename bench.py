@@ -56,7 +56,7 @@ MIN_BLOCKS = 5
 # node). The passes run in fixed point: the FP64 pipe only converts results (the moments; six
 # of the nine populations). These are the fallback for sources other than those of COUNTS.
 FP64_PER_NODE = {"rho_psi": 3.2, "collide": 6.8}
-ALU_PER_NODE = {"rho_psi": 241, "collide": 361}
+ALU_PER_NODE = {"rho_psi": 251, "collide": 372}
 # ALU pipe issue rate: 64 thread instructions per SM per clock (ncu's
 # sm__pipe_alu_cycles_active scale: 82.7 % active at 16.6e12 instructions/s)
 ALU_PER_SM_CLK = 64
@@ -85,13 +85,13 @@ FD_ALU_PER_POINT = 826 + 826 + 2 * 154
 # node. They hold for the device code whose digest is recorded with them; once it
 # changes, traffic is null and the source counts above are used until the capture is
 # repeated.
-COUNTS = {"sources": "c2ec4fc6a7c6de15",
-          "rho_psi": {"dram_bytes": 1320026880, "fp64_per_node": 3.156, "alu_per_node": 240.8},
-          "collide": {"dram_bytes": 1334366208, "fp64_per_node": 6.780, "alu_per_node": 360.8},
+COUNTS = {"sources": "c49d0d6a802c8ff8",
+          "rho_psi": {"dram_bytes": 1319949056, "fp64_per_node": 3.156, "alu_per_node": 250.8},
+          "collide": {"dram_bytes": 1335902976, "fp64_per_node": 6.780, "alu_per_node": 372.2},
           # the pipelined plan's mixed kernel: one launch runs the density pass of one
           # group and the collision pass of the other (half the nodes each); a step is
           # two launches
-          "mixed": {"dram_bytes": 1356397568}}
+          "mixed": {"dram_bytes": 1364653056}}
 KERNEL_SOURCES = ("batch_kernels.cuh", "step_device.cuh", "eos_dev.cuh", "eos.cuh", "fp64.cuh", "fixsum.cuh",
                   "fixmul.cuh", "eos_fixed.cuh", "collide_fixed.cuh", "internal.h")
 
