@@ -85,7 +85,7 @@ FD_ALU_PER_POINT = 826 + 826 + 2 * 154
 # node. They hold for the device code whose digest is recorded with them; once it
 # changes, traffic is null and the source counts above are used until the capture is
 # repeated.
-COUNTS = {"sources": "c49d0d6a802c8ff8",
+COUNTS = {"sources": "94e8be60002ff6fc",
           "rho_psi": {"dram_bytes": 1319949056, "fp64_per_node": 3.156, "alu_per_node": 250.8},
           "collide": {"dram_bytes": 1335902976, "fp64_per_node": 6.780, "alu_per_node": 372.2},
           # the pipelined plan's mixed kernel: one launch runs the density pass of one

@@ -1,9 +1,9 @@
 // Batched engine: many independent lattices (uneven sizes, their own EOS and
 // relaxation times, one collision kind) advanced together.
 //
-// Work is partitioned by blocks, not by instances: the density/psi pass runs one
-// 256-node block per work item; the collision pass runs one 256-thread tile per
-// work item, with a tile shape (tw x th, tw*th = 256) chosen per instance so that
+// Work is partitioned by items, not by instances: the density/psi pass has one item per 256
+// nodes, the collision pass one per tile of 256 nodes, with a tile shape (tw x th, tw*th =
+// 256) chosen per instance so that
 // narrow lattices (the 4-wide planar ones) do not leave threads idle. A
 // device-resident table maps each work item to its instance. Three ways to run a
 // step, chosen by the autotuner:

@@ -398,9 +398,9 @@ __device__ __forceinline__ Place place_of(const StepArgs& a, int x, int y) {
 }
 
 // psi at the node and its eight neighbours (C, E, W, N, S, NE, NW, SW, SE) by bit pattern,
-// wall ghosts beyond the walls. Loaded from global memory through L1: the nine values of a
-// 32 x 8 tile come from 34 x 10 distinct ones, and a shared-memory tile with its halo
-// arithmetic and barrier cost 150 instructions per node more than these loads.
+// wall ghosts beyond the walls. Loaded from global memory through L1, which neighbouring
+// nodes' stencils share: a shared-memory tile with its halo arithmetic and barrier cost 150
+// instructions per node more than these loads.
 __device__ __forceinline__ void load_psi(const StepArgs& a, const Place& p, fx::u64 (&v)[9]) {
   const unsigned long long* psi = reinterpret_cast<const unsigned long long*>(a.psi);
   v[0] = psi[p.r + p.x];
