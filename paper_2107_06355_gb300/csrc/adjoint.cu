@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kNT, KIND == kShearTau ? 8 : 10) k_adj_collide
   if (x < a.nx) {
     constexpr bool kShear = KIND == kShearTau;
     const Place pl = place_of(a, x, y);
-    const int N = (int)a.n, node = pl.r + x;
+    const int N = (int)a.n, node = pl.r + x;  // 9 n < 2^31
     fx::u64 psi[9];
     load_psi(a, pl, psi);
     double mu[9];
@@ -556,8 +556,8 @@ __global__ void __launch_bounds__(kNT, KIND == kShearTau ? 8 : 10) k_adj_collide
         B[8 * N + node] = xd_b;
       }
       if (kShear) {
-        B[9 * N + node] = o.m7_b;
-        B[10 * N + node] = o.m8_b;
+        B[(int64_t)9 * N + node] = o.m7_b;
+        B[(int64_t)10 * N + node] = o.m8_b;
       }
       zs_b = o.zs_b;
       B[node] = rb;
