@@ -14,8 +14,8 @@
 // tau_a omega^2.
 // A product of U and a velocity keeps it in U's units to 2 places, 2^-54 of the largest
 // mu; the stored lambda's own rounding is 2^-53. Reports a node outside the domain (that
-// of the forward, |u|, |h|, |K| below rho, mu outside the frames), for which the caller
-// runs the double-precision form. Against extended precision the gradient of 50 steps in the
+// of the forward, |u|, |h|, |K| below rho, the largest mu between 2^-300 and 2^400 or all
+// nine zero), for which the caller runs the double-precision form. Against extended precision the gradient of 50 steps in the
 // initial density has an rms error of 5.7e-15 of its rms (two-phase 6.2e-15); with rounded
 // double-precision stages it had 8.1e-15 (9.4e-15).
 //
@@ -87,7 +87,14 @@ PPLBM_FX bool collide_reverse_fixed(const CollideFix& k, const u64 (&psi)[9], do
 #pragma unroll
   for (int i = 1; i < 9; i += 2) mm = max3(mm, mag_hi(b[i]), mag_hi(b[i + 1]));
   ok = ok && mm < (1423u << 20);
-  const int el = ((int)(mm >> 20) > 723 ? (int)(mm >> 20) : 723) + 10;  // below 2^-300 they count as zero
+  if (mm < (723u << 20)) {
+    // below 2^-300 the double-precision form keeps what this frame would drop; all zeros are exact
+    u64 any = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) any |= b[i] << 1;
+    ok = ok && any == 0;
+  }
+  const int el = ((int)(mm >> 20) > 723 ? (int)(mm >> 20) : 723) + 10;
   i64 t[9];
 #pragma unroll
   for (int i = 0; i < 9; ++i) t[i] = with_sign(shr_u(significand(b[i]), el - (int)(mag_hi(b[i]) >> 20)), b[i]);

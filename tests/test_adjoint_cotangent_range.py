@@ -1,0 +1,70 @@
+"""The reverse pass over the whole range of cotangents: a loss scaled by a power of two gives
+the gradient scaled by it. Host build of csrc/adjoint_fixed.cuh (rows that it accepts are
+bitwise the scaled rows, the others are reported), and rollouts on the GPU."""
+import numpy as np
+import pytest
+
+import lbm_inputs as I
+from test_adjoint_fixed_host import af, nodes, reverse  # noqa: F401
+
+
+@pytest.mark.parametrize("shear", [0, 1])
+def test_scaled_cotangents(af, shear):  # noqa: F811
+    """Every value is linear in mu, and a power of two only shifts the frame: bitwise."""
+    rows = nodes(np.random.default_rng(5), 40, -3, -0.5, 0.1, 0.1, 0.5)
+    rows[:, 14:] *= 2.0 ** -np.floor(np.log2(np.abs(rows[:, 14:]).max(axis=1, keepdims=True)))  # largest in [1, 2)
+    want, ok = reverse(af, rows, shear, (0.6, 0.0))
+    assert ok.all()
+    linear = [0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11]
+    for k in (-300, -100, 100, 250, 300, 301, 310, 340, 360, 400, 700, 1000, 1030, 1060):
+        r = rows.copy()
+        r[:, 14:] = np.ldexp(r[:, 14:], -k)
+        got, acc = reverse(af, r, shear, (0.6, 0.0))
+        assert np.array_equal(acc, np.full(len(rows), k <= 300)), k
+        if k <= 300:
+            assert np.array_equal(got[:, linear], np.ldexp(want[:, linear], -k)), k
+
+
+@pytest.mark.parametrize("shear", [0, 1])
+def test_zero_cotangents_are_inside(af, shear):  # noqa: F811
+    rows = nodes(np.random.default_rng(6), 3, -1, -1, 0.05, 0.05, 0.5)
+    rows[:, 14:] = 0.0
+    rows[1, 14:18] = -0.0
+    rows[2, 20] = 5e-324
+    got, acc = reverse(af, rows, shear, (0.6, 0.0))
+    assert acc.tolist() == [True, True, False]
+    assert not got[:2, :12].any()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("relax, kappa", [(dict(), 0.0), (dict(), 0.3), (dict(kind=1, tau_l=0.6, visc_ratio=3.0), 0.0),
+                                          (dict(kind=1, tau_l=0.6, visc_ratio=3.0), 0.3)])
+@pytest.mark.parametrize("k", [250, 310, 400])
+def test_scaled_loss(relax, kappa, k):
+    """20 steps on 40 x 36: the nodes outside the frames take the double-precision form, which
+    agrees with the fixed-point one to a few hundred roundings of 2^-53 of the largest lambda,
+    amplified by 1/rho_v on vapour nodes (1e-12 in the tests of one step): 1e-10 of the
+    largest value over 20 steps. dL/dalpha is a sum over the nodes with random weights: 1e-10
+    of its terms, four digits left for what they cancel."""
+    torch = pytest.importorskip("torch")
+    import paper_2107_06355_gb300 as P
+    from paper_2107_06355_gb300 import adjoint as A
+
+    eos = P.EOSParams(P.EOS_SMOOTH, 0.5, 0.363, 2.0, 0.775)
+    d = P.eos_setup(eos)
+    nx, ny = 40, 36
+    rho = torch.tensor(I.perturbed(I.planar(nx, ny, d["rho_v"], d["rho_l"], W=8.0), 1e-3, 2), device="cuda")
+    spec = A.RolloutSpec(nx, ny, P.BC_PERIODIC, eos, P.Relax(kappa=kappa, **relax), nsteps=20)
+    w = torch.tensor(np.random.default_rng(3).standard_normal((ny, nx)), device="cuda")
+
+    def gradient(scale):
+        x = rho.clone().requires_grad_(True)
+        t = torch.tensor(0.775, dtype=torch.float64, requires_grad=True)
+        (A.rollout(x, t, spec) * (w * scale)).sum().backward()
+        return x.grad, float(t.grad)
+
+    g0, a0 = gradient(1.0)
+    g1, a1 = gradient(2.0 ** -k)
+    assert bool(torch.isfinite(g0).all()) and float(g0.abs().max()) > 0.0
+    assert float((g1 * 2.0 ** k - g0).abs().max()) < 1e-10 * float(g0.abs().max())
+    assert abs(a1 * 2.0 ** k - a0) < 1e-6 * abs(a0)
