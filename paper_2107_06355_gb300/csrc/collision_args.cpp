@@ -51,10 +51,15 @@ static int64_t fixed(long double x, int k, int bits, int* ok) {
 }
 
 // A branch psi^2 2^-s = k3 rho + A + B g((rho - rho0) / a), rho up to rho_top: an ellipse
-// (|rho - rho0| <= a) or the cubic (a its span)
+// (|rho - rho0| <= a) or the cubic (a its span). *ok is cleared when a is not positive and
+// finite: a block that no set-up made.
 static LoopFix loop_branch(bool ellipse, long double rho_top, long double rho0, long double a, long double A,
                            long double B, int* ok) {
   LoopFix L{};
+  if (!(a > 0.0L) || !std::isfinite(a) || !std::isfinite(rho_top)) {
+    *ok = 0;
+    return L;
+  }
   int e;
   std::frexp(ellipse ? std::fmax(rho_top, 2.0L * a) : rho_top, &e);  // < 2^e
   L.q = (ellipse ? 63 : 62) - e;
@@ -62,7 +67,7 @@ static LoopFix loop_branch(bool ellipse, long double rho_top, long double rho0, 
     L.c = fixed(a, L.q, 62, ok);
     B = B / a * std::ldexp(1.0L, 62 - L.q);
   } else {
-    while (std::ldexp(1.0L / a, 126 - L.up - L.q) >= 0x1.8p62L) ++L.up;
+    while (L.up <= 12 && std::ldexp(1.0L / a, 126 - L.up - L.q) >= 0x1.8p62L) ++L.up;
     if (L.up > 12) *ok = 0;  // the span is far below a frame this coarse
     L.c = fixed(1.0L / a, 126 - L.up - L.q, 63, ok);
   }
