@@ -97,9 +97,9 @@ struct FDEosArgs {
 // psi and p of one density: in fixed point on the integer pipes (eos_fixed.cuh), p from
 // psi^2 before its root; a density outside that domain in double precision. In double
 // precision throughout (25 FP64 instructions per point) the pass was bound by the FP64
-// pipe.
-__global__ void __launch_bounds__(128) k_fd_eos(const __grid_constant__ FDEosArgs a, const double* __restrict__ rho,
-                                                double* __restrict__ psi, double* __restrict__ p, int64_t n) {
+// pipe. (Plain pointers: the blocks are resident while the previous launch still writes rho.)
+__global__ void __launch_bounds__(128) k_fd_eos(const __grid_constant__ FDEosArgs a, const double* rho, double* psi,
+                                                double* p, int64_t n) {
   using namespace fx;
   begin_dependent();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;

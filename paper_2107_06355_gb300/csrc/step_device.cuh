@@ -31,7 +31,7 @@ namespace pplbm {
 // Sec. III.D, InteractionPotential); error word on a non-finite or non-positive density or
 // psi^2. Runs for the nodes outside the fixed-point path's domain.
 template <int KIND>
-__device__ __forceinline__ void rho_psi_double(const StepArgs& a, const double* __restrict__ f, int i) {
+__device__ __forceinline__ void rho_psi_double(const StepArgs& a, const double* f, int i) {
   const int N = (int)a.n;  // 9 n < 2^31: plane offsets fit 32 bits
   const double f0 = f[i], f1 = f[N + i], f2 = f[2 * N + i], f3 = f[3 * N + i], f4 = f[4 * N + i];
   const double f5 = f[5 * N + i], f6 = f[6 * N + i], f7 = f[7 * N + i], f8 = f[8 * N + i];
@@ -84,7 +84,7 @@ __device__ __forceinline__ void rho_psi_double(const StepArgs& a, const double* 
 }
 
 template <int KIND>
-__device__ __noinline__ void rho_psi_general(const StepArgs& a, const double* __restrict__ f, int i) {
+__device__ __noinline__ void rho_psi_general(const StepArgs& a, const double* f, int i) {
   rho_psi_double<KIND>(a, f, i);
 }
 
@@ -99,8 +99,9 @@ __device__ __noinline__ void rho_psi_general(const StepArgs& a, const double* __
 // node) that pipe was 85 % busy and the pass took 107 us; over a batch of 12.9 M nodes
 // 0.444 ms before, 0.282 ms now. The rms error of psi is 0.30 ulp on every branch (0.58
 // next to the vapour at T_r = 0.35), where double precision gave 0.4 to 1.0 (22).
+// (f is a plain pointer: the kernels that run several steps write it themselves.)
 template <int KIND>
-__device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* __restrict__ f, int i) {
+__device__ __forceinline__ void rho_psi_node(const StepArgs& a, const double* f, int i) {
   using namespace fx;
   const int N = (int)a.n;
   u64 b[9];
