@@ -86,14 +86,9 @@ PPLBM_FX bool collide_reverse_fixed(const CollideFix& k, const u64 (&psi)[9], do
   u32 mm = mag_hi(b[0]);
 #pragma unroll
   for (int i = 1; i < 9; i += 2) mm = max3(mm, mag_hi(b[i]), mag_hi(b[i + 1]));
-  ok = ok && mm < (1423u << 20);
-  if (mm < (723u << 20)) {
-    // below 2^-300 the double-precision form keeps what this frame would drop; all zeros are exact
-    u64 any = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) any |= b[i] << 1;
-    ok = ok && any == 0;
-  }
+  // below 2^-300 the double-precision form keeps what this frame would drop (subnormals under
+  // 2^-1042, whose upper words are zero, count as zero)
+  ok = ok && mm < (1423u << 20) && mm - 1u >= (723u << 20) - 1u;
   const int el = ((int)(mm >> 20) > 723 ? (int)(mm >> 20) : 723) + 10;
   i64 t[9];
 #pragma unroll

@@ -16,7 +16,7 @@ def test_scaled_cotangents(af, shear):  # noqa: F811
     want, ok = reverse(af, rows, shear, (0.6, 0.0))
     assert ok.all()
     linear = [0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11]
-    for k in (-300, -100, 100, 250, 300, 301, 310, 340, 360, 400, 700, 1000, 1030, 1060):
+    for k in (-300, -100, 100, 250, 300, 301, 310, 340, 360, 400, 700, 1000, 1030, 1040):
         r = rows.copy()
         r[:, 14:] = np.ldexp(r[:, 14:], -k)
         got, acc = reverse(af, r, shear, (0.6, 0.0))
@@ -30,7 +30,7 @@ def test_zero_cotangents_are_inside(af, shear):  # noqa: F811
     rows = nodes(np.random.default_rng(6), 3, -1, -1, 0.05, 0.05, 0.5)
     rows[:, 14:] = 0.0
     rows[1, 14:18] = -0.0
-    rows[2, 20] = 5e-324
+    rows[2, 20] = 1e-310
     got, acc = reverse(af, rows, shear, (0.6, 0.0))
     assert acc.tolist() == [True, True, False]
     assert not got[:2, :12].any()
