@@ -67,7 +67,8 @@ inline cudaLaunchConfig_t cluster_config(int lattices, ClusterShape shape, cudaL
 
 // One thread per node: 128 threads per block up to 2,048 nodes and 256 above, in a power of
 // two of blocks; {0, 0} (the step kernels) for lattices of more than `limit` nodes, for more
-// than 65,536 in all, or where the device cannot hold such a cluster.
+// than 65,536 in all, where the device cannot hold such a cluster, or too few of them at a time
+// (clusters_pay).
 // The lines, us per step, clusters / two launches: one lattice of 256 to 2,048 nodes 6.7 / 7.9
 // (two-phase 7.7 / 9.0, with the source 8.5 / 9.5, six rates 9.4 / 10.5), of 3,072 or 4,096
 // 8.5 / 7.9 (10.1 / 9.0, 11.6 / 9.5, 14.8 / 10.5), so 2,048 (kClusterNodes). The batched
@@ -88,7 +89,7 @@ inline ClusterShape cluster_shape(const void* kernel, int limit, int64_t max_nod
   const cudaLaunchConfig_t cfg = cluster_config(lattices, shape, at, nullptr);
   int fit = 0;
   if (cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) != cudaSuccess) cudaGetLastError();
-  return fit > 0 ? shape : ClusterShape{0, 0};
+  return clusters_pay(shape.blocks, lattices, fit) ? shape : ClusterShape{0, 0};
 }
 
 // launches `lattices` clusters of the given shape

@@ -74,6 +74,20 @@ struct ClusterShape {
   int blocks, threads;
 };
 constexpr int kClusterSteps = 1000;
+// Whether `lattices` clusters of `blocks` blocks, `fit` of which the device holds at a time, are
+// to run rather than the step kernels. A cluster runs a whole call's steps, so clusters beyond
+// those resident double the time, triple it and so on, and all have the blocks of the largest
+// lattice, most of them idle beside one that is much larger than the rest. us per step, step
+// kernels / clusters: 1,024 lattices of 16 nodes (1 block, 912 resident) 9.9 / 6.4 and 4,096 of
+// them 27 / 16; of 60 nodes each beside one of 512 (4 blocks, 222) 200: 7.4 / 7.0, 400: 8.5 /
+// 8.3, 800: 10.5 / 15.5; beside one of 2,048 (16 blocks, 47) 64: 6.4 / 7.7, 400: 8.6 / 34;
+// beside one of 4,096 (21) 32: 5.8 / 7.7, 400: 9.2 / 68; 16 two-phase lattices of 4,096 with
+// the source (14) 8.0 / 10.8. So any number of single blocks, two rounds of up to 8 blocks,
+// and one of 16.
+inline bool clusters_pay(int blocks, int lattices, int fit) {
+  if (fit <= 0) return false;
+  return blocks == 1 || lattices <= (int64_t)fit * (blocks <= 8 ? 2 : 1);
+}
 ClusterShape small_lattice_shape(const StepArgs& a);
 void launch_cluster_steps(const StepArgs& a, ClusterShape shape, int nsteps, void* stream);
 void launch_fields(const StepArgs& a, double* rho, double* ux, double* uy, double* psi_out, void* stream);
