@@ -3,8 +3,10 @@
 //
 // The nine adjoints mu_i of the populations become integers in one frame (units of
 // 2^(el - 1086), headroom 10: every sum below stays under 2^63 with velocities under
-// 0.875), so the adjoints U of the populations' inputs (reduced_populations_transpose) are
-// exact. Scaled by rho every factor between them and the adjoints of rho, j and h is a velocity, kept as u 2^63: with s = 1/36,
+// 0.875) with two places more, so the adjoints U of the populations' inputs
+// (reduced_populations_transpose) are exact up to mu's rounding and are rounded once. Scaled
+// by rho every factor between them and the adjoints of rho, j and h is a velocity, kept as
+// u 2^63: with s = 1/36,
 //   36 J_b  = U3 p_y + U1 q_x, U3 h_x + U2 q_y      (p = P/rho, q = Q/rho, h = F/(2 rho))
 //   36 j_b  = J_b + U4 + U1 u_x, J_b + U5 + U3 u_x + U2 u_y
 //   36 rho_b = U0 - J_b . u,  36 h_b = J_b + 2 P_b + 3 Q_b (+ U3 u_y),
@@ -13,11 +15,15 @@
 // 36 rho_b += (U7 A7 + U8 A8)/rho (omega - tau_a omega^2), as -rho d omega/d rho = omega -
 // tau_a omega^2.
 // A product of U and a velocity keeps it in U's units to 2 places, 2^-54 of the largest
-// mu; the stored lambda's own rounding is 2^-53. Reports a node outside the domain (that
-// of the forward, |u|, |h|, |K| below rho, the largest mu between 2^-300 and 2^400 or all
-// nine zero), for which the caller runs the double-precision form. Against extended precision the gradient of 50 steps in the
-// initial density has an rms error of 5.7e-15 of its rms (two-phase 6.2e-15); with rounded
-// double-precision stages it had 8.1e-15 (9.4e-15).
+// mu; the stored lambda's own rounding is 2^-53. mu itself needs an unbiased rounding: over a
+// long rollout lambda's c . j_b grows beyond rho_b, and mu cut off towards zero at 2^-53 of the
+// largest shrank rho_b: the gradient of 400 steps in the initial density had an rms error of
+// 2.9e-13 of its rms against extended precision (two-phase 2.4e-13), 1.7e-14 (1.2e-14) so, and
+// 4.3e-14 with rounded double-precision stages; of 100 steps 1.4e-14, 3.0e-15 and 1.0e-14. It costs
+// 3 % of a gradient's step on 1024^2.
+// Reports a node outside the domain (that of the forward, |u|, |h|, |K| below rho, the largest
+// mu between 2^-300 and 2^400 or all nine zero), for which the caller runs the double-precision
+// form.
 //
 // Compiles for the host too.
 #pragma once
@@ -90,16 +96,23 @@ PPLBM_FX bool collide_reverse_fixed(const CollideFix& k, const u64 (&psi)[9], do
   // 2^-1042, whose upper words are zero, count as zero)
   ok = ok && mm < (1423u << 20) && mm - 1u >= (723u << 20) - 1u;
   const int el = ((int)(mm >> 20) > 723 ? (int)(mm >> 20) : 723) + 10;
+  // mu and the sums of them carry two places more (72 2^56 < 2^63); what joins products is
+  // rounded to whole units. mu is rounded to nearest, ties to even: half of the ties are
+  // exact halves of doubles a few octaves below the largest (rho_b beside a large j_b)
   i64 t[9];
 #pragma unroll
-  for (int i = 0; i < 9; ++i) t[i] = with_sign(shr_u(significand(b[i]), el - (int)(mag_hi(b[i]) >> 20)), b[i]);
+  for (int i = 0; i < 9; ++i) {
+    const u64 m = shr_u(significand(b[i]), el - 4 - (int)(mag_hi(b[i]) >> 20));
+    t[i] = with_sign((m + 1 + ((m >> 2) & 1ull)) >> 2, b[i]);
+  }
+  auto whole = [](i64 n) { return (n + 2) >> 2; };
   const i64 a13 = t[1] + t[3], a24 = t[2] + t[4], s57 = t[5] + t[7], s68 = t[6] + t[8];
   const i64 d57 = t[5] - t[7], d68 = t[6] - t[8], dg = s57 + s68;
-  const i64 U0 = 16 * t[0] + 4 * (a13 + a24) + dg;
-  const i64 U1 = 3 * dg - 24 * t[0] + 12 * a13 - 6 * a24, U2 = 3 * dg - 24 * t[0] - 6 * a13 + 12 * a24;
-  const i64 U3 = 9 * (s57 - s68);
-  const i64 U4 = 12 * (t[1] - t[3]) + 3 * (d57 - d68), U5 = 12 * (t[2] - t[4]) + 3 * (d57 + d68);
-  const i64 U6 = a13 + a24 + dg - 8 * t[0], U7 = 9 * (a13 - a24);
+  const i64 U0 = 16 * t[0] + 4 * (a13 + a24) + dg;  // with its two places
+  const i64 U1 = whole(3 * dg - 24 * t[0] + 12 * a13 - 6 * a24), U2 = whole(3 * dg - 24 * t[0] - 6 * a13 + 12 * a24);
+  const i64 U3 = whole(9 * (s57 - s68));
+  const i64 U4 = whole(12 * (t[1] - t[3]) + 3 * (d57 - d68)), U5 = whole(12 * (t[2] - t[4]) + 3 * (d57 + d68));
+  const i64 U6 = whole(a13 + a24 + dg - 8 * t[0]), U7 = whole(9 * (a13 - a24));
   // products with a velocity are in units of 2: doubled where they join whole ones
   const Factor f1 = factor(U1), f2 = factor(U2), f3 = factor(U3);
   i64 Jxb = 2 * (mulhi(f3, fpy) + mulhi(f1, fqx)), Jyb = 2 * (mulhi(f3, fvx) + mulhi(f2, fqy));
@@ -107,8 +120,8 @@ PPLBM_FX bool collide_reverse_fixed(const CollideFix& k, const u64 (&psi)[9], do
   const i64 Pxb = U4, Pyb = U5 + 2 * mulhi(f3, fux);
   i64 hx0 = 2 * mulhi(f3, fuy), hy0 = 0, jy0 = 0, Kxb = 0, Kyb = 0, rb0 = 0;
   const int kl = el - 1086;
-  // n / 36 in units of 2^(kl - 4): times 16/36
-  auto over36 = [&](i64 n) { return frame_to_double(mulhi(factor(n), factor((i64)kFourNinths)), kl - 4); };
+  // n / 36 in units of 2^(k - 4): times 16/36
+  auto over36 = [&](i64 n, int k) { return frame_to_double(mulhi(factor(n), factor((i64)kFourNinths)), k - 4); };
   if (SHEAR) {
     const i64 w = one_minus_omega(k, L, er, &ok);
     ok = ok && in_range(w, 0x40000000u);
@@ -137,17 +150,18 @@ PPLBM_FX bool collide_reverse_fixed(const CollideFix& k, const u64 (&psi)[9], do
     Kyb = 2 * mulhi(g7, fuy);
     jy0 = -2 * mulhi(g8, fux);
     hx0 += 2 * mulhi(g8, fuy);
-    o->m7_b = over36(B7);
-    o->m8_b = over36(B8);
+    o->m7_b = over36(B7, kl);
+    o->m8_b = over36(B8, kl);
     if (SRC) o->om = frame_to_double(om, -61);
   }
   // 36 times the adjoints of rho, j, h
-  const i64 Rb = U0 - 2 * (mulhi(factor(Jxb), fux) + mulhi(factor(Jyb), fuy)) + rb0;
+  const i64 Ru = rb0 - 2 * (mulhi(factor(Jxb), fux) + mulhi(factor(Jyb), fuy));
+  ok = ok && in_range(Ru, 0x10000000u);  // with U0 < 36 2^56 below 2^63
   const i64 Xb = Jxb + Pxb + Qxb + Kxb, Yb = Jyb + Pyb + Qyb + Kyb + jy0;
   const i64 Hx = hx0 + Jxb + 2 * Pxb + 3 * Qxb - Kxb, Hy = hy0 + Jyb + 2 * Pyb + 3 * Qyb - Kyb;
-  o->rho_b = over36(Rb);
-  o->jx_b = over36(Xb);
-  o->jy_b = over36(Yb);
+  o->rho_b = over36(U0 + 4 * Ru, kl - 2);
+  o->jx_b = over36(Xb, kl);
+  o->jy_b = over36(Yb, kl);
   // through h = cH g: gx_b = cH/36 Hx + 2 zs U6 gx, psi_b = (hf/36) (Hx gx + Hy gy)
   const Factor fHx = factor(Hx), fHy = factor(Hy);
   const int n6 = spare_bits(U6);
