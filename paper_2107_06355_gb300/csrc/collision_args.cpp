@@ -26,7 +26,8 @@ int collision_kind(const pplbm_relax* r) {
 
 fx::FixNum fixnum(double x, int div) {
   fx::FixNum r{0, -4096, 0};
-  if (x == 0.0 || !std::isfinite(x)) return r;
+  if (x == 0.0) return r;
+  if (!std::isfinite(x)) return fx::FixNum{1ll << 62, 4096, 0};
   int e;
   const int64_t s = (int64_t)std::ldexp(std::frexp(std::fabs(x), &e), 53);  // |x| = s 2^(e - 53)
   unsigned __int128 q = ((unsigned __int128)s << 72) / (unsigned)div;       // |x| / div = q 2^(e - 125)

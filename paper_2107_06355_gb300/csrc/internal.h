@@ -57,7 +57,8 @@ struct StepArgs {
 // (collision_args.cpp).
 int collision_kind(const pplbm_relax* r);
 // x / div as a fixed-point factor m 2^e, 2^62 <= |m| < 2^63, rounded to nearest; m = 0
-// for 0, with an exponent that shifts every product out (collision_args.cpp).
+// for 0, with an exponent that shifts every product out. An infinity or NaN gets an exponent
+// that no frame holds: every node leaves the fixed-point path (collision_args.cpp).
 fx::FixNum fixnum(double x, int div);
 // The EOS d with interaction parameter G as fixed-point factors (collision_args.cpp).
 EosFix make_eos_fix(const pplbm_eos_derived& d, double G);
