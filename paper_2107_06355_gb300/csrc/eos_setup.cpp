@@ -17,6 +17,8 @@
 //  * eps: Newton's method from eps = 2 (Sec. III.A).
 #include <cmath>
 #include <cstring>
+#include <memory>
+#include <new>
 
 #include "../../include/pplbm.h"
 #include "eos.cuh"
@@ -71,13 +73,14 @@ constexpr int kPanels = 48;
 // The set-up's root finders integrate over the same three regions many times, so the
 // nodes (an exponential each) are formed once per region, and Newton's method on eps keeps
 // the logarithms too: 0.65 ms per Smooth set-up (4.4 with an exponential, a power and an
-// indirect call per evaluation), 1.2 ms Modified Smooth (1.9), 1.3 ms Peng (3.0).
+// indirect call per evaluation), 1.2 ms Modified Smooth (1.9), 1.3 ms Peng (3.0). They are kept
+// on the heap (8 KB a region, 23 KB with the logarithms): a caller's thread may have a small
+// stack.
 struct LogNodes {
   static constexpr int n = kPanels * GaussLegendre::n;
   double rho[n];
   double h2;  // half a panel's width
-  LogNodes() = default;
-  LogNodes(double lo, double hi) {
+  void set(double lo, double hi) {
     const GaussLegendre& g = gl();
     const double s0 = std::log(lo), s1 = std::log(hi);
     const double h = (s1 - s0) / kPanels;
@@ -325,7 +328,7 @@ struct MechIntegral {
     nreg = e.mode == PPLBM_EOS_PENG ? 1 : 3;
     for (int r = 0; r < nreg; ++r) {
       Region& g = regions[r];
-      g.q = LogNodes(edges[r], edges[r + 1]);
+      g.q.set(edges[r], edges[r + 1]);
       for (int i = 0; i < LogNodes::n; ++i) {
         const double rho = g.q.rho[i], psi2 = eos_psi2(e, rho);
         g.f[i] = mech_term(e, d, rho, psi2);
@@ -334,17 +337,28 @@ struct MechIntegral {
     }
   }
 
+  // (the sums in the order of LogNodes::integrate)
   void at(double eps, double* g_out, double* dg_out) const {
+    const GaussLegendre& gauss = gl();
     double g = 0.0, dg = 0.0;
-    double t[LogNodes::n];
     for (const Region* p = regions; p != regions + nreg; ++p) {
-      const Region& r = *p;
-      for (int i = 0; i < LogNodes::n; ++i) t[i] = r.f[i] * std::exp(-0.5 * eps * r.ln[i]);
-      g += r.q.integrate([&](int i) { return t[i]; });
-      if (dg_out) dg += r.q.integrate([&](int i) { return -0.5 * r.ln[i] * t[i]; });
+      double total = 0.0, dtotal = 0.0;
+      for (int j = 0; j < LogNodes::n; j += GaussLegendre::n) {
+        double acc = 0.0, dacc = 0.0;
+        for (int k = 0; k < GaussLegendre::n; ++k) {
+          const int i = j + k;
+          const double t = p->f[i] * std::exp(-0.5 * eps * p->ln[i]);
+          acc += gauss.w[k] * t * p->q.rho[i];
+          dacc += gauss.w[k] * (-0.5 * p->ln[i] * t) * p->q.rho[i];
+        }
+        total += p->q.h2 * acc;
+        dtotal += p->q.h2 * dacc;
+      }
+      g += total;
+      dg += dtotal;
     }
     *g_out = g;
-    if (dg_out) *dg_out = dg;
+    *dg_out = dg;
   }
 };
 
@@ -356,11 +370,12 @@ static double mech_integral_0(const pplbm_eos_derived& d, const LogNodes& q) {
 
 // Newton from eps = 2 on g(eps) = 0 (Sec. III.A)
 bool solve_eps(const pplbm_eos_derived& d, double& eps_out) {
-  const MechIntegral m(d);
+  const std::unique_ptr<const MechIntegral> m(new (std::nothrow) MechIntegral(d));
+  if (!m) return false;
   double eps = 2.0;
   for (int it = 0; it < 100; ++it) {
     double g, dg;
-    m.at(eps, &g, &dg);
+    m->at(eps, &g, &dg);
     if (!std::isfinite(g) || !std::isfinite(dg) || dg == 0.0) return false;
     const double step = g / dg;
     eps -= step;
@@ -415,7 +430,9 @@ extern "C" pplbm_status pplbm_eos_setup(const pplbm_eos_params* p, double G, ppl
     d.dpdrho_v = liq.dp(d.rho_v);
     d.dpdrho_l = liq.dp(d.rho_l);
     const double rt = p->r_theta;
-    const LogNodes loop(d.rho_v, d.rho_l);
+    const std::unique_ptr<LogNodes> loop(new (std::nothrow) LogNodes);
+    if (!loop) return PPLBM_ERR_EOS_SETUP;
+    loop->set(d.rho_v, d.rho_l);
     auto with_rho_m = [&](double rm) {
       pplbm_eos_derived t = d;
       t.rho_m = rm;
@@ -428,7 +445,7 @@ extern "C" pplbm_status pplbm_eos_setup(const pplbm_eos_params* p, double G, ppl
       const EosConst e = make_eos_const(t);
       for (int k = 0; k <= 64; ++k)  // psi^2 must stay positive on the loop
         if (!(eos_psi2(e, t.rho_v + (t.rho_l - t.rho_v) * k / 64.0) > 0.0)) return (double)NAN;
-      return mech_integral_0(t, loop);
+      return mech_integral_0(t, *loop);
     };
     const double span = d.rho_l - d.rho_v;
     double prev_x = d.rho_v + 1e-3 * span, prev_f = resid(prev_x), rm = NAN;
@@ -463,7 +480,12 @@ extern "C" pplbm_status pplbm_eos_setup(const pplbm_eos_params* p, double G, ppl
     const double lo = d.p_sat + 1e-9 * (hi - d.p_sat);
     const bool modified = p->mode == PPLBM_EOS_SMOOTH_MOD;
     // the Maxwell residual's regions; p_max does not enter the third
-    const LogNodes q1(d.rho_v, d.rho_max), q2(d.rho_max, d.rho_min), q3(d.rho_min, d.rho_l);
+    const std::unique_ptr<LogNodes[]> q(new (std::nothrow) LogNodes[3]);
+    if (!q) return PPLBM_ERR_EOS_SETUP;
+    LogNodes &q1 = q[0], &q2 = q[1], &q3 = q[2];
+    q1.set(d.rho_v, d.rho_max);
+    q2.set(d.rho_max, d.rho_min);
+    q3.set(d.rho_min, d.rho_l);
     const double part3 = maxwell_part(make_eos_const(d), d.p_sat, q3);
     auto resid = [&](double pm) {
       pplbm_eos_derived t = d;
