@@ -121,7 +121,7 @@ PPLBM_FX bool collide_reverse_fixed(const CollideFix& k, const u64 (&psi)[9], do
   i64 hx0 = 2 * mulhi(f3, fuy), hy0 = 0, jy0 = 0, Kxb = 0, Kyb = 0, rb0 = 0;
   const int kl = el - 1086;
   // n / 36 in units of 2^(k - 4): times 16/36
-  auto over36 = [&](i64 n, int k) { return frame_to_double(mulhi(factor(n), factor((i64)kFourNinths)), k - 4); };
+  auto over36 = [&](i64 n, int k) { return frame_to_double(mulhi_k(factor((i64)kFourNinths), factor(n)), k - 4); };
   if (SHEAR) {
     const i64 w = one_minus_omega(k, L, er, &ok);
     ok = ok && in_range(w, 0x40000000u);

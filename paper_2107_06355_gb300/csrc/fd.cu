@@ -364,6 +364,7 @@ using fx::factor;
 using fx::i64;
 using fx::mulhi;
 using fx::mulhi2;
+using fx::mulhi_k;
 using fx::u32;
 
 __device__ __forceinline__ u32 i32_of(i64 x) { return (u32)((u64)x >> 32); }
@@ -406,10 +407,10 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
     const Factor kS = factor(k.kS4), kL = factor(k.kL), kD = factor(k.kD);
     // 4 S_a, S_0 = Pd_0 Pxx + Pd_1 Dxy / 4
     const i64 s0 = mulhi2(factor(4 * pd0), factor(pxx), q, f1), s1 = mulhi2(factor(4 * pd1), factor(pyy), q, f0);
-    F0 = mulhi(kS, factor(up(s0, 3))) + mulhi(kL, factor(up(mulhi(f0, fl), 3))) +
-         mulhi(kD, factor(up(mulhi(fc, factor(dl0)), 1)));
-    F1 = mulhi(kS, factor(up(s1, 3))) + mulhi(kL, factor(up(mulhi(f1, fl), 3))) +
-         mulhi(kD, factor(up(mulhi(fc, factor(dl1)), 1)));
+    F0 = mulhi_k(kS, factor(up(s0, 3))) + mulhi_k(kL, factor(up(mulhi(f0, fl), 3))) +
+         mulhi_k(kD, factor(up(mulhi(fc, factor(dl0)), 1)));
+    F1 = mulhi_k(kS, factor(up(s1, 3))) + mulhi_k(kL, factor(up(mulhi(f1, fl), 3))) +
+         mulhi_k(kD, factor(up(mulhi(fc, factor(dl1)), 1)));
   }
   // velocities, one frame for both components (9 values each: C, E, W, N, S, NE, NW, SW, SE)
   u64 ub[2][9];
@@ -461,7 +462,7 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
   const Factor cA = factor(k.cA), ux = factor(vel[0]), uy = factor(vel[1]), fDv = factor(Dv), fSh = factor(Sh);
   // mass: -cA (rho div u + u . grad rho)
   const i64 m = mulhi(factor(r[0]), fDv) + mulhi2(ux, factor(Dr0), uy, factor(Dr1));
-  *drho = fx::frame_to_double(-mulhi(cA, factor(up(m, 3))), er + eu + 125 + k.eA);
+  *drho = fx::frame_to_double(-mulhi_k(cA, factor(up(m, 3))), er + eu + 125 + k.eA);
   // viscous terms
   i64 v1 = k.v1, v2 = k.v2, v3 = k.v3, v4 = k.v4, w1 = k.v1;  // w1: the one of rho U_yy
   if (VV) {
@@ -479,24 +480,24 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
   }
   const Factor f1 = factor(v1), f2 = factor(v2), f3 = factor(v3), f4 = factor(v4), fw = factor(w1);
   const Factor dr0 = factor(2 * Dr0), dr1 = factor(2 * Dr1), r2 = factor(2 * r[0]);
-  const i64 V0 = mulhi(f1, factor(up(mulhi2(dr0, factor(D[0][0]), factor(Dr1), fSh), 1))) +
-                 mulhi(f2, factor(mulhi(dr0, fDv))) +
-                 mulhi(r2, factor(mulhi2(f3, factor(xx[0]), f4, factor(xy[1])) + mulhi(fw, factor(yy[0]))));
-  const i64 V1 = mulhi(f1, factor(up(mulhi2(dr1, factor(D[1][1]), factor(Dr0), fSh), 1))) +
-                 mulhi(f2, factor(mulhi(dr1, fDv))) +
-                 mulhi(r2, factor(mulhi2(f3, factor(yy[1]), f4, factor(xy[0])) + mulhi(fw, factor(xx[1]))));
+  const i64 V0 = mulhi_k(f1, factor(up(mulhi2(dr0, factor(D[0][0]), factor(Dr1), fSh), 1))) +
+                 mulhi_k(f2, factor(mulhi(dr0, fDv))) +
+                 mulhi(r2, factor(mulhi_k(f3, factor(xx[0])) + mulhi_k(f4, factor(xy[1])) + mulhi_k(fw, factor(yy[0]))));
+  const i64 V1 = mulhi_k(f1, factor(up(mulhi2(dr1, factor(D[1][1]), factor(Dr0), fSh), 1))) +
+                 mulhi_k(f2, factor(mulhi(dr1, fDv))) +
+                 mulhi(r2, factor(mulhi_k(f3, factor(yy[1])) + mulhi_k(f4, factor(xy[0])) + mulhi_k(fw, factor(xx[1]))));
   // (V - F - cA dp) / rho
   const int eV = er + eu + 127 + k.ev, eF = 2 * es + 125 + k.eF, eP = egp - 1086 + 64 + k.eA;
   const int e = max(max(eV, eF), eP);
-  const i64 a0 = fx::shr_s(V0, e - eV) - fx::shr_s(F0, e - eF) - fx::shr_s(mulhi(cA, factor(Dp0)), e - eP);
-  const i64 a1 = fx::shr_s(V1, e - eV) - fx::shr_s(F1, e - eF) - fx::shr_s(mulhi(cA, factor(Dp1)), e - eP);
+  const i64 a0 = fx::shr_s(V0, e - eV) - fx::shr_s(F0, e - eF) - fx::shr_s(mulhi_k(cA, factor(Dp0)), e - eP);
+  const i64 a1 = fx::shr_s(V1, e - eV) - fx::shr_s(F1, e - eF) - fx::shr_s(mulhi_k(cA, factor(Dp1)), e - eP);
   ok = ok && (u32)(i32_of(a0) + 0x08000000u) < 0x10000000u && (u32)(i32_of(a1) + 0x08000000u) < 0x10000000u;
   const Factor inv = factor(fx::reciprocal<8>(fx::significand(rb[0])));
   const int e1 = e + 1022 - (int)(fx::hi32(rb[0]) >> 20);
   // advection: cA u . grad u
   const Factor ux2 = factor(2 * vel[0]), uy2 = factor(2 * vel[1]);
-  const i64 y0 = mulhi(cA, factor(up(mulhi2(ux2, factor(D[0][0]), uy2, factor(D[1][0])), 3)));
-  const i64 y1 = mulhi(cA, factor(up(mulhi2(ux2, factor(D[0][1]), uy2, factor(D[1][1])), 3)));
+  const i64 y0 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][0]), uy2, factor(D[1][0])), 3)));
+  const i64 y1 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][1]), uy2, factor(D[1][1])), 3)));
   const int e2 = 2 * eu + 124 + k.eA, em = max(e1, e2);
   *dux = fx::frame_to_double(fx::shr_s(mulhi(factor(up(a0, 3)), inv), em - e1) - fx::shr_s(y0, em - e2), em);
   *duy = fx::frame_to_double(fx::shr_s(mulhi(factor(up(a1, 3)), inv), em - e1) - fx::shr_s(y1, em - e2), em);

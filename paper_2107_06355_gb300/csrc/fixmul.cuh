@@ -124,6 +124,13 @@ PPLBM_FX i64 mulhi(Factor x, Factor y) {
   return mad(x.hi, y.hi, m >> 31);
 }
 
+// Upper 64 bits of k x for a constant k: the product of the low halves has the mean lo/2 units of
+// k's low half instead of 1/4, which would leave up to 1/4 unit in every result.
+PPLBM_FX i64 mulhi_k(Factor k, Factor x) {
+  const i64 m = mad(k.hi, x.lo, mad(x.hi, k.lo, (1 << 30) + (k.lo >> 1)));
+  return mad(k.hi, x.hi, m >> 31);
+}
+
 // Upper 64 bits of x y + z w (the middle partial sums of both below 2^63 in magnitude:
 // factors below 2^62); error below 4 units, on average none.
 PPLBM_FX i64 mulhi2(Factor x, Factor y, Factor z, Factor w) {

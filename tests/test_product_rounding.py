@@ -18,6 +18,7 @@ def mh(tmp_path_factory):
     lib = C.CDLL(so)
     lib.mh_product.argtypes = [C.c_longlong] + [C.c_void_p] * 3
     lib.mh_pair.argtypes = [C.c_longlong] + [C.c_void_p] * 5
+    lib.mh_constant.argtypes = [C.c_longlong, C.c_longlong] + [C.c_void_p] * 2
     return lib
 
 
@@ -41,6 +42,20 @@ def test_mean_error(mh, bits, terms):
     f = [rng.integers(-(1 << b), 1 << b, n) for b in bits * terms]
     err = errors(mh, *f)
     assert np.abs(err).max() < 2.0 * terms and abs(err.mean()) < 0.02 * terms
+
+
+@pytest.mark.parametrize("k", [0x71C71C71C71C71C7, 0x1999999999999A00, -0x1999999999999A00, 1 << 61,
+                               (1 << 61) + 0x7FFFFFFF, (1 << 61) + 0xFFFFFFFE])
+@pytest.mark.parametrize("bits", [62, 50, 40])
+def test_mean_error_with_a_constant(mh, k, bits):
+    """As above with the low halves' product at its mean for this constant (half its low half):
+    the same bounds, for constants whose low half is 0, all ones, or in between; zero stays zero."""
+    x = np.random.default_rng(bits).integers(-(1 << bits), 1 << bits, 40_000)
+    x[0] = 0
+    out = np.zeros(len(x), np.int64)
+    mh.mh_constant(len(x), k, x.ctypes.data, out.ctypes.data)
+    err = np.array([((int(o) << 64) - k * int(v)) / 2.0**64 for o, v in zip(out, x)])
+    assert out[0] == 0 and np.abs(err).max() < 2.0 and abs(err.mean()) < 0.02
 
 
 def test_zero_factors(mh):
