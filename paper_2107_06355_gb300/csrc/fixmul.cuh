@@ -124,13 +124,12 @@ PPLBM_FX i64 mulhi(Factor x, Factor y) {
   return mad(x.hi, y.hi, m >> 31);
 }
 
-// Upper 64 bits of k x for a constant k, whose halves' fractions lo, hi are known: the product of
-// the low halves has the mean lo/2 instead of 1/4, and x's dropped bit the mean hi/4 instead of
-// none, which would leave up to 1/2 unit in every result. (The addend stays below one unit, so
-// that x = 0 gives 0: where 1/2 + lo/2 + hi/4 exceeds it, the rest, at most 1/4, remains.)
+// Upper 64 bits of k x for a constant k: the product of the low halves has the mean lo/2 units of
+// k's low half instead of 1/4, which would leave up to 1/4 unit in every result. (x's lowest
+// bit, which a factor drops, counts for hi/4 on average where it is not empty; the
+// finite-difference update's factors are shifted up or come from doubles.)
 PPLBM_FX i64 mulhi_k(Factor k, Factor x) {
-  const u32 mean = (1u << 30) + ((u32)k.lo >> 1) + (u32)(k.hi >> 2);
-  const i64 m = mad(k.hi, x.lo, mad(x.hi, k.lo, (i64)(mean < 0x7FFFFFFFu ? mean : 0x7FFFFFFFu)));
+  const i64 m = mad(k.hi, x.lo, mad(x.hi, k.lo, (1 << 30) + (k.lo >> 1)));
   return mad(k.hi, x.hi, m >> 31);
 }
 
