@@ -347,15 +347,20 @@ __device__ __noinline__ void fd_update_general(const FDArgs& a, int x, int y) {
 //   F (the psi terms)      in units of 2^(2 es + 125 + eF),
 //   V (the viscous terms)  in units of 2^(er + eu + 127 + ev),
 //   cA dp                  in units of 2^(ep + 64 + eA);
-// V - F - cA dp is formed in the coarsest of the three, divided by rho and joined with the
-// advection. The units are below the rounding errors that the stored doubles bring into
-// the differences (2^-53 psi, u, rho): F is kept to 2^-56 psi^2 of its coefficients, V to
-// 2^-56 rho u, so the results' errors are those of the double-precision form. Conditions:
-// psi, rho positive, all fields between 2^-320 and 2^100 (smaller velocities and pressures
-// count as zero), and accelerations that leave 3 bits of their frame free.
+// V - F - cA dp is formed in units of 2^-60 of the largest of the three, divided by rho and
+// joined with the advection. The units are below the rounding errors that the stored doubles
+// bring into the differences (2^-53 psi, u, rho): F is kept to 2^-56 psi^2 of its coefficients,
+// V to 2^-56 rho u, so the results' errors are those of the double-precision form. They must
+// have no mean, which nothing takes back out of a velocity: with products rounded down and the
+// three cut to the coarsest of their units, a 44 x 40 droplet gained 2e-18 per step in both
+// components (rms error against extended precision after 400 steps 7.4e-16; 1.0e-16 so, and in
+// double precision), with tau(rho) 5e-17 (2.3e-14; 1.0e-16, in double precision 7.7e-17), a
+// shear flow of 1e-3 1.4e-18 (5.4e-16; 3e-19 and 2e-19). It costs 3 to 4 % of a step.
+// Conditions: psi, rho positive, all fields between 2^-320 and 2^100 (smaller velocities and
+// pressures count as zero).
 //
 // What bounds it: instruction issue and the integer ALU pipe (640 instructions per point, 390
-// of them on that pipe). With its products on the FP64 pipe (54 to 60 instructions per
+// of them on that pipe, before the 40 of the common unit). With its products on the FP64 pipe (54 to 60 instructions per
 // point) and every difference rounded to a double in integer code (1,950) both pipes were 80
 // to 90 % busy. Per step (two updates, two density passes): 1200 x 500 264 -> 115 us, 2048 x
 // 1024 804 -> 314, 600 x 250 with tau(rho) 99 -> 55; 102, 310 and 42 with dependent launches.
@@ -467,9 +472,9 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
   i64 v1 = k.v1, v2 = k.v2, v3 = k.v3, v4 = k.v4, w1 = k.v1;  // w1: the one of rho U_yy
   if (VV) {
     // mu = rho n1, n1 = g0 + g1 rho, mu_B = rho n2, n2 = e0 - g1 rho; d mu / d rho = n1 + g1 rho
-    const int d = k.ev - (er + 64 + k.g1.e);
+    const int d = k.ev - (er + 62 + k.g1.e);  // two places up: 0 or more for rho up to 2 rho_l
     ok = ok && d >= 0;
-    const i64 gr = fx::shr_s(mulhi(factor(k.g1.m), factor(r[0])), d);
+    const i64 gr = fx::shr_s(up(mulhi(factor(k.g1.m), factor(r[0])), 2), d);
     ok = ok && (u32)(i32_of(gr) + 0x10000000u) < 0x20000000u;
     const i64 n1 = k.g0 + gr, n2 = k.e0 - gr;
     w1 = n1;
@@ -489,18 +494,26 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
   // (V - F - cA dp) / rho
   const int eV = er + eu + 127 + k.ev, eF = 2 * es + 125 + k.eF, eP = egp - 1086 + 64 + k.eA;
   const int e = max(max(eV, eF), eP);
-  const i64 a0 = fx::shr_s(V0, e - eV) - fx::shr_s(F0, e - eF) - fx::shr_s(mulhi_k(cA, factor(Dp0)), e - eP);
-  const i64 a1 = fx::shr_s(V1, e - eV) - fx::shr_s(F1, e - eF) - fx::shr_s(mulhi_k(cA, factor(Dp1)), e - eP);
-  ok = ok && (u32)(i32_of(a0) + 0x08000000u) < 0x10000000u && (u32)(i32_of(a1) + 0x08000000u) < 0x10000000u;
+  // the three in a unit that the largest of them sets (of the two components): 2^-60 of it
+  const i64 P0 = mulhi_k(cA, factor(Dp0)), P1 = mulhi_k(cA, factor(Dp1));
+  auto free_places = [&](i64 x, i64 y, int ex) {
+    return fx::clz64((u64)(x ^ (x >> 63)) | (u64)(y ^ (y >> 63))) + (e - ex);
+  };
+  const int n = min(min(free_places(V0, V1, eV), free_places(F0, F1, eF)), min(free_places(P0, P1, eP), 64)) - 4;
+  ok = ok && n >= 0;
+  const int nV = n - (e - eV), nF = n - (e - eF), nP = n - (e - eP);
+  auto moved = [](i64 x, int k) { return k >= 0 ? up(x, k) : fx::shr_s(x, -k); };
+  const i64 a0 = moved(V0, nV) - moved(F0, nF) - moved(P0, nP);
+  const i64 a1 = moved(V1, nV) - moved(F1, nF) - moved(P1, nP);
   const Factor inv = factor(fx::reciprocal<8>(fx::significand(rb[0])));
-  const int e1 = e + 1022 - (int)(fx::hi32(rb[0]) >> 20);
+  const int e1 = e - n + 1025 - (int)(fx::hi32(rb[0]) >> 20);
   // advection: cA u . grad u
   const Factor ux2 = factor(2 * vel[0]), uy2 = factor(2 * vel[1]);
   const i64 y0 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][0]), uy2, factor(D[1][0])), 3)));
   const i64 y1 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][1]), uy2, factor(D[1][1])), 3)));
   const int e2 = 2 * eu + 124 + k.eA, em = max(e1, e2);
-  *dux = fx::frame_to_double(fx::shr_s(mulhi(factor(up(a0, 3)), inv), em - e1) - fx::shr_s(y0, em - e2), em);
-  *duy = fx::frame_to_double(fx::shr_s(mulhi(factor(up(a1, 3)), inv), em - e1) - fx::shr_s(y1, em - e2), em);
+  *dux = fx::frame_to_double(fx::shr_s(mulhi(factor(a0), inv), em - e1) - fx::shr_s(y0, em - e2), em);
+  *duy = fx::frame_to_double(fx::shr_s(mulhi(factor(a1), inv), em - e1) - fx::shr_s(y1, em - e2), em);
   return ok;
 }
 
@@ -569,14 +582,14 @@ int frame_of(std::initializer_list<double> v, int* ok) {
 
 fx::i64 in_frame(double x, int e) { return (fx::i64)std::llrint(std::ldexp((long double)x, -e)); }
 
-FDFix fd_fix(const FDArgs& a, bool vary) {
+FDFix fd_fix(const FDArgs& a, bool vary, double rho_l) {
   FDFix k;
   std::memset(&k, 0, sizeof(k));
   k.ok = 1;
   k.eF = frame_of({0.25 * a.kS, a.kL, a.kD}, &k.ok);
   k.eA = frame_of({a.cA}, &k.ok);
-  // tau_nu(rho): the largest of the combinations for rho up to 4
-  k.ev = vary ? frame_of({16.0 * a.g0, 16.0 * a.e0, 64.0 * a.g1}, &k.ok) : frame_of({a.v1, a.v2, a.v3, a.v4}, &k.ok);
+  // tau_nu(rho): room for the combinations with rho up to 2 rho_l (denser points take the general form)
+  k.ev = vary ? frame_of({4.0 * a.g0, 4.0 * a.e0, 8.0 * rho_l * a.g1}, &k.ok) : frame_of({a.v1, a.v2, a.v3, a.v4}, &k.ok);
   if (!k.ok) return k;
   k.kS4 = in_frame(0.25 * a.kS, k.eF);
   k.kL = in_frame(a.kL, k.eF);
@@ -738,7 +751,7 @@ pplbm_status pplbm_fd_step(pplbm_fd* f, int64_t nsteps, double dt) {
   }
   a.psi = f->psi;
   a.p = f->p;
-  g.k = fd_fix(a, f->var_visc);
+  g.k = fd_fix(a, f->var_visc, f->derived.rho_l);
   const int64_t n = f->n, np = f->np, off = f->off;
   const unsigned wb = (unsigned)((f->nx + 63) / 64);
   const double two_dy = 2.0 * f->dx, psi_l = f->derived.psi_l;
