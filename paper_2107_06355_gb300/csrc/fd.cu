@@ -340,7 +340,8 @@ __device__ __noinline__ void fd_update_general(const FDArgs& a, int x, int y) {
 // ---- the update in fixed point ------------------------------------------------------
 //
 // Every field's stencil values become integers in one frame (psi: 13 values, the two
-// velocity components together: 18, rho and p: 3 each), so differences are exact, and the
+// velocity components together: 18, unless their largest values are a factor of 2^7 or more
+// apart; rho and p: 3 each), so differences are exact, and the
 // products of differences are taken to 64 bits (fixmul.cuh) in frames that follow from
 // the fields' and the constants'. With psi in units of 2^es (psi < 2^60), u of 2^eu (u <
 // 2^59), rho of 2^er and p of 2^ep (below 2^61):
@@ -355,9 +356,12 @@ __device__ __noinline__ void fd_update_general(const FDArgs& a, int x, int y) {
 // three cut to the coarsest of their units, a 44 x 40 droplet gained 2e-18 per step in both
 // components (rms error against extended precision after 400 steps 7.4e-16; 1.0e-16 so, and in
 // double precision), with tau(rho) 5e-17 (2.3e-14; 1.0e-16, in double precision 7.7e-17), a
-// shear flow of 1e-3 1.4e-18 (5.4e-16; 3e-19 and 2e-19). It costs 3 to 4 % of a step.
-// Conditions: psi, rho positive, all fields between 2^-320 and 2^100 (smaller velocities and
-// pressures count as zero).
+// shear flow of 1e-3 1.4e-18 (5.4e-16; 3e-19 and 2e-19). It costs 3 to 4 % of a step. A velocity
+// component much smaller than the other (a shear of 1e-8 across a uniform drift of 0.1) would
+// lose places in a common frame: 4e-16 after 400 steps; 3e-24 so, as in double precision, for
+// another 2 to 3 % of a step.
+// Conditions: psi, rho positive, all fields between 2^-320 and 2^100 (velocities may be zero;
+// smaller pressures count as zero).
 //
 // What bounds it: instruction issue and the integer ALU pipe (640 instructions per point, 390
 // of them on that pipe, before the 40 of the common unit). With its products on the FP64 pipe (54 to 60 instructions per
@@ -382,6 +386,10 @@ __device__ __forceinline__ i64 fd_term(u64 b, int eg) {
 }
 
 __device__ __forceinline__ i64 up(i64 x, int k) { return (i64)((u64)x << k); }
+
+// x 2^k for k of either sign, and |x| up to one
+__device__ __forceinline__ i64 moved(i64 x, int k) { return k >= 0 ? up(x, k) : fx::shr_s(x, -k); }
+__device__ __forceinline__ u64 mag(i64 x) { return (u64)(x ^ (x >> 63)); }
 
 template <bool PRED, bool VV>
 __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k, const int (&cx)[5],
@@ -417,9 +425,10 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
     F1 = mulhi_k(kS, factor(up(s1, 3))) + mulhi_k(kL, factor(up(mulhi(f1, fl), 3))) +
          mulhi_k(kD, factor(up(mulhi(fc, factor(dl1)), 1)));
   }
-  // velocities, one frame for both components (9 values each: C, E, W, N, S, NE, NW, SW, SE)
+  // velocities (9 values each: C, E, W, N, S, NE, NW, SW, SE), in one frame, or each in its own
+  // where the smaller one would lose places that the stored doubles have (see far)
   u64 ub[2][9];
-  u32 mu = 0;
+  int eu[2];  // units 2^eu
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const double* f = c == 0 ? a.ux : a.uy;
@@ -427,24 +436,56 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
                       at(f, 1, 1), at(f, -1, 1), at(f, -1, -1), at(f, 1, -1)};
 #pragma unroll
     for (int i = 0; i < 9; ++i) ub[c][i] = v[i];
+    u32 mu = 0;
 #pragma unroll
     for (int i = 0; i < 9; i += 3)
       mu = max(mu, fx::max3(fx::mag_hi(v[i]), fx::mag_hi(v[i + 1]), fx::mag_hi(v[i + 2])));
+    ok = ok && mu < kTop && mu - 1u >= (703u << 20) - 1u;  // all zero, or the largest at least 2^-320
+    eu[c] = mu != 0u ? (int)(mu >> 20) - 1081 : -100000;
   }
-  ok = ok && mu < kTop;
-  const int egu = max((int)(mu >> 20), 703) + 5, eu = egu - 1086;
+  const int em_u = max(max(eu[0], eu[1]), 703 - 1081);
+  const bool far = em_u - min(eu[0], eu[1]) - 7u < 50000u;  // apart by 7 or more, neither zero
+  if (!far) eu[0] = eu[1] = em_u;
   i64 vel[2], D[2][2], xx[2], yy[2], xy[2];  // D[axis][component]
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     i64 v[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) v[i] = fd_term(ub[c][i], egu);
+    for (int i = 0; i < 9; ++i) v[i] = fd_term(ub[c][i], eu[c] + 1086);
     vel[c] = v[0];
     D[0][c] = PRED ? v[1] - v[0] : v[0] - v[2];
     D[1][c] = PRED ? v[3] - v[0] : v[0] - v[4];
     xx[c] = v[1] + v[2] - 2 * v[0];
     yy[c] = v[3] + v[4] - 2 * v[0];
     xy[c] = (v[5] - v[8]) - (v[6] - v[7]);
+  }
+  if (far) {
+    vel[0] = fx::shr_s(vel[0], em_u - eu[0]);
+    vel[1] = fx::shr_s(vel[1], em_u - eu[1]);
+  }
+  // advection: cA u . grad u_c in units of 2^(em_u + eu_c + 124 + eA)
+  const Factor cA = factor(k.cA), ux2 = factor(2 * vel[0]), uy2 = factor(2 * vel[1]);
+  const i64 y0 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][0]), uy2, factor(D[1][0])), 3)));
+  const i64 y1 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][1]), uy2, factor(D[1][1])), 3)));
+  const int ey0 = em_u + eu[0] + 124 + k.eA, ey1 = em_u + eu[1] + 124 + k.eA;
+  int ed = em_u;  // the differences' unit from here on: set by the largest of them if far
+  if (far) {
+    int g[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const u64 any = mag(D[0][c]) | mag(D[1][c]) | mag(xx[c]) | mag(yy[c]) | mag(xy[c]);
+      g[c] = any ? eu[c] - max(fx::clz64(any) - 4, 0) : -100000;  // zeros set none
+    }
+    ed = max(g[0], g[1]);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int to = eu[c] - ed;
+      D[0][c] = moved(D[0][c], to);
+      D[1][c] = moved(D[1][c], to);
+      xx[c] = moved(xx[c], to);
+      yy[c] = moved(yy[c], to);
+      xy[c] = moved(xy[c], to);
+    }
   }
   const i64 Dv = D[0][0] + D[1][1], Sh = D[0][1] + D[1][0];
   // rho and p at the point and its one-sided neighbours
@@ -464,10 +505,12 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
   }
   const i64 Dr0 = PRED ? r[1] - r[0] : r[0] - r[1], Dr1 = PRED ? r[2] - r[0] : r[0] - r[2];
   const i64 Dp0 = PRED ? p[1] - p[0] : p[0] - p[1], Dp1 = PRED ? p[2] - p[0] : p[0] - p[2];
-  const Factor cA = factor(k.cA), ux = factor(vel[0]), uy = factor(vel[1]), fDv = factor(Dv), fSh = factor(Sh);
+  const Factor ux = factor(vel[0]), uy = factor(vel[1]), fDv = factor(Dv), fSh = factor(Sh);
   // mass: -cA (rho div u + u . grad rho)
-  const i64 m = mulhi(factor(r[0]), fDv) + mulhi2(ux, factor(Dr0), uy, factor(Dr1));
-  *drho = fx::frame_to_double(-mulhi_k(cA, factor(up(m, 3))), er + eu + 125 + k.eA);
+  i64 div = mulhi(factor(r[0]), fDv);
+  if (far) div = fx::shr_s(div, em_u - ed);
+  const i64 m = div + mulhi2(ux, factor(Dr0), uy, factor(Dr1));
+  *drho = fx::frame_to_double(-mulhi_k(cA, factor(up(m, 3))), er + em_u + 125 + k.eA);
   // viscous terms
   i64 v1 = k.v1, v2 = k.v2, v3 = k.v3, v4 = k.v4, w1 = k.v1;  // w1: the one of rho U_yy
   if (VV) {
@@ -492,28 +535,25 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
                  mulhi_k(f2, factor(mulhi(dr1, fDv))) +
                  mulhi(r2, factor(mulhi_k(f3, factor(yy[1])) + mulhi_k(f4, factor(xy[0])) + mulhi_k(fw, factor(xx[1]))));
   // (V - F - cA dp) / rho
-  const int eV = er + eu + 127 + k.ev, eF = 2 * es + 125 + k.eF, eP = egp - 1086 + 64 + k.eA;
+  const int eV = er + ed + 127 + k.ev, eF = 2 * es + 125 + k.eF, eP = egp - 1086 + 64 + k.eA;
   const int e = max(max(eV, eF), eP);
-  // the three in a unit that the largest of them sets (of the two components): 2^-60 of it
+  // the three in a unit that the largest of them sets (of the two components): 2^-60 of it;
+  // zeros set none
   const i64 P0 = mulhi_k(cA, factor(Dp0)), P1 = mulhi_k(cA, factor(Dp1));
   auto free_places = [&](i64 x, i64 y, int ex) {
-    return fx::clz64((u64)(x ^ (x >> 63)) | (u64)(y ^ (y >> 63))) + (e - ex);
+    const u64 both = mag(x) | mag(y);
+    return both ? fx::clz64(both) + (e - ex) : 4096;
   };
-  const int n = min(min(free_places(V0, V1, eV), free_places(F0, F1, eF)), min(free_places(P0, P1, eP), 64)) - 4;
+  const int n = min(min(free_places(V0, V1, eV), free_places(F0, F1, eF)), free_places(P0, P1, eP)) - 4;
   ok = ok && n >= 0;
   const int nV = n - (e - eV), nF = n - (e - eF), nP = n - (e - eP);
-  auto moved = [](i64 x, int k) { return k >= 0 ? up(x, k) : fx::shr_s(x, -k); };
   const i64 a0 = moved(V0, nV) - moved(F0, nF) - moved(P0, nP);
   const i64 a1 = moved(V1, nV) - moved(F1, nF) - moved(P1, nP);
   const Factor inv = factor(fx::reciprocal<8>(fx::significand(rb[0])));
   const int e1 = e - n + 1025 - (int)(fx::hi32(rb[0]) >> 20);
-  // advection: cA u . grad u
-  const Factor ux2 = factor(2 * vel[0]), uy2 = factor(2 * vel[1]);
-  const i64 y0 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][0]), uy2, factor(D[1][0])), 3)));
-  const i64 y1 = mulhi_k(cA, factor(up(mulhi2(ux2, factor(D[0][1]), uy2, factor(D[1][1])), 3)));
-  const int e2 = 2 * eu + 124 + k.eA, em = max(e1, e2);
-  *dux = fx::frame_to_double(fx::shr_s(mulhi(factor(a0), inv), em - e1) - fx::shr_s(y0, em - e2), em);
-  *duy = fx::frame_to_double(fx::shr_s(mulhi(factor(a1), inv), em - e1) - fx::shr_s(y1, em - e2), em);
+  const int em0 = max(e1, ey0), em1 = max(e1, ey1);
+  *dux = fx::frame_to_double(fx::shr_s(mulhi(factor(a0), inv), em0 - e1) - fx::shr_s(y0, em0 - ey0), em0);
+  *duy = fx::frame_to_double(fx::shr_s(mulhi(factor(a1), inv), em1 - e1) - fx::shr_s(y1, em1 - ey1), em1);
   return ok;
 }
 
