@@ -567,9 +567,10 @@ pplbm_status pplbm_fixsum_collision_eval(long long n, int32_t shear, const doubl
 pplbm_status pplbm_fixsum_adjoint_eval(long long n, int32_t shear, const double* mu, const double* a,
                                        const double* gth, const double* lam, double* out, void* stream);
 
-/* FP64 issue-rate probe, the denominator of the step's arithmetic roofline (the
- * step's per-node arithmetic is double precision throughout, Sec. II; on this GPU
- * arithmetic issue, not memory, bounds it). Launches blocks_per_sm x (SM count)
+/* FP64 issue-rate probe, a denominator of the step's arithmetic roofline (the step's
+ * fields are doubles, Sec. II, its per-node arithmetic is 64-bit fixed point on the
+ * integer pipes and conversions to double, with double-precision forms for the nodes that
+ * leave the frames; on this GPU arithmetic issue, not memory, bounds it). Launches blocks_per_sm x (SM count)
  * blocks of 256 threads; each thread runs `iters` rounds of `chains` (1, 2, 4, 8,
  * 16 or 32) independent chains of one FP64 operation: op 0 fused multiply-add,
  * 1 add, 2 multiply; op 3 runs chains of the integer-pipe addition the step kernels

@@ -5,7 +5,7 @@
 // nodes, the collision pass one per tile of 256 nodes, with a tile shape (tw x th, tw*th =
 // 256) chosen per instance so that
 // narrow lattices (the 4-wide planar ones) do not leave threads idle. A
-// device-resident table maps each work item to its instance. Three ways to run a
+// device-resident table maps each work item to its instance. Four ways to run a
 // step, chosen by the autotuner:
 //   PLAN_LAUNCHES   two launches per step covering every instance;
 //   PLAN_GRAPH      the same two launches, two steps captured in a CUDA graph that

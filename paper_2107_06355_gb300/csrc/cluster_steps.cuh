@@ -5,8 +5,9 @@
 // for 256 x 4 nodes with plain launches, 7.9 with dependent ones (dependent_launch.cuh), of
 // which the arithmetic's latency is about 4.5. Here the cluster's blocks share the nodes, and
 // the hardware cluster barrier (release / acquire, no spinning in software) separates the
-// passes: 6.7 us. The per-node arithmetic is the step kernels', so the results are bitwise
-// theirs.
+// passes: 6.7 us (an interface at T_r = 0.6, some of whose nodes take the double-precision
+// collision; 5.6 at T_r = 0.8, where few do). The per-node arithmetic is the step kernels', so
+// the results are bitwise theirs.
 #pragma once
 
 #include <cuda_runtime.h>

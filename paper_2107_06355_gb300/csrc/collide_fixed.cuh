@@ -24,8 +24,10 @@
 // |J|, |Q| (and K = j - h) below 0.8 2^e (2^e <= rho), |zz| below 2^58 and the rows
 // 7, 8 corrections below 2^57, every population's sum stays below 2^63 in magnitude:
 // f1 is the largest, (8 + 18 0.64 + 12 0.8) 2^57.83 + 9 2^57 + 2^58 < 2^62.99. A node outside these
-// bounds (|u| of order one, a density out of the range of the frames, a population at
-// or below zero) is reported, and the caller runs the general collision.
+// bounds is reported, and the caller runs the general collision: nodes on the steep side of an
+// interface, where the Li term's product, before its shift, is 2^56 or more (to_frame asks for
+// six free places even where it then shifts right), and also |u| of order one, a density out
+// of the range of the frames, a population at or below zero, a constant that is not finite.
 #pragma once
 
 #include "fixmul.cuh"

@@ -360,8 +360,10 @@ __device__ __noinline__ void fd_update_general(const FDArgs& a, int x, int y) {
 // component much smaller than the other (a shear of 1e-8 across a uniform drift of 0.1) would
 // lose places in a common frame: 4e-16 after 400 steps; 3e-24 so, as in double precision, for
 // another 2 to 3 % of a step.
-// Conditions: psi, rho positive, all fields between 2^-320 and 2^100 (velocities may be zero;
-// smaller pressures count as zero).
+// Conditions: psi, rho positive, all fields between 2^-320 and 2^100, velocities from 2^-900 on
+// (smaller velocities and pressures count as zero: around a droplet in a fluid at rest they fall
+// off to nothing over hundreds of points, and in double precision every one of them would
+// take the time of three).
 //
 // What bounds it: instruction issue and the integer ALU pipe (640 instructions per point, 390
 // of them on that pipe, before the 40 of the common unit). With its products on the FP64 pipe (54 to 60 instructions per
@@ -379,6 +381,7 @@ using fx::u32;
 __device__ __forceinline__ u32 i32_of(i64 x) { return (u32)((u64)x >> 32); }
 
 constexpr int kFDThreads = 128, kFDBlocks = 5;
+constexpr int kLowest = -1000;  // of the results' units: exponents stay those of normal doubles
 
 // a value of either sign in the frame with top exponent eg, truncated in magnitude
 __device__ __forceinline__ i64 fd_term(u64 b, int eg) {
@@ -440,10 +443,10 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
 #pragma unroll
     for (int i = 0; i < 9; i += 3)
       mu = max(mu, fx::max3(fx::mag_hi(v[i]), fx::mag_hi(v[i + 1]), fx::mag_hi(v[i + 2])));
-    ok = ok && mu < kTop && mu - 1u >= (703u << 20) - 1u;  // all zero, or the largest at least 2^-320
-    eu[c] = mu != 0u ? (int)(mu >> 20) - 1081 : -100000;
+    ok = ok && mu < kTop;
+    eu[c] = mu >= (123u << 20) ? (int)(mu >> 20) - 1081 : -100000;  // below 2^-900 it counts as zero
   }
-  const int em_u = max(max(eu[0], eu[1]), 703 - 1081);
+  const int em_u = max(max(eu[0], eu[1]), 123 - 1081);
   const bool far = em_u - min(eu[0], eu[1]) - 7u < 50000u;  // apart by 7 or more, neither zero
   if (!far) eu[0] = eu[1] = em_u;
   i64 vel[2], D[2][2], xx[2], yy[2], xy[2];  // D[axis][component]
@@ -510,7 +513,8 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
   i64 div = mulhi(factor(r[0]), fDv);
   if (far) div = fx::shr_s(div, em_u - ed);
   const i64 m = div + mulhi2(ux, factor(Dr0), uy, factor(Dr1));
-  *drho = fx::frame_to_double(-mulhi_k(cA, factor(up(m, 3))), er + em_u + 125 + k.eA);
+  const int er0 = er + em_u + 125 + k.eA, er1 = max(er0, kLowest);
+  *drho = fx::frame_to_double(fx::shr_s(-mulhi_k(cA, factor(up(m, 3))), er1 - er0), er1);
   // viscous terms
   i64 v1 = k.v1, v2 = k.v2, v3 = k.v3, v4 = k.v4, w1 = k.v1;  // w1: the one of rho U_yy
   if (VV) {
@@ -551,7 +555,7 @@ __device__ __forceinline__ bool fd_update_fixed(const FDArgs& a, const FDFix& k,
   const i64 a1 = moved(V1, nV) - moved(F1, nF) - moved(P1, nP);
   const Factor inv = factor(fx::reciprocal<8>(fx::significand(rb[0])));
   const int e1 = e - n + 1025 - (int)(fx::hi32(rb[0]) >> 20);
-  const int em0 = max(e1, ey0), em1 = max(e1, ey1);
+  const int em0 = max(max(e1, ey0), kLowest), em1 = max(max(e1, ey1), kLowest);
   *dux = fx::frame_to_double(fx::shr_s(mulhi(factor(a0), inv), em0 - e1) - fx::shr_s(y0, em0 - ey0), em0);
   *duy = fx::frame_to_double(fx::shr_s(mulhi(factor(a1), inv), em1 - e1) - fx::shr_s(y1, em1 - ey1), em1);
   return ok;
@@ -707,7 +711,7 @@ pplbm_status pplbm_fd_create(pplbm_fd** out, const pplbm_lattice* lattice, const
   if (!out) return PPLBM_ERR_ARG;
   *out = nullptr;
   if (!lattice || !eos || !workspace || lattice->nx < 1 || lattice->ny < 1 || lattice->reserved != 0) return PPLBM_ERR_ARG;
-  if (lattice->ny > 65535 * 8) return PPLBM_ERR_ARG;  // the update pass's grid: 8-row tiles on its y axis
+  if (lattice->ny > 65535 * 8) return PPLBM_ERR_ARG;  // k_fd_update_general's grid: 8-row tiles on its y axis
   if (fd_walls(lattice) < 0) return PPLBM_ERR_ARG;
   if (!(tau_nu > 0.5) || !(tau_e > 0.0) || !(dx > 0.0)) return PPLBM_ERR_ARG;
   if (workspace_bytes < pplbm_fd_workspace_bytes(lattice)) return PPLBM_ERR_ARG;

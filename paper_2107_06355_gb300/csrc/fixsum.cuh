@@ -19,9 +19,11 @@
 // (number of operands) x 2^(G - 11) ulp of the largest operand of the exact sum
 // (the truncated bits), i.e. within 0.57 ulp for a sum of nine positive operands.
 // Against a chain of IEEE additions (a rounding per addition) it costs a fraction
-// of the integer instructions of the software additions of fp64.cuh and keeps the
-// FP64 pipe, the step's bottleneck, free; symmetric operand sets give exactly
-// cancelling sums (integer addition is associative).
+// of the integer instructions of the software additions of fp64.cuh, and none of the
+// FP64 pipe's; symmetric operand sets give exactly cancelling sums (integer addition is
+// associative). The step's fixed-point paths (fixmul.cuh) round nothing before their
+// results; these rounded sums serve their double-precision forms, the fields and the
+// reverse pass's gathers.
 //
 // Domain: positive normal finite operands below 2^1008 (callers test them, or
 // rely on the density pass's error word, which flags any non-finite or non-positive

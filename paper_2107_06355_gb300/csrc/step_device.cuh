@@ -38,8 +38,7 @@ __device__ __forceinline__ void rho_psi_double(const StepArgs& a, const double* 
   double rho, jx, jy, m7 = 0.0, m8 = 0.0;
   // When all nine populations are positive normal doubles (every bulk and interface
   // node of a physical state), the moments are exact integer sums in one fixed-point
-  // frame, each rounded once (fixsum.cuh): integer-pipe work only, leaving the FP64
-  // pipe, the pass's bottleneck, the EOS. Otherwise the same moments as IEEE sums.
+  // frame, each rounded once (fixsum.cuh). Otherwise the same moments as IEEE sums.
   const double fv[9] = {f0, f1, f2, f3, f4, f5, f6, f7, f8};
   unsigned max_hi = 0;
   if (KIND != kFullMrt && fx::positive_normal_range(fv, &max_hi)) {
@@ -204,8 +203,8 @@ template <int KIND, bool ST = false>
 __device__ __forceinline__ void collide_reduced(const StepArgs& a, int64_t node, double rho, double jx, double jy,
                                                 double psi0, double gx, double gy, const SurfQ& sq, Post& out,
                                                 double* ux_o, double* uy_o) {
-  // Additions run on the integer pipe (add_int, bitwise the FP64 add): the FP64
-  // pipe, this pass's bottleneck, keeps the products and fused multiply-adds.
+  // Additions run on the integer pipe (add_int, bitwise the FP64 add); the FP64 pipe, which
+  // bounds this form, keeps the products and fused multiply-adds.
   const double cH = a.half_force * psi0;  // h = cH g, cH = -G psi / 24
   const double hx = cH * gx, hy = cH * gy;
   const double inv_rho = fast_rcp(rho);
@@ -266,7 +265,8 @@ __device__ __forceinline__ void collide_reduced(const StepArgs& a, int64_t node,
 }
 
 // The same collision (Lambda = I, or rows 7, 8 at omega = 1/tau(rho) for kShearTau),
-// without the surface-tension source, arranged so that the FP64 pipe does only the
+// without the surface-tension source, for the nodes that leave the fixed-point path
+// (collide_general), arranged so that the FP64 pipe does only the
 // products, the reciprocals and the Li term (19 FP64 instructions per node for unit
 // relaxation times, 32 for the two-phase set): the sums J = j + h, P = j + 2h,
 // P + h (and j - h) come from one fixed-point frame, and the nine populations are
@@ -418,8 +418,10 @@ __device__ __forceinline__ void load_psi(const StepArgs& a, const Place& p, fx::
 }
 
 // The collision of a node outside the domain of the fixed-point path (collide_fixed.cuh):
-// force sums, then the general forms above. Kept out of line: it is rare, and inlined it
-// would set the kernels' register count.
+// force sums, then the general forms above. Out of line: inlined it would set the kernels'
+// register count. 2 to 3 % of a droplet's nodes take it, those on the steep side of the
+// interface, where the Li term leaves its frame (192^2, T_r = 0.6: 20 % of the rows of 32 have
+// one at every step; two-phase 128^2 at T_r = 0.35: 8 to 11 % and 45 to 49 %).
 template <int KIND, bool ST>
 __device__ __noinline__ void collide_general(const StepArgs& a, int x, int y, Post* out) {
   const Place pl = place_of(a, x, y);
@@ -566,7 +568,7 @@ __device__ __forceinline__ void guard_node(const StepArgs& a, int64_t i, double*
     v[2] += 1.0;
   } else {
     const int y = (int)(i / a.nx), x = (int)(i - (int64_t)y * a.nx);
-    // the collision pass's stencil sums (the same arithmetic, so the same force)
+    // the collision pass's stencil sums, rounded here to doubles
     double gx, gy;
     fx::shan_chen_stencil(psi_near(a, x, y, 1, 0), psi_near(a, x, y, -1, 0), psi_near(a, x, y, 0, 1),
                           psi_near(a, x, y, 0, -1), psi_near(a, x, y, 1, 1), psi_near(a, x, y, -1, 1),

@@ -65,7 +65,7 @@ def test_shear_flow(form):
 
 @pytest.mark.parametrize("form", ["constant", "vary"])
 @pytest.mark.parametrize("swap", [False, True])
-@pytest.mark.parametrize("small", [1e-8, 1e-3, 1e-60])
+@pytest.mark.parametrize("small", [1e-8, 1e-3, 1e-60, 1e-250])
 def test_small_component_beside_a_large_one(form, swap, small):
     """A uniform liquid drifting at 0.1 across a shear of amplitude `small`: the small component
     keeps the accuracy of its own size. Its right-hand side has about 20 roundings of 2^-53 of its
