@@ -22,7 +22,7 @@
 // 4.3e-14 with rounded double-precision stages; of 100 steps 1.4e-14, 3.0e-15 and 1.0e-14. It costs
 // 3 % of a gradient's step on 1024^2.
 // Reports a node outside the domain (that of the forward, |u|, |h|, |K| below rho, the largest
-// mu between 2^-300 and 2^400 or all nine zero), for which the caller runs the double-precision
+// mu between 2^-700 and 2^400 or all nine zero), for which the caller runs the double-precision
 // form.
 //
 // Compiles for the host too.
@@ -92,10 +92,13 @@ PPLBM_FX bool collide_reverse_fixed(const CollideFix& k, const u64 (&psi)[9], do
   u32 mm = mag_hi(b[0]);
 #pragma unroll
   for (int i = 1; i < 9; i += 2) mm = max3(mm, mag_hi(b[i]), mag_hi(b[i + 1]));
-  // below 2^-300 the double-precision form keeps what this frame would drop (subnormals under
-  // 2^-1042, whose upper words are zero, count as zero)
-  ok = ok && mm < (1423u << 20) && mm - 1u >= (723u << 20) - 1u;
-  const int el = ((int)(mm >> 20) > 723 ? (int)(mm >> 20) : 723) + 10;
+  // below 2^-700, and where zs_b, the smallest of the results, would leave the doubles' range,
+  // the double-precision form keeps what this frame would drop (subnormals under 2^-1042, whose
+  // upper words are zero, count as zero). A loss of one node has such adjoints far from it: of 300
+  // steps back on 1024^2 half of them are below 2^-300.
+  ok = ok && mm < (1423u << 20) && mm - 1u >= (323u << 20) - 1u;
+  const int el = ((int)(mm >> 20) > 323 ? (int)(mm >> 20) : 323) + 10;
+  ok = ok && (mm == 0u || el + 2 * eg >= 2236);  // 2^(kl + 2 eg - 2164) >= 2^-1014
   // mu and the sums of them carry two places more (72 2^56 < 2^63); what joins products is
   // rounded to whole units. mu is rounded to nearest, ties to even: half of the ties are
   // exact halves of doubles a few octaves below the largest (rho_b beside a large j_b)
