@@ -56,13 +56,13 @@ MIN_BLOCKS = 5
 # node). The passes run in fixed point: the FP64 pipe only converts results (the moments; six
 # of the nine populations). These are the fallback for sources other than those of COUNTS.
 FP64_PER_NODE = {"rho_psi": 3.2, "collide": 6.8}
-ALU_PER_NODE = {"rho_psi": 251, "collide": 372}
+ALU_PER_NODE = {"rho_psi": 257, "collide": 381}
 # ALU pipe issue rate: 64 thread instructions per SM per clock (ncu's
 # sm__pipe_alu_cycles_active scale: 82.7 % active at 16.6e12 instructions/s)
 ALU_PER_SM_CLK = 64
 # the two-phase relaxation (rows 7, 8 relax with 1/tau(rho)), walls (ncu on the impact lattice)
 FP64_PER_NODE_SHEAR = {"rho_psi": 5.0, "collide": 6.5}
-ALU_PER_NODE_SHEAR = {"rho_psi": 248, "collide": 444}
+ALU_PER_NODE_SHEAR = {"rho_psi": 254, "collide": 459}
 # algorithmic bytes per node of each pass as built (moments handed from pass 1 to
 # pass 2): pass 1 reads 9 f and writes psi + 3 moments (5 with tau(rho)); pass 2
 # reads the moments and the psi tile and writes 9 f
@@ -73,10 +73,10 @@ BYTES_PER_NODE_SHEAR = {"rho_psi": 72 + 48, "collide": 40 + 8 + 72}
 BYTES_PER_NODE_SCOPE = 232
 # FP64-pipe and integer-pipe (ALU) instructions of one MacCormack step per grid point
 # (ncu, sm__inst_executed_pipe_fp64 / _alu x 32 per point, one kernel per capture, the
-# 2048 x 1024 grid of fd_throughput): predictor 6.0 / 826, corrector 12.0 / 826, two EOS
-# passes of 1.0 / 154
+# 2048 x 1024 grid of fd_throughput): predictor 6.0 / 958, corrector 12.0 / 958, two EOS
+# passes of 1.0 / 162
 FD_FP64_PER_POINT = 6.0 + 12.0 + 2 * 1.0
-FD_ALU_PER_POINT = 826 + 826 + 2 * 154
+FD_ALU_PER_POINT = 958 + 958 + 2 * 162
 
 # Per launch of each batched pass on the headline workload (all 64 lattices), from
 # one ncu capture per kernel (--metrics dram__bytes_read.sum, dram__bytes_write.sum,
@@ -85,13 +85,13 @@ FD_ALU_PER_POINT = 826 + 826 + 2 * 154
 # node. They hold for the device code whose digest is recorded with them; once it
 # changes, traffic is null and the source counts above are used until the capture is
 # repeated.
-COUNTS = {"sources": "94e8be60002ff6fc",
-          "rho_psi": {"dram_bytes": 1319949056, "fp64_per_node": 3.156, "alu_per_node": 250.8},
-          "collide": {"dram_bytes": 1335902976, "fp64_per_node": 6.780, "alu_per_node": 372.2},
+COUNTS = {"sources": "30fdca84cf083d11",
+          "rho_psi": {"dram_bytes": 1320013056, "fp64_per_node": 3.156, "alu_per_node": 257.2},
+          "collide": {"dram_bytes": 1336054272, "fp64_per_node": 6.780, "alu_per_node": 381.3},
           # the pipelined plan's mixed kernel: one launch runs the density pass of one
           # group and the collision pass of the other (half the nodes each); a step is
           # two launches
-          "mixed": {"dram_bytes": 1364653056}}
+          "mixed": {"dram_bytes": 1370570496}}
 KERNEL_SOURCES = ("batch_kernels.cuh", "step_device.cuh", "eos_dev.cuh", "eos.cuh", "fp64.cuh", "fixsum.cuh",
                   "fixmul.cuh", "eos_fixed.cuh", "collide_fixed.cuh", "internal.h")
 

@@ -506,13 +506,13 @@ __device__ __noinline__ void adj_collide_general(const AdjArgs& g, int x, int y,
   B[5 * N + node] = gyb;
 }
 
-// A1. What bounds it: integer issue on large lattices (1,090 instructions per node, 590 on
-// the ALU pipe; with the two-phase set and the source 1,780, 890), latency on small ones. With
+// A1. What bounds it: integer issue on large lattices (1,170 instructions per node, 690 on
+// the ALU pipe; with the two-phase set and the source 1,780, 890 before mu was rounded), latency on small ones. With
 // its products on the FP64 pipe (41 to 122 instructions per node) and every stage's sums
-// rounded to doubles in integer code it was bound by both pipes: 1024^2 108 us, now 50 (with
-// the two-phase set and the source 256, now 113). In fixed point with blocks of 256 threads
+// rounded to doubles in integer code it was bound by both pipes: 1024^2 108 us, now 55 (with
+// the two-phase set and the source 256, 113 before mu was rounded). In fixed point with blocks of 256 threads
 // and a block-wide sum it took 68 (141) there, but 35 us against 23 before on 300 x 125.
-// 10 resident blocks (96 registers), 8 for the two-phase set (128), without spills.
+// 10 resident blocks (at most 96 registers), 8 for the two-phase set (128), without spills.
 template <int KIND, bool ST>
 __global__ void __launch_bounds__(kNT, KIND == kShearTau ? 8 : 10) k_adj_collide(const __grid_constant__ AdjArgs g) {
   begin_dependent();
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kNT, KIND == kShearTau ? 8 : 10) k_adj_collide
 // the block-wide sums on the FP64 pipe (121 instructions per warp and node, 12 additions per
 // slot in each block's trees, up to 90 block barriers) that pipe was 81 % busy: 1024^2 248
 // us, now 85 (two-phase with the source 156, now 82). A gradient's step in all, 256^2 60 us
-// -> 28, 1024^2 466 -> 180, 300 x 125 with the source 64 -> 31, 60^2 46 -> 16. 12 resident
+// -> 29, 1024^2 466 -> 188, 300 x 125 with the source 64 -> 31, 60^2 46 -> 16. 12 resident
 // blocks (80 registers); 16 (64 registers) gain 1 % at 1024^2 and lose 10 % at 256^2.
 template <int KIND, bool ST>
 __global__ void __launch_bounds__(kNT, 12) k_adj_rho_psi(const __grid_constant__ AdjArgs g) {

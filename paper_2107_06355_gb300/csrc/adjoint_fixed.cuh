@@ -18,9 +18,9 @@
 // mu; the stored lambda's own rounding is 2^-53. mu itself needs an unbiased rounding: over a
 // long rollout lambda's c . j_b grows beyond rho_b, and mu cut off towards zero at 2^-53 of the
 // largest shrank rho_b: the gradient of 400 steps in the initial density had an rms error of
-// 2.9e-13 of its rms against extended precision (two-phase 2.4e-13), 1.7e-14 (1.2e-14) so, and
+// 2.9e-13 of its rms against extended precision (two-phase 2.4e-13), 1.4e-14 (1.1e-14) so, and
 // 4.3e-14 with rounded double-precision stages; of 100 steps 1.4e-14, 3.0e-15 and 1.0e-14. It costs
-// 3 % of a gradient's step on 1024^2.
+// 4 % of a gradient's step on 1024^2.
 // Reports a node outside the domain (that of the forward, |u|, |h|, |K| below rho, the largest
 // mu between 2^-700 and 2^400 or all nine zero), for which the caller runs the double-precision
 // form.

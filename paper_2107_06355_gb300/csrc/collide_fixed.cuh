@@ -5,13 +5,13 @@
 //
 // What bounds it: the integer ALU pipe and instruction issue (ncu on 2048 x 1024, unit
 // relaxation times: 665 instructions per node, the ALU pipe 70 % and the multiply-add
-// pipe 61 % busy, FP64 27 %). With its products on the FP64 pipe and each sum rounded to a
+// pipe 58 % busy, FP64 27 %). With its products on the FP64 pipe and each sum rounded to a
 // double in integer code the collision took 19 FP64 and about 1,020 integer ALU
 // instructions per node; here nothing is rounded before the populations, so the
 // normalise-and-round steps are gone except the nine of the result, and a product costs
 // three 32 x 32 multiply-adds instead of an FP64 instruction worth 32. Collision pass of
-// a batch of 12.9 M nodes: 0.783 ms before, 0.383 ms now; two-phase 2048 x 1024: 154 and
-// 74 us; a step with six relaxation times, 1300 x 810: 362 and 88 us. Against
+// a batch of 12.9 M nodes: 0.783 ms before, 0.388 ms now; two-phase 2048 x 1024: 154 and
+// 75 us; a step with six relaxation times, 1300 x 810: 362 and 84 us. Against
 // quad precision the populations' rms error is 0.34 ulp (0.41 two-phase), where the rounded
 // stages gave 0.64 (0.67).
 //

@@ -365,11 +365,12 @@ __device__ __noinline__ void fd_update_general(const FDArgs& a, int x, int y) {
 // off to nothing over hundreds of points, and in double precision every one of them would
 // take the time of three).
 //
-// What bounds it: instruction issue and the integer ALU pipe (640 instructions per point, 390
-// of them on that pipe, before the 40 of the common unit). With its products on the FP64 pipe (54 to 60 instructions per
+// What bounds it: instruction issue and the integer ALU pipe (1,470 to 1,500 instructions per
+// point, 960 of them on that pipe). With its products on the FP64 pipe (54 to 60 instructions per
 // point) and every difference rounded to a double in integer code (1,950) both pipes were 80
 // to 90 % busy. Per step (two updates, two density passes): 1200 x 500 264 -> 115 us, 2048 x
-// 1024 804 -> 314, 600 x 250 with tau(rho) 99 -> 55; 102, 310 and 42 with dependent launches.
+// 1024 804 -> 314, 600 x 250 with tau(rho) 99 -> 55; 102, 310 and 40 with dependent launches,
+// 111, 343 and 44 with results that have no mean error.
 using fx::Factor;
 using fx::factor;
 using fx::i64;
